@@ -67,9 +67,10 @@ typedef struct pisp_options {
   int32_t relax_small;  /* supernode amalgamation: merge while pivot block <= this (default 8) */
   double relax_zeros;   /* ... or while explicit zeros <= this fraction (default 0.05) */
   int32_t solve_schedule; /* 0 = persistent: one launch per solve direction whose
-                             CTAs take (front, k, RHS chunk) tasks in level order
-                             and wait (boundedly) for their dependencies;
-                             1 = one launch per level and front-size class */
+                             CTAs take the fronts' tasks in the order of the
+                             assembly forest (forward by height, backward by
+                             depth) and wait (boundedly) for their dependencies;
+                             1 = one launch per height, or depth */
   int32_t factor_policy;  /* fronts wider than 64: 0 (default) = one CTA each while
                              the front fits in shared memory; larger fronts, of
                              any size, in one persistent launch per level where
@@ -91,20 +92,20 @@ typedef struct pisp_options {
                              shared memory, wider fronts as owner tiles;
                              a task waits (boundedly) only for its children's
                              completion counters */
-  int32_t solve_kfuse;    /* persistent solve: shifts per segment task of a front
+  int32_t solve_kfuse;    /* solves by segments (forward, and backward with one
+                             right-hand side): shifts per segment task of a front
                              with at most 32 pivots (0 = 1): larger values pay a
                              front's dependency wait and structure loads once
                              for several shifts, smaller ones run more tasks
                              in parallel */
-  int32_t solve_warp_maxF; /* persistent solve: widest front (with at most 32
-                              pivots) solved by one 32-lane segment, in blocks
-                              of 32 rows (0 = 32); wider fronts are solved by a
-                              whole CTA per (front, k, RHS chunk) */
-  int32_t solve_ctas_per_sm; /* persistent solve: resident CTAs per SM, 2, 3 or 4
-                                (register budgets 128, 80, 64 per thread; 0 = 3
-                                for FP32 factors, 2 for FP64): more CTAs hide
-                                more latency of a batch's many small fronts,
-                                fewer spill less on wide fronts */
+  int32_t solve_warp_maxF; /* solves: widest front (with at most 32 pivots) solved
+                              by one warp (0 = 32, at least 32); wider fronts are
+                              solved by whole CTAs */
+  int32_t solve_ctas_per_sm; /* solves of several right-hand sides: resident CTAs
+                                per SM, 2, 3 or 4 (register budgets 128, 80, 64
+                                per thread; 0 = 2): more CTAs hide more latency of
+                                a large batch's many small fronts, fewer spill
+                                less and crowd the counters less */
   int32_t factor_smem_maxF; /* factor policy 4: widest front factored by one CTA
                                in shared memory (0 = the limit: 160 in FP32,
                                112 in FP64); wider fronts become owner tiles */
@@ -310,11 +311,12 @@ int pisp_graph_launch(pisp_handle* h);
 
 /* The bounded device waits (no counterpart in the paper).  Every dependency
  * wait of the persistent solves polls a completion counter at most `polls`
- * times (about 64 ns apart) and then gives up: it records the failure, the
- * task goes on with whatever data is there, the launch ends normally, and
+ * times (32 ns apart at first, up to 1 us in a long wait) and then gives up: it
+ * records the failure, the task goes on with whatever data is there, the launch
+ * ends normally, and
  * pisp_get_status returns PISP_ERR_TIMEOUT until the next
  * pisp_factor_perturbed clears the record.  polls = 0 restores the default
- * (2^22 polls, a few tenths of a second per wait).  unreachable != 0 is a test
+ * (2^22 polls, a few seconds per wait).  unreachable != 0 is a test
  * hook: the next solves also wait on one completion target raised by one, which
  * no task ever reaches, so that a wait runs out on purpose (results of those
  * solves are not valid); unreachable = 0 restores the true targets.  Applies

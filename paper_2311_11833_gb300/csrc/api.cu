@@ -59,14 +59,20 @@ struct pisp_handle {
   double analyze_ms = 0.0;
   // device symbolic
   Buf c0, ns, ms, inst, front_off, vec_off, row_off, child_off, child, amap_off, amap_src,
-      amap_dst, amap_coff, rows, emap, perm, iperm, row_inst, row_ptr, col, parent, inv_off, inv_child, inv_a, inv_vbase,
-      inv_cF, inv_col, at_ptr, at_row, at_src;
+      amap_dst, amap_coff, rows, emap, perm, iperm, row_inst, row_ptr, col, parent, inv_off, inv_child, inv_a, inv_pos,
+      inv_cF, inv_col, at_ptr, at_row, at_src, pcol, at_prow;
   // persistent solve schedule (depends on K and R)
   int32_t schedule = 0;
   int32_t factor_policy = 0;
   int32_t units_K = 0, units_R = 0;
-  int32_t n_units_f = 0, n_units_b = 0, units_maxF = 0;
-  Buf units_f, units_b, ticket, done, serr, nch, d_wl;
+  int32_t n_units_f = 0, n_units_b = 0;
+  int32_t units_wide = 0;                     // largest chunk of a front with more than 32 pivots
+  size_t ctr_tickets = 0, ctr_half = 0;       // tickets, and all counters, of one direction
+  std::vector<int32_t> lvl_units_f, lvl_units_b;  // first unit of each stage (one launch per stage)
+  // front records in unit-list order; counters, forward then backward: the
+  // tickets, the finished tasks per (front, column group), the solved blocks of
+  // the fronts with more than 32 pivots
+  Buf units_f, units_b, desc, ctr, serr;
   // adaptive FP64 residual sweeps (pisp_set_refinement): stopping tolerance
   // (0 = every sweep for every instance), the instance range [lo, hi] of
   // each persistent solve unit, the compacted unit lists and their lengths,
@@ -93,11 +99,11 @@ struct pisp_handle {
   // level plans (depend on the factor precision)
   int plan_precision = 0;
   std::vector<pisp::LevelPlan> plans;
-  std::vector<int32_t> h_small, h_big, h_all;
+  std::vector<int32_t> h_small, h_big;
   std::vector<pisp::BigFrontHost> h_bigF;
   std::vector<pisp::DagTask> h_dag;
   int32_t dag_max_flags = 0;
-  Buf d_small, d_big, d_all, d_dag, dag_ticket, dag_flags;
+  Buf d_small, d_big, d_dag, dag_ticket, dag_flags;
   // one-launch factorisation (factor policy 4): all-level task list, the
   // warp-front list, completion targets, counters and owner release flags
   int32_t n_ftasks = 0, fac_CH = 32, fac_nflags = 0;
@@ -318,11 +324,9 @@ int build_persistent_factor(pisp_handle* h, int precision, int32_t K) {
 // solve classes.
 int build_plans(pisp_handle* h, int precision) {
   const pisp::Symbolic& S = h->sym;
-  const int scls[6] = {8, 16, 32, 128, 512, INT_MAX};
   h->plans.assign(S.n_levels, pisp::LevelPlan());
   h->h_small.clear();
   h->h_big.clear();
-  h->h_all.clear();
   h->h_bigF.clear();
   h->h_dag.clear();
   h->dag_max_flags = 0;
@@ -411,20 +415,6 @@ int build_plans(pisp_handle* h, int precision) {
       h->h_dag.insert(h->h_dag.end(), tk.begin(), tk.end());
       h->dag_max_flags = std::max(h->dag_max_flags, nfl);
     }
-    lo = 0;
-    for (int c = 0; c < 6; ++c) {
-      pisp::LevelPlan::Group G{(int64_t)h->h_all.size(), 0, 0, 0};
-      for (int32_t s : lst) {
-        const int F = S.sn[s].F();
-        if (F > lo && F <= scls[c]) {
-          h->h_all.push_back(s);
-          ++G.count;
-          G.maxF = std::max(G.maxF, F);
-        }
-      }
-      if (G.count) lp.sgroups[lp.n_sgroups++] = G;
-      lo = scls[c];
-    }
     // algorithmic bytes per perturbation: what each kernel family must read
     // and write at least (values, indices, factor entries, vectors)
     const double p = (double)esize(precision);
@@ -449,7 +439,6 @@ int build_plans(pisp_handle* h, int precision) {
   }
   TRY(upload(h, h->d_small, h->h_small));
   TRY(upload(h, h->d_big, h->h_big));
-  TRY(upload(h, h->d_all, h->h_all));
   TRY(upload(h, h->d_dag, h->h_dag));
   if (!h->dag_ticket.ensure(sizeof(int)) || !h->dag_flags.ensure((size_t)h->dag_max_flags * sizeof(int)))
     return fail(h, PISP_ERR_OOM, "device allocation failed (factor schedule)");
@@ -463,114 +452,179 @@ int build_plans(pisp_handle* h, int precision) {
   return PISP_OK;
 }
 
-// Work units of the persistent solve, per level: fronts with more than 32
-// pivots, or wider than h->warp_maxF, get one unit per (front, k, RHS chunk),
-// solved by a whole CTA; every other front is split into segment tasks of 8,
-// 16 or 32 lanes by its size (32 lanes, in blocks of 32 rows, for fronts
-// wider than 32 with at most 32 pivots), one task per (front, group of
-// h->kfuse consecutive shifts, RHS chunk of 8), 256/SEG tasks per unit.
-// Within a level the CTA units come first, then the segment groups from the
-// widest down; the forward order is levels bottom-up, the backward order
-// top-down.  The fronts of the segment groups are listed in h->h_wl.
-int build_units(pisp_handle* h, int32_t K, int32_t R) {
+// groups of the completion counters (SolveArgs::NG)
+int counter_groups(const pisp_handle* h, int32_t K, int32_t R, bool fwd) {
+  return fwd || R == 1 ? K : (K * pisp::rhs_stride(h->precision, R) + 31) / 32;
+}
+
+// Work units of the solves.  Fronts with more than 32 pivots are CTA tasks per
+// (256 rows, shift, RHS chunk); other fronts wider than h->warp_maxF (at least
+// 32) CTA tasks per (shift, RHS chunk of 8); the rest segment tasks of 8, 16 or
+// 32 lanes by their size, one per group of h->kfuse consecutive shifts and RHS
+// chunk of 8.  Backward solves of several right-hand sides take column groups
+// instead: one CTA task, or one warp's task (8 a unit), per front and group.
+// The forward list goes by the fronts' height above the leaves, the backward
+// list by their depth below the root: each as soon as what it waits for can be
+// done, so that the CTAs in flight hold ready units (by falling height, a
+// root's leaf children would come last, and fronts next to the leaves wait in
+// line behind chains of tall ones: 150 us against 106 us for the backward solve
+// of the 2000-bus grid).  Within a stage the CTA tasks come first, those with
+// the longest way to go before the others, then the warps' tasks from the widest
+// down, by instance, so that the adaptive sweeps' compaction drops whole units.
+// The fronts' records are listed in the order the units name them.
+struct UnitList {
+  std::vector<pisp::SolveUnit> units;
+  std::vector<int32_t> rng;    // [lo, hi] instance range per unit
+  std::vector<int32_t> order;  // front of each record
+  std::vector<int32_t> start;  // first unit of each stage, and the number of units
+};
+
+// tasks[s]: tasks of front s per completion counter
+int build_unit_list(pisp_handle* h, int32_t K, int32_t R, const std::vector<int32_t>& stage,
+                    const std::vector<int32_t>& left, bool fwd, std::vector<int32_t>& tasks, int32_t& wide,
+                    UnitList& out) {
   const pisp::Symbolic& S = h->sym;
-  const int segch = (R + pisp::kSolveChunk - 1) / pisp::kSolveChunk;
-  std::vector<std::vector<pisp::SolveUnit>> per_level(S.n_levels);
-  std::vector<int32_t> nch(S.sn.size(), segch);
-  std::vector<std::vector<int32_t>> per_level_rng(S.n_levels);  // [lo, hi] instance range per unit
-  std::vector<int32_t> wl;
-  int maxF = 0;
-  for (int l = 0; l < S.n_levels; ++l) {
-    auto& U = per_level[l];
-    auto& UR = per_level_rng[l];
-    std::vector<int32_t> lst(S.level_sn.begin() + S.level_off[l], S.level_sn.begin() + S.level_off[l + 1]);
-    std::sort(lst.begin(), lst.end(), [&](int32_t a, int32_t b) {
-      const int fa = S.sn[a].F(), fb = S.sn[b].F();
-      return fa != fb ? fa > fb : a < b;  // widest first
-    });
-    std::vector<int32_t> blk, g32w, g32, g16, g8;
+  const int NG = counter_groups(h, K, R, fwd);
+  const bool cols = !fwd && R > 1;
+  const int kf = std::max(1, std::min(h->kfuse, (int)K));
+  const int rchunks = R == 1 ? 1 : (R + pisp::kSolveChunk - 1) / pisp::kSolveChunk;
+  std::vector<std::vector<int32_t>> at;
+  for (size_t q = 0; q < S.sn.size(); ++q) {
+    if ((size_t)stage[q] >= at.size()) at.resize(stage[q] + 1);
+    at[stage[q]].push_back((int32_t)q);
+  }
+  out.order.reserve(S.sn.size());
+  auto cta_unit = [&](int32_t sn, const pisp::SolveUnit& u) {
+    out.units.push_back(u);
+    out.rng.push_back(S.sn[sn].instance);
+    out.rng.push_back(S.sn[sn].instance);
+  };
+  for (auto& lst : at) {
+    out.start.push_back((int32_t)out.units.size());
+    std::vector<int32_t> cta, seg[4];  // segments of 8, 16, 32 lanes; warps
+    auto wide_rows = [&](int32_t sn) {  // tasks of 256 rows
+      return ((fwd ? S.sn[sn].F() : S.sn[sn].ns()) + pisp::kWideUnitRows - 1) / pisp::kWideUnitRows;
+    };
     for (int32_t sn : lst) {
       const int F = S.sn[sn].F(), ns = S.sn[sn].ns();
-      if (ns > 32 || F > std::max(32, h->warp_maxF)) blk.push_back(sn);
-      else if (F > 32) g32w.push_back(sn);
-      else if (F > 16) g32.push_back(sn);
-      else if (F > 8) g16.push_back(sn);
-      else g8.push_back(sn);
+      if (ns > 32 || F > std::max(32, h->warp_maxF)) cta.push_back(sn);
+      else seg[cols ? 3 : (F > 16 ? 2 : (F > 8 ? 1 : 0))].push_back(sn);
+      tasks[sn] = cols ? 1 : rchunks;
     }
-    const int rc = pisp::pick_chunk(std::max<int>(1, (int)blk.size()), K, R);
-    const int bch = (R + rc - 1) / rc;
-    for (int32_t sn : blk) {
-      maxF = std::max(maxF, S.sn[sn].F());
-      nch[sn] = bch;
-      for (int k = 0; k < K; ++k)
-        for (int c = 0; c < bch; ++c) {
-          U.push_back({pisp::kUnitBlk, sn, k, c, rc});
-          UR.push_back(S.sn[sn].instance);
-          UR.push_back(S.sn[sn].instance);
-        }
-    }
-    auto seg_group = [&](const std::vector<int32_t>& g, int seg) -> int {
-      if (g.empty()) return PISP_OK;
-      const int kind = seg == 8 ? pisp::kUnitSeg8 : (seg == 16 ? pisp::kUnitSeg16 : pisp::kUnitSeg32);
-      const int64_t off = (int64_t)wl.size();
-      const int kf = std::max(1, std::min(h->kfuse, (int)K));
-      const int64_t tasks = (int64_t)g.size() * ((K + kf - 1) / kf) * segch;
-      if (tasks >= INT32_MAX || off >= INT32_MAX) return fail(h, PISP_ERR_UNSUPPORTED, "too many solve tasks");
-      wl.insert(wl.end(), g.begin(), g.end());
-      const int64_t per_front = (int64_t)((K + kf - 1) / kf) * segch;
-      for (int64_t b = 0; b < tasks; b += 256 / seg) {
-        U.push_back({kind, (int32_t)off, (int32_t)b, (int32_t)tasks, kf});
-        int32_t lo = INT32_MAX, hi = -1;
-        for (int64_t q = b; q < std::min(tasks, b + 256 / seg); q += 1) {
-          const int32_t in = S.sn[g[q / per_front]].instance;
-          lo = std::min(lo, in);
-          hi = std::max(hi, in);
-        }
-        UR.push_back(lo);
-        UR.push_back(hi);
+    std::sort(cta.begin(), cta.end(), [&](int32_t a, int32_t b) {
+      if (left[a] != left[b]) return left[a] > left[b];
+      const int fa = S.sn[a].F(), fb = S.sn[b].F();
+      return fa != fb ? fa > fb : a < b;
+    });
+    const int rc = pisp::wide_chunk(h->precision, R);
+    for (int32_t sn : cta) {
+      const int32_t slot = (int32_t)out.order.size();
+      out.order.push_back(sn);
+      if (S.sn[sn].ns() <= 32) {
+        for (int g = 0; g < NG; ++g)
+          for (int c = 0; c < tasks[sn]; ++c) cta_unit(sn, {pisp::kUnitCta, slot, g, c});
+        continue;
       }
-      return PISP_OK;
-    };
-    TRY(seg_group(g32w, 32));
-    TRY(seg_group(g32, 32));
-    TRY(seg_group(g16, 16));
-    TRY(seg_group(g8, 8));
+      const int ch = (R + rc - 1) / rc, nq = wide_rows(sn);
+      wide = std::max(wide, rc);
+      tasks[sn] = cols ? nq * K * ch : nq * ch;
+      // the rows solved first, first: a task waits only for tasks before it
+      for (int q = 0; q < nq; ++q)
+        for (int k = 0; k < K; ++k)
+          for (int c = 0; c < ch; ++c)
+            cta_unit(sn, {pisp::kUnitWide | rc << 4, slot, k | (fwd ? q : nq - 1 - q) << 8, c});
+    }
+    for (int w = 3; w >= 0; --w) {
+      std::vector<int32_t>& g = seg[w];
+      if (g.empty()) continue;
+      const int kind = w == 3 ? pisp::kUnitCol : (w == 2 ? pisp::kUnitSeg32 : (w == 1 ? pisp::kUnitSeg16 : pisp::kUnitSeg8));
+      const int per_unit = w == 3 ? 8 : 256 / (8 << w);
+      const int64_t per_front = w == 3 ? NG : (int64_t)((K + kf - 1) / kf) * rchunks;
+      std::sort(g.begin(), g.end(), [&](int32_t a, int32_t b) {
+        if (S.sn[a].instance != S.sn[b].instance) return S.sn[a].instance < S.sn[b].instance;
+        const int fa = S.sn[a].F(), fb = S.sn[b].F();
+        return fa != fb ? fa > fb : a < b;
+      });
+      const int32_t off = (int32_t)out.order.size();
+      const int64_t n = (int64_t)g.size() * per_front;
+      if (n >= INT32_MAX) return fail(h, PISP_ERR_UNSUPPORTED, "too many solve tasks");
+      out.order.insert(out.order.end(), g.begin(), g.end());
+      for (int64_t b = 0; b < n; b += per_unit) {
+        out.units.push_back({kind | (w == 3 ? 0 : kf << 4), off, (int32_t)b, (int32_t)n});
+        out.rng.push_back(S.sn[g[b / per_front]].instance);
+        out.rng.push_back(S.sn[g[(std::min(n, b + per_unit) - 1) / per_front]].instance);
+      }
+    }
   }
+  if (out.units.size() >= (size_t)INT32_MAX) return fail(h, PISP_ERR_UNSUPPORTED, "too many solve tasks");
+  out.start.push_back((int32_t)out.units.size());
+  return PISP_OK;
+}
+
+int build_units(pisp_handle* h, int32_t K, int32_t R) {
+  const pisp::Symbolic& S = h->sym;
+  const size_t nS = S.sn.size();
+  // parents have larger numbers than their children
+  std::vector<int32_t> height(nS), depth(nS, 0);
+  for (size_t q = 0; q < nS; ++q) height[q] = S.sn[q].level;
+  for (size_t q = nS; q-- > 0;)
+    if (S.sn[q].parent >= 0) depth[q] = depth[S.sn[q].parent] + 1;
+  UnitList f, b;
+  std::vector<int32_t> nf(nS, 1), nb(nS, 1);
+  int32_t wide = 0;
+  TRY(build_unit_list(h, K, R, height, depth, true, nf, wide, f));
+  TRY(build_unit_list(h, K, R, depth, height, false, nb, wide, b));
+  // completion targets: forward, every task of a front's children; backward,
+  // every task of its parent, as the counters count them
+  const int NG = std::max(counter_groups(h, K, R, true), counter_groups(h, K, R, false));
+  auto whole = [&](int32_t q) { return R > 1 && S.sn[q].ns() > 32; };  // backward
+  std::vector<int32_t> need(nS, 0);
+  for (size_t q = 0; q < nS; ++q)
+    if (S.sn[q].parent >= 0) need[S.sn[q].parent] += nf[q];
   if (h->wait_unreachable) {
     // test hook: one front's completion target can never be reached, so the
     // waits on it (its parent's in the forward pass, its children's in the
     // backward pass) run out of polls
-    for (size_t q = 0; q < S.sn.size(); ++q)
+    for (size_t q = 0; q < nS; ++q)
       if (S.sn[q].parent >= 0) {
-        nch[q] += 1;
+        need[S.sn[q].parent] += 1;
+        nb[q] += 1;
         break;
       }
   }
-  std::vector<pisp::SolveUnit> f, b;
-  std::vector<int32_t> rf, rb;
-  for (int l = 0; l < S.n_levels; ++l) {
-    f.insert(f.end(), per_level[l].begin(), per_level[l].end());
-    rf.insert(rf.end(), per_level_rng[l].begin(), per_level_rng[l].end());
+  // counters of the fronts with more than 32 pivots (at most one per right-hand side)
+  std::vector<int32_t> flag(nS, 0);
+  int64_t nflags = 0;
+  for (size_t q = 0; q < nS; ++q)
+    if (S.sn[q].ns() > 32) {
+      flag[q] = (int32_t)nflags;
+      nflags += (int64_t)K * R;
+      if (nflags >= INT32_MAX) return fail(h, PISP_ERR_UNSUPPORTED, "too many solve tasks");
+    }
+  std::vector<pisp::FrontDesc> desc(2 * nS);  // forward order, then backward order
+  for (size_t q = 0; q < 2 * nS; ++q) {
+    const int32_t sn = q < nS ? f.order[q] : b.order[q - nS];
+    const pisp::Supernode& n = S.sn[sn];
+    desc[q] = {n.c0, n.ns(), n.F(), n.instance, S.front_off[sn], S.vec_off[sn], n.row_off, n.parent, sn, need[sn],
+               n.parent >= 0 ? nb[n.parent] : 0, flag[sn],
+               (whole(sn) ? pisp::kSelfWhole : 0) | (n.parent >= 0 && whole(n.parent) ? pisp::kParentWhole : 0)};
   }
-  for (int l = S.n_levels - 1; l >= 0; --l) {
-    b.insert(b.end(), per_level[l].begin(), per_level[l].end());
-    rb.insert(rb.end(), per_level_rng[l].begin(), per_level_rng[l].end());
-  }
-  TRY(upload(h, h->units_f, f));
-  TRY(upload(h, h->units_b, b));
-  TRY(upload(h, h->rng_f, rf));
-  TRY(upload(h, h->rng_b, rb));
-  if (!h->units_fc.ensure(f.size() * sizeof(pisp::SolveUnit)) ||
-      !h->units_bc.ensure(b.size() * sizeof(pisp::SolveUnit)) || !h->ucount.ensure(2 * sizeof(int32_t)))
+  TRY(upload(h, h->units_f, f.units));
+  TRY(upload(h, h->units_b, b.units));
+  TRY(upload(h, h->rng_f, f.rng));
+  TRY(upload(h, h->rng_b, b.rng));
+  TRY(upload(h, h->desc, desc));
+  if (!h->units_fc.ensure(f.units.size() * sizeof(pisp::SolveUnit)) ||
+      !h->units_bc.ensure(b.units.size() * sizeof(pisp::SolveUnit)) || !h->ucount.ensure(2 * sizeof(int32_t)) ||
+      !h->serr.ensure(sizeof(int)) || !h->ctr.ensure(2 * (f.start.size() + b.start.size() + 8 + (nS * (size_t)NG + (size_t)nflags) * pisp::kCtrStride) * sizeof(int)))
     return fail(h, PISP_ERR_OOM, "device allocation failed (solve schedule)");
-  TRY(upload(h, h->nch, nch));
-  TRY(upload(h, h->d_wl, wl));
-  if (!h->ticket.ensure(2 * sizeof(int)) || !h->serr.ensure(sizeof(int)) ||
-      !h->done.ensure((size_t)S.sn.size() * K * sizeof(int)))
-    return fail(h, PISP_ERR_OOM, "device allocation failed (solve schedule)");
-  h->n_units_f = (int32_t)f.size();
-  h->n_units_b = (int32_t)b.size();
-  h->units_maxF = maxF;
+  h->n_units_f = (int32_t)f.units.size();
+  h->n_units_b = (int32_t)b.units.size();
+  h->lvl_units_f = f.start;
+  h->lvl_units_b = b.start;
+  h->units_wide = wide;
+  h->ctr_tickets = (f.start.size() + b.start.size()) / 8 * 8 + 8;  // more than one per stage
+  h->ctr_half = h->ctr_tickets + (nS * (size_t)NG + (size_t)nflags) * pisp::kCtrStride;
   h->units_K = K;
   h->units_R = R;
   return PISP_OK;
@@ -644,65 +698,102 @@ int count(pisp_handle* h, int n) {
   return PISP_OK;
 }
 
-// forward + backward over all levels; `rhs` broadcast [N][R] (original order)
-// or per-perturbation [N][K][R] (permuted order); results to `out`
-// (and added to `acc` when given).  Adaptive sweeps (persistent schedule):
-// act skips the fronts of instances that have stopped and the compacted unit
-// lists are walked.
-int solve_pass(pisp_handle* h, bool trans, const double* rhs, int rhs_mode, double* out,
-               double* acc, int32_t R, const uint8_t* act = nullptr) {
+// Right-hand sides and outputs of one forward + backward solve: b (FP64,
+// broadcast, original order) or rk (factor precision, per shift, permuted
+// order); xt the solution in the factor precision, xd (may be null) in FP64,
+// stored or added (solve_persistent.h).
+struct SolveIO {
+  const double* b;
+  const void* rk;
+  void* xt;
+  double* xd;
+  int xd_mode;
+};
+
+template <typename T>
+int solve_pass_t(pisp_handle* h, bool trans, const SolveIO& io, int32_t R, const uint8_t* act) {
   const int L = h->sym.n_levels;
-  if (!trans && h->schedule == 0) {
-    if (h->units_K != h->K || h->units_R != R) TRY(build_units(h, h->K, R));
-    const size_t nd = (size_t)h->sym.sn.size() * h->K * sizeof(int);
-    double bf = 0, bb = 0;
-    for (int l = 0; l < L; ++l) {
-      bf += h->K * (h->plans[l].bytes_fwd_a + h->plans[l].bytes_fwd_b * R);
-      bb += h->K * (h->plans[l].bytes_bwd_a + h->plans[l].bytes_bwd_b * R);
-    }
-    if (acc) bb += 16.0 * h->sym.N * h->K * R;
-    CK(cudaMemsetAsync(h->ticket.p, 0, 2 * sizeof(int), h->stream));
-    CK(cudaMemsetAsync(h->done.p, 0, nd, h->stream));
-    const bool cmp = act != nullptr;  // gated: the compacted lists (whole lists before the first test)
-    const int* ucf = cmp ? h->ucount.as<int>() : nullptr;
-    const int* ucb = cmp ? h->ucount.as<int>() + 1 : nullptr;
-    int pb = prof_begin(h);
-    int n = pisp::launch_solve_persistent(
-        h->precision, true, h->sd, (cmp ? h->units_fc : h->units_f).as<pisp::SolveUnit>(), h->n_units_f, ucf, act,
-        h->ticket.as<int>(), h->done.as<int>(), h->serr.as<int>(), h->nch.as<int>(), h->d_wl.as<int32_t>(),
-        h->fronts.p, rhs, rhs_mode, h->V.p, out, acc, R, h->K, h->units_maxF, h->solve_ctas, h->wait_polls,
-        h->stream);
-    TRY(count(h, n));
-    prof_end(h, pb, PISP_PROF_FORWARD, bf, n);
-    CK(cudaMemsetAsync(h->done.p, 0, nd, h->stream));
-    pb = prof_begin(h);
-    n = pisp::launch_solve_persistent(
-        h->precision, false, h->sd, (cmp ? h->units_bc : h->units_b).as<pisp::SolveUnit>(), h->n_units_b, ucb, act,
-        h->ticket.as<int>() + 1, h->done.as<int>(), h->serr.as<int>(), h->nch.as<int>(), h->d_wl.as<int32_t>(),
-        h->fronts.p, rhs, rhs_mode, h->V.p, out, acc, R, h->K, h->units_maxF, h->solve_ctas, h->wait_polls,
-        h->stream);
-    TRY(count(h, n));
-    prof_end(h, pb, PISP_PROF_BACKWARD, bb, n);
-    return PISP_OK;
-  }
+  double bf = 0, bb = 0;
   for (int l = 0; l < L; ++l) {
-    const pisp::LevelPlan& lp = h->plans[l];
-    const int pb = prof_begin(h);
-    const int n = pisp::launch_forward_level(h->precision, trans, h->sd, lp, h->d_all.as<int32_t>(),
-                                             h->fronts.p, rhs, rhs_mode, h->V.p, R, h->K, h->stream);
-    TRY(count(h, n));
-    prof_end(h, pb, PISP_PROF_FORWARD, h->K * (lp.bytes_fwd_a + lp.bytes_fwd_b * R), n);
+    bf += h->K * (h->plans[l].bytes_fwd_a + h->plans[l].bytes_fwd_b * R);
+    bb += h->K * (h->plans[l].bytes_bwd_a + h->plans[l].bytes_bwd_b * R);
   }
-  for (int l = L - 1; l >= 0; --l) {
-    const pisp::LevelPlan& lp = h->plans[l];
+  if (io.xd && io.xd_mode == pisp::kXdAdd) bb += 16.0 * h->sym.N * h->K * R;
+  const bool cmp = act != nullptr;  // gated: the compacted lists (whole lists before the first test)
+  const bool persistent = h->schedule == 0;
+  int* ctr = h->ctr.as<int>();
+  const size_t nd = h->ctr_half;
+  pisp::SolveArgs<T> a{};
+  a.inv_off = h->sd.inv_off;
+  a.inv_pos = h->sd.inv_pos;
+  a.rows = h->sd.rows;
+  a.perm = h->sd.perm;
+  a.act = act;
+  a.err = h->serr.as<int>();
+  a.polls = h->wait_polls > 0 ? h->wait_polls : (int64_t)1 << 22;
+  a.fronts = h->fronts.as<T>();
+  a.b = io.b;
+  a.rk = (const T*)io.rk;
+  a.V = h->V.as<T>();
+  a.xt = (T*)io.xt;
+  a.xd = io.xd;
+  a.xd_mode = io.xd_mode;
+  a.R = R;
+  a.K = h->K;
+  a.RV = pisp::rhs_stride(h->precision, R);
+  a.RX = pisp::rhs_stride64(R);
+  a.vec = a.RV % (16 / (int)sizeof(T)) == 0;
+  a.vecd = a.RX % 2 == 0;
+  CK(cudaMemsetAsync(ctr, 0, 2 * nd * sizeof(int), h->stream));
+  for (int dir = 0; dir < 2; ++dir) {  // forward, backward
+    a.desc = h->desc.as<pisp::FrontDesc>() + (dir == 0 ? 0 : h->sym.sn.size());
     const int pb = prof_begin(h);
-    const int n = pisp::launch_backward_level(h->precision, trans, h->sd, lp, h->d_all.as<int32_t>(),
-                                              h->fronts.p, h->V.p, out, acc, R, h->K, h->stream);
+    int n = 0;
+    auto go = [&](int count) {
+      return dir == 0 ? pisp::launch_solve_dir<T, true>(trans, a, count, h->units_wide, h->solve_ctas, h->stream)
+                      : pisp::launch_solve_dir<T, false>(trans, a, count, h->units_wide, h->solve_ctas, h->stream);
+    };
+    const int total = dir == 0 ? h->n_units_f : h->n_units_b;
+    a.NG = counter_groups(h, h->K, R, dir == 0);
+    a.ticket = ctr + (dir == 0 ? 0 : nd);
+    a.wide = a.ticket + h->ctr_tickets + h->sym.sn.size() * (size_t)a.NG * pisp::kCtrStride;
+    if (persistent) {
+      a.units = (dir == 0 ? (cmp ? h->units_fc : h->units_f) : (cmp ? h->units_bc : h->units_b)).as<pisp::SolveUnit>();
+      a.ucount = cmp ? h->ucount.as<int>() + dir : nullptr;
+      a.nunits = total;
+      a.done = a.ticket + h->ctr_tickets;
+      n = go(total);
+    } else {
+      a.units = (dir == 0 ? h->units_f : h->units_b).as<pisp::SolveUnit>();
+      const auto& lv = dir == 0 ? h->lvl_units_f : h->lvl_units_b;
+      for (size_t l = 0; l + 1 < lv.size() && n >= 0; ++l) {
+        a.first = lv[l];
+        a.nunits = lv[l + 1] - lv[l];
+        const int m = go(a.nunits);
+        n = m < 0 ? -1 : n + m;
+        ++a.ticket;
+      }
+    }
     TRY(count(h, n));
-    prof_end(h, pb, PISP_PROF_BACKWARD,
-             h->K * (lp.bytes_bwd_a + lp.bytes_bwd_b * R) + (acc ? 16.0 * h->sym.N * h->K * R / L : 0.0), n);
+    prof_end(h, pb, dir == 0 ? PISP_PROF_FORWARD : PISP_PROF_BACKWARD, dir == 0 ? bf : bb, n);
   }
   return PISP_OK;
+}
+
+// forward + backward over all levels with L U, or with trans with U^T L^T.
+// Adaptive sweeps (persistent schedule): act skips the fronts of instances
+// that have stopped and the compacted unit lists are walked.
+int solve_pass(pisp_handle* h, bool trans, const SolveIO& io, int32_t R, const uint8_t* act = nullptr) {
+  if (h->units_K != h->K || h->units_R != R) TRY(build_units(h, h->K, R));
+  return h->precision == PISP_FP32 ? solve_pass_t<float>(h, trans, io, R, act)
+                                   : solve_pass_t<double>(h, trans, io, R, act);
+}
+
+// The uncorrected solve of b into X (FP64): with FP64 factors X is itself the
+// working solution, with FP32 factors that is Y.
+SolveIO first_solve(pisp_handle* h, const double* b, double* X) {
+  if (h->precision == PISP_FP64) return {b, nullptr, X, nullptr, pisp::kXdStore};
+  return {b, nullptr, h->Y.p, X, pisp::kXdStore};
 }
 
 // Sweeps per instance of the last solve, and for s = 1 .. max_sweeps the
@@ -760,17 +851,17 @@ int sweep_body(pisp_handle* h, const double* rhs, double* X_out, int32_t R, int3
   uint8_t* act = h->r_act.as<uint8_t>();
   const pisp::ActiveSet as{act, h->r_nact.as<int32_t>(), h->r_ai.as<int32_t>(), h->r_arow.as<int64_t>(),
                            h->d_inst_off.as<int64_t>()};
-  TRY(count(h, pisp::launch_residual_per_k(h->sd, h->vals.as<double>(), h->D.as<double>(), sh, rhs, X_out, R,
-                                           h->Rk.as<double>(), as,
+  TRY(count(h, pisp::launch_residual_per_k(h->precision, h->sd, h->vals.as<double>(), h->D.as<double>(), sh, rhs,
+                                           X_out, R, h->Rk.p, as,
                                            persistent ? pisp::kResActive : pisp::kResZeroStopped, h->stream)));
   // the corrections go to Y only: the stats launch below adds them to X
   const bool prof_was = h->prof_on;
   h->prof_on = false;
-  const int rc = solve_pass(h, false, h->Rk.as<double>(), pisp::RHS_PER_K, h->Y.as<double>(), nullptr, R,
+  const int rc = solve_pass(h, false, {nullptr, h->Rk.p, h->Y.p, nullptr, pisp::kXdStore}, R,
                             persistent ? act : nullptr);
   h->prof_on = prof_was;
   TRY(rc);
-  TRY(count(h, pisp::launch_refine_stats(h->sd, as, X_out, h->Y.as<double>(), h->K, R,
+  TRY(count(h, pisp::launch_refine_stats(h->precision, h->sd, as, X_out, h->Y.p, h->K, R,
                                          h->r_dmax.as<unsigned long long>(), h->r_xmax.as<unsigned long long>(),
                                          h->stream)));
   TRY(count(h, pisp::launch_refine_decide(G, R, h->sweep_tol, S, h->r_sweep.as<int32_t>(), cond, 1, act,
@@ -856,7 +947,7 @@ int run_sweep_loop(pisp_handle* h, const double* rhs, double* X_out, int32_t R, 
 // stopping test holds, as a device-side loop.
 int solve_core(pisp_handle* h, const double* rhs, double* X_out, int32_t R, int32_t sweeps,
                const pisp::Shifts& sh) {
-  TRY(solve_pass(h, false, rhs, pisp::RHS_BROADCAST, X_out, nullptr, R));
+  TRY(solve_pass(h, false, first_solve(h, rhs, X_out), R));
   const double N = (double)h->sym.N, KR = (double)h->K * R;
   const bool adapt = h->sweep_tol > 0.0 && sweeps > 0;
   const int32_t G = h->sym.G;
@@ -868,11 +959,11 @@ int solve_core(pisp_handle* h, const double* rhs, double* X_out, int32_t R, int3
     const pisp::ActiveSet none{};
     for (int it = 0; it < sweeps; ++it) {
       const int pb = prof_begin(h);
-      const int n = pisp::launch_residual_per_k(h->sd, h->vals.as<double>(), h->D.as<double>(), sh, rhs, X_out, R,
-                                                h->Rk.as<double>(), none, pisp::kResAll, h->stream);
+      const int n = pisp::launch_residual_per_k(h->precision, h->sd, h->vals.as<double>(), h->D.as<double>(), sh, rhs,
+                                                X_out, R, h->Rk.p, none, pisp::kResAll, h->stream);
       TRY(count(h, n));
       prof_end(h, pb, PISP_PROF_RESIDUAL, h->sym.nnzA * 12.0 + N * 20.0 + N * R * 8.0 + 2.0 * N * KR * 8.0, n);
-      TRY(solve_pass(h, false, h->Rk.as<double>(), pisp::RHS_PER_K, h->Y.as<double>(), X_out, R));
+      TRY(solve_pass(h, false, {nullptr, h->Rk.p, h->Y.p, X_out, pisp::kXdAdd}, R));
     }
     return PISP_OK;
   }
@@ -908,9 +999,10 @@ int solve_core(pisp_handle* h, const double* rhs, double* X_out, int32_t R, int3
 }
 
 int ensure_solve_buffers(pisp_handle* h, int32_t R) {
-  const size_t nkr = (size_t)h->sym.N * h->K * R * sizeof(double);
-  const size_t v = (size_t)h->K * R * h->sym.vec_off.back() * esize(h->precision);
-  if (!h->V.ensure(v) || !h->X.ensure(nkr) || !h->Y.ensure(nkr) || !h->Rk.ensure(nkr))
+  const size_t kv = (size_t)h->K * pisp::rhs_stride(h->precision, R) * esize(h->precision);
+  const size_t nk = (size_t)h->sym.N * h->K * pisp::rhs_stride64(R) * sizeof(double);
+  if (!h->V.ensure(kv * h->sym.vec_off.back()) || !h->X.ensure(nk) || !h->Y.ensure(kv * h->sym.N) ||
+      !h->Rk.ensure(kv * h->sym.N))
     return fail(h, PISP_ERR_OOM, "device allocation failed (solve workspace)");
   return PISP_OK;
 }
@@ -1061,7 +1153,14 @@ int analyze_impl(pisp_handle* h, int32_t G, const int32_t* n, const int64_t* row
   TRY(upload(h, h->inv_off, S.inv_off));
   TRY(upload(h, h->inv_child, S.inv_child));
   TRY(upload(h, h->inv_a, S.inv_a));
-  TRY(upload(h, h->inv_vbase, S.inv_vbase));
+  {
+    std::vector<int64_t> pos(S.inv_col.size());
+    for (size_t q = 0; q < pos.size(); ++q) pos[q] = S.vec_off[S.inv_child[q]] + S.inv_col[q];
+    TRY(upload(h, h->inv_pos, pos));
+    std::vector<int32_t> pc(cl.size());
+    for (size_t e = 0; e < pc.size(); ++e) pc[e] = S.iperm[cl[e]];
+    TRY(upload(h, h->pcol, pc));
+  }
   TRY(upload(h, h->inv_cF, S.inv_cF));
   TRY(upload(h, h->inv_col, S.inv_col));
   {
@@ -1081,6 +1180,8 @@ int analyze_impl(pisp_handle* h, int32_t G, const int32_t* n, const int64_t* row
     TRY(upload(h, h->at_ptr, atp));
     TRY(upload(h, h->at_row, atr));
     TRY(upload(h, h->at_src, ats));
+    for (int32_t& i : atr) i = S.iperm[i];
+    TRY(upload(h, h->at_prow, atr));
   }
   pisp::SymDev& sd = h->sd;
   sd.c0 = h->c0.as<int32_t>();
@@ -1107,7 +1208,9 @@ int analyze_impl(pisp_handle* h, int32_t G, const int32_t* n, const int64_t* row
   sd.inv_off = h->inv_off.as<int64_t>();
   sd.inv_child = h->inv_child.as<int32_t>();
   sd.inv_a = h->inv_a.as<int32_t>();
-  sd.inv_vbase = h->inv_vbase.as<int64_t>();
+  sd.inv_pos = h->inv_pos.as<int64_t>();
+  sd.pcol = h->pcol.as<int32_t>();
+  sd.at_prow = h->at_prow.as<int32_t>();
   sd.inv_cF = h->inv_cF.as<int32_t>();
   sd.inv_col = h->inv_col.as<int32_t>();
   sd.at_ptr = h->at_ptr.as<int64_t>();
@@ -1346,7 +1449,7 @@ int pisp_refine(pisp_handle* h, const double* b, double* x, int32_t R, int32_t i
   // pisp_adjoint refuse until the next pisp_solve
   if (h->solved && R > h->R) h->solved = false;
   TRY(ensure_solve_buffers(h, R));
-  const size_t nkr = (size_t)h->sym.N * h->K * R * sizeof(double);
+  const size_t nkr = (size_t)h->sym.N * h->K * pisp::rhs_stride64(R) * sizeof(double);
   const size_t nr = (size_t)h->sym.N * R * sizeof(double);
   if (!h->X2.ensure(nkr) || !h->rtmp.ensure(nr) || !h->dtmp.ensure(nr))
     return fail(h, PISP_ERR_OOM, "device allocation failed (refine workspace)");
@@ -1373,17 +1476,17 @@ int pisp_adjoint(pisp_handle* h, const double* g, const double* w, double* grad_
   double ww[PISP_K_MAX];
   TRY(set_weights(h, w, ww));
   const int32_t R = h->R;
-  if (!h->Lam.ensure((size_t)h->sym.N * h->K * R * sizeof(double)))
+  if (!h->Lam.ensure((size_t)h->sym.N * h->K * pisp::rhs_stride64(R) * sizeof(double)))
     return fail(h, PISP_ERR_OOM, "device allocation failed (adjoint workspace)");
   const pisp::Shifts sh = make_shifts(h, ww);
-  TRY(solve_pass(h, true, g, pisp::RHS_BROADCAST, h->Lam.as<double>(), nullptr, R));
+  TRY(solve_pass(h, true, first_solve(h, g, h->Lam.as<double>()), R));
   // FP64 residual sweeps of every lambda_k on the transposed systems, as the
   // forward sweeps do for x_k: with FP32 factors the adjoint then reaches the
   // FP64 definition too (Rk and Y are the solve's workspace, sized for R)
   for (int it = 0; it < sweeps; ++it) {
-    TRY(count(h, pisp::launch_residual_T_per_k(h->sd, h->vals.as<double>(), h->D.as<double>(), sh, g,
-                                               h->Lam.as<double>(), R, h->Rk.as<double>(), h->stream)));
-    TRY(solve_pass(h, true, h->Rk.as<double>(), pisp::RHS_PER_K, h->Y.as<double>(), h->Lam.as<double>(), R));
+    TRY(count(h, pisp::launch_residual_T_per_k(h->precision, h->sd, h->vals.as<double>(), h->D.as<double>(), sh, g,
+                                               h->Lam.as<double>(), R, h->Rk.p, h->stream)));
+    TRY(solve_pass(h, true, {nullptr, h->Rk.p, h->Y.p, h->Lam.as<double>(), pisp::kXdAdd}, R));
   }
   if (grad_b) TRY(count(h, pisp::launch_combine(h->sd, h->Lam.as<double>(), sh, R, grad_b, h->stream)));
   if (grad_values)

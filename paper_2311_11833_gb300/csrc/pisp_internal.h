@@ -40,7 +40,6 @@ struct SymDev {
   const int64_t* inv_off;    // [sum F + 1] contributions to position vec_off[s] + j
   const int32_t* inv_child;  //   contributing child
   const int32_t* inv_a;      //   its update-row index
-  const int64_t* inv_vbase;  //   the child's vec_off
   const int32_t* inv_cF;     //   the child's front size
   const int32_t* inv_col;    //   position in the child's front
   const int32_t* perm;       // [N] perm[new] = old
@@ -51,6 +50,9 @@ struct SymDev {
   const int64_t* at_ptr;     // [N+1] CSC of A: entries of column j at at_ptr[j]..at_ptr[j+1]
   const int32_t* at_row;     //   their rows
   const int32_t* at_src;     //   their CSR entry indices
+  const int64_t* inv_pos;    // inverse extend-add map as positions: vec_off[child] + inv_col
+  const int32_t* pcol;       // [nnz] permuted column of every CSR entry
+  const int32_t* at_prow;    // [nnz] permuted row of every CSC entry
   int64_t N;
   int32_t S;
 };
@@ -85,9 +87,6 @@ struct LevelPlan {
   int32_t dag_flags = 0;
   int32_t dag_owner = 0;      // 1: the tasks are owner tiles
   int32_t own_ch = 0;         //    rows per owner tile (a multiple of 32)
-  // every front of the level for the solves, grouped by size class
-  Group sgroups[8];
-  int32_t n_sgroups = 0;
   // algorithmic bytes per perturbation (a + b * R) of each kernel family,
   // used for the achieved-bandwidth figures of the profiling interface
   double bytes_fsmall = 0, bytes_fbig = 0;
@@ -190,42 +189,87 @@ int max_big_front(int precision);
 // largest front the solve kernels can take
 int max_solve_front(int precision);
 
-// ---- solve (solve.cu) ----
-enum RhsMode { RHS_BROADCAST = 0, RHS_PER_K = 1 };
-
-// Work unit of the persistent solve schedule.  Segment units cover 256/SEG
-// consecutive segment tasks of one group (a task = one front, a group of d
-// consecutive shifts, one RHS chunk of 8): a = offset of the group in the
-// schedule's front list, b = first task, c = tasks in the group, d = shifts
-// per task.  Block units are one (front a, perturbation b, RHS chunk c of d
-// right-hand sides), solved by a whole CTA.
-enum UnitKind { kUnitSeg8 = 0, kUnitSeg16 = 1, kUnitSeg32 = 2, kUnitBlk = 3 };
+// ---- solve (solve_persistent.h; solve.cu) ----
+// Work unit of the solves: 16 bytes, read at once.  x = kind | d << 4.
+//   kUnitSeg8/16/32 (forward, and backward with one right-hand side): 256 / SEG
+//     consecutive segment tasks of one group (a task = one front, a group of d
+//     consecutive shifts, one chunk of 8 right-hand sides or the only one): a =
+//     the group's first front record, b = first task, c = tasks in the group;
+//   kUnitCol (backward, several right-hand sides): 8 consecutive warp tasks of
+//     one group (a task = one front, one group of 32 columns (k, r)), a, b, c as
+//     above;
+//   kUnitCta: one front (record a) with at most 32 pivots, for the shift b and
+//     RHS chunk c, or for the column group b;
+//   kUnitWide: a front (record a) with more than 32 pivots, b = shift | q << 8
+//     with q the 256 rows taken, RHS chunk c of d right-hand sides.
+enum UnitKind { kUnitSeg8 = 0, kUnitSeg16 = 1, kUnitSeg32 = 2, kUnitCol = 3, kUnitCta = 4, kUnitWide = 5 };
 struct SolveUnit {
-  int32_t kind, a, b, c, d;
+  int32_t x, a, b, c;
 };
-constexpr int kSolveChunk = 8;  // largest RHS chunk of a task (segment tasks use exactly 8)
 
-// One launch solving every level of the forest (forward = L, bottom-up, or
-// backward = U, top-down).  ticket (1 int) and done (S*K ints) must be zero;
-// nch[s] is the number of RHS chunks (tasks) per (front s, k); err is set to 1
-// if a bounded dependency wait gave up after `polls` polls (<= 0: the default
-// limit of 2^22 polls); ctas = resident CTAs per SM the kernel is compiled
-// for (2, 3 or 4; <= 0: 3 for FP32, 2 for FP64).  Adaptive sweeps: ucount
-// (device, or nullptr) holds the length of a compacted list (nunits is then
-// its capacity), act[g] (device, or nullptr) = 0 skips instance g's fronts.
-int launch_solve_persistent(int precision, bool forward, const SymDev& sd, const SolveUnit* units,
-                            int nunits, const int* ucount, const uint8_t* act, int* ticket, int* done,
-                            int* err, const int* nch, const int32_t* d_all, const void* fronts,
-                            const double* rhs, int rhs_mode, void* V, double* out, double* acc, int32_t R,
-                            int32_t K, int32_t max_blk_F, int32_t ctas, int64_t polls, cudaStream_t st);
-// RHS chunk for the CTAs solving one big front at a time (persistent schedule)
-int pick_chunk(int fronts_in_level, int K, int R);
-int launch_forward_level(int precision, bool trans, const SymDev& sd, const LevelPlan& lp,
-                         const int32_t* d_all, const void* fronts, const double* rhs,
-                         int rhs_mode, void* V, int32_t R, int32_t K, cudaStream_t st);
-int launch_backward_level(int precision, bool trans, const SymDev& sd, const LevelPlan& lp,
-                          const int32_t* d_all, const void* fronts, const void* V, double* out,
-                          double* acc, int32_t R, int32_t K, cudaStream_t st);
+// What a solve task needs to know of its front, in unit-list order: one
+// 64-byte read in place of a chain of lookups.  needF = its children's tasks,
+// needB = its parent's, as the completion counters count them.
+enum FrontWhole { kSelfWhole = 1, kParentWhole = 2 };
+struct alignas(16) FrontDesc {
+  int32_t c0, ns, F, inst;
+  int64_t fo, vo;  // prefix sums of F^2 and F
+  int64_t ro;      // first update row in `rows`
+  int32_t parent, s;
+  int32_t needF, needB;
+  int32_t flag;   // more than 32 pivots: first of its counters in `wide`
+  int32_t whole;  // FrontWhole: counted at group 0 only
+};
+
+constexpr int kCtrStride = 8;  // ints between completion counters: a 32-byte sector each
+
+constexpr int kSolveChunk = 8;  // right-hand sides of a segment task, where there are several
+
+// xd_mode: what a backward solve does with its FP64 output
+enum XdMode { kXdStore = 0, kXdAdd = 1 };
+
+// Arguments of one solve launch (solve_persistent.h says what the arrays hold).
+template <typename T>
+struct SolveArgs {
+  const FrontDesc* desc;
+  const int64_t *inv_off, *inv_pos;
+  const int32_t *rows, *perm;
+  const SolveUnit* units;
+  int32_t first, nunits;  // the launch's units are first .. first + nunits - 1
+  const int* ucount;      // length of a compacted list, or nullptr: nunits
+  const uint8_t* act;     // per-instance flags of the adaptive sweeps, or nullptr: all
+  int* ticket;            // zero
+  int* done;              // [S][NG] finished tasks, zero; nullptr (one launch per stage): nothing to wait for
+  int* wide;              // solved blocks per (front with more than 32 pivots, shift, chunk), zero
+  int* err;               // set if a wait gave up
+  int64_t polls;
+  const T* fronts;
+  const double* b;        // broadcast right-hand side, or nullptr: rk
+  const T* rk;
+  T* V;
+  T* xt;
+  double* xd;             // FP64 output, or nullptr
+  int32_t xd_mode, R, K, RV, RX, vec, vecd;
+  int32_t NG;     // groups of the completion counters: K shifts, or ceil(K RV / 32) column groups
+  int32_t stage;  // per-warp shared memory of the column tasks (set by the launch)
+};
+
+// row strides of the vectors for R right-hand sides: in the factor precision
+// (16-byte accesses) and in FP64
+inline int32_t rhs_stride(int precision, int32_t R) {
+  const int32_t n = precision == PISP_FP32 ? 4 : 2;
+  return R <= 2 && R < n ? R : (R + n - 1) / n * n;
+}
+inline int32_t rhs_stride64(int32_t R) { return R == 1 ? 1 : (R + 1) / 2 * 2; }
+
+// One launch of the forward (L, or U^T with trans) or backward (U, L^T) solve;
+// ctas = resident CTAs per SM it is compiled for (2, 3, 4; <= 0: 3 for FP32,
+// 2 for FP64); wide = the largest chunk of a front with more than 32 pivots.  Returns the kernels launched or -1.
+template <typename T, bool FWD>
+int launch_solve_dir(bool trans, const SolveArgs<T>& a, int32_t nunits, int32_t wide, int32_t ctas, cudaStream_t st);
+// right-hand sides and rows of a task of a front with more than 32 pivots
+int wide_chunk(int precision, int R);
+constexpr int kWideUnitRows = 256;
 int launch_combine(const SymDev& sd, const double* X, const Shifts& sh, int32_t R, double* x,
                    cudaStream_t st);
 // The instances still iterating in the adaptive sweeps (device arrays
@@ -244,14 +288,14 @@ struct ActiveSet {
 // of instances that have stopped (whose correction is then exactly 0, for a
 // solve that is not gated); only the rows of the active set.
 enum ResidualMode { kResAll = 0, kResZeroStopped = 1, kResActive = 2 };
-int launch_residual_per_k(const SymDev& sd, const double* vals, const double* D,
+int launch_residual_per_k(int precision, const SymDev& sd, const double* vals, const double* D,
                           const Shifts& sh, const double* b, const double* X, int32_t R,
-                          double* Rk, const ActiveSet& as, int mode, cudaStream_t st);
+                          void* Rk, const ActiveSet& as, int mode, cudaStream_t st);
 // Per instance g of the active set: X += Y on its rows, then per RHS r the
 // largest |Y| and |X| over its rows and all k, atomically maxed into
 // dmax/xmax [G][R] (zero on entry) as bit patterns.
-int launch_refine_stats(const SymDev& sd, const ActiveSet& as, double* X, const double* Y, int32_t K, int32_t R,
-                        unsigned long long* dmax, unsigned long long* xmax, cudaStream_t st);
+int launch_refine_stats(int precision, const SymDev& sd, const ActiveSet& as, double* X, const void* Y, int32_t K,
+                        int32_t R, unsigned long long* dmax, unsigned long long* xmax, cudaStream_t st);
 // One CTA: the stopping test after sweep s = *sweep + 1 (s >= S: every
 // instance stops), *sweep = s, nsw[g] = the sweeps instance g took, dmax /
 // xmax zeroed again, then the active set: pre[g] = the active instances
@@ -274,9 +318,9 @@ int launch_compact_units(const SolveUnit* uf, const int32_t* rf, int32_t nf, Sol
                          const int32_t* rb, int32_t nb, SolveUnit* cb, const int32_t* pre, int32_t* cnt,
                          int32_t* ucount, cudaStream_t st);
 // FP64 residuals of the transposed perturbed systems (adjoint sweeps)
-int launch_residual_T_per_k(const SymDev& sd, const double* vals, const double* D,
+int launch_residual_T_per_k(int precision, const SymDev& sd, const double* vals, const double* D,
                             const Shifts& sh, const double* g, const double* Lam, int32_t R,
-                            double* Rk, cudaStream_t st);
+                            void* Rk, cudaStream_t st);
 int launch_residual(const SymDev& sd, const double* vals, const double* b, const double* x,
                     int32_t R, double* r, cudaStream_t st);
 int launch_axpy(int64_t n, const double* y, double* x, cudaStream_t st);

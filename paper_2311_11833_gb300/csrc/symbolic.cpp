@@ -539,12 +539,10 @@ std::string analyze(int32_t G, const int32_t* n, const int64_t* row_ptr,
         S.inv_a[q] = a;
       }
     }
-    S.inv_vbase.resize(S.inv_child.size());
     S.inv_cF.resize(S.inv_child.size());
     S.inv_col.resize(S.inv_child.size());
     for (size_t q = 0; q < S.inv_child.size(); ++q) {
       const Supernode& c = S.sn[S.inv_child[q]];
-      S.inv_vbase[q] = S.vec_off[S.inv_child[q]];
       S.inv_cF[q] = c.F();
       S.inv_col[q] = c.ns() + S.inv_a[q];
     }
@@ -706,14 +704,14 @@ std::string validate(const Symbolic& S) {
   // inverse extend-add map
   if (!prefix_ok(S.inv_off, (size_t)V + 1, (int64_t)S.inv_child.size())) return bad("inverse map offsets");
   const size_t nI = S.inv_child.size();
-  if (S.inv_a.size() != nI || S.inv_vbase.size() != nI || S.inv_cF.size() != nI || S.inv_col.size() != nI)
+  if (S.inv_a.size() != nI || S.inv_cF.size() != nI || S.inv_col.size() != nI)
     return bad("inverse map sizes");
   for (int64_t p = 0; p < nS; ++p)
     for (int64_t j = 0; j < S.sn[p].F(); ++j)
       for (int64_t q = S.inv_off[S.vec_off[p] + j]; q < S.inv_off[S.vec_off[p] + j + 1]; ++q) {
         const int32_t c = S.inv_child[q];
         if (c < 0 || c >= nS || S.sn[c].parent != p || S.inv_a[q] < 0 || S.inv_a[q] >= S.sn[c].ms ||
-            S.emap[S.sn[c].row_off + S.inv_a[q]] != j || S.inv_vbase[q] != S.vec_off[c] ||
+            S.emap[S.sn[c].row_off + S.inv_a[q]] != j ||
             S.inv_cF[q] != S.sn[c].F() || S.inv_col[q] != S.sn[c].ns() + S.inv_a[q])
           return bad("inverse map entries");
       }

@@ -63,7 +63,6 @@ struct Symbolic {
   std::vector<int64_t> inv_off;        // [sum F + 1]
   std::vector<int32_t> inv_child;      // child supernode
   std::vector<int32_t> inv_a;          // row index in the child's update part
-  std::vector<int64_t> inv_vbase;      // vec_off of the child (its front-vector block)
   std::vector<int32_t> inv_cF;         // the child's front size
   std::vector<int32_t> inv_col;        // ns(child) + inv_a: position in the child's front
   // children lists
