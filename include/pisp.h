@@ -71,7 +71,12 @@ typedef struct pisp_options {
                              assembly forest (forward by height, backward by
                              depth) and wait (boundedly) for their dependencies;
                              1 = one launch per height, or depth */
-  int32_t factor_policy;  /* fronts wider than 64: 0 (default) = one CTA each while
+  int32_t factor_policy;  /* 0 (default) = by the work: one launch as under 4, with
+                             its options chosen, where that was measured ahead
+                             (FP32 while no front is wider than 1024; FP64 from
+                             8192 (front, shift) pairs on), else level by level:
+                             fronts of at most 32 by segments (FP64: one CTA
+                             each), wider ones one CTA each while
                              the front fits in shared memory; larger fronts, of
                              any size, in one persistent launch per level where
                              each CTA owns a tile (a 32-column block of a (front,
@@ -80,16 +85,16 @@ typedef struct pisp_options {
                              applies the earlier panels as they are released;
                              1 = thread-block clusters of up to 8 CTAs holding the
                              front in distributed shared memory wherever it fits;
-                             2 = as 0 but larger fronts as a tile DAG (column-block
+                             2 = level by level, larger fronts as a tile DAG (column-block
                              assembly, panel and update tasks in one persistent
                              launch per level, with look-ahead);
-                             3 = as 0 but larger fronts by a blocked factorisation
+                             3 = level by level, larger fronts by a blocked factorisation
                              in global memory (one panel launch and one
                              tiled-update launch per 32 pivots);
                              4 = ONE persistent launch for every level, shift
-                             and instance: fronts of at most 32 one warp each,
-                             fronts up to factor_smem_maxF one CTA each in
-                             shared memory, wider fronts as owner tiles;
+                             and instance: fronts of at most 32 by segments of
+                             8, 16 or 32 lanes, fronts up to factor_smem_maxF one
+                             CTA each in shared memory, wider fronts as owner tiles;
                              a task waits (boundedly) only for its children's
                              completion counters */
   int32_t solve_kfuse;    /* solves by segments (forward, and backward with one

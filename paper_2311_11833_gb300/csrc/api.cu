@@ -58,7 +58,7 @@ struct pisp_handle {
   pisp::Symbolic sym;
   double analyze_ms = 0.0;
   // device symbolic
-  Buf c0, ns, ms, inst, front_off, vec_off, row_off, child_off, child, amap_off, amap_src,
+  Buf c0, ns, ms, inst, front_off, vec_off, row_off, child_off, child, cdesc, amap_off, amap_src,
       amap_dst, amap_coff, rows, emap, perm, iperm, row_inst, row_ptr, col, parent, inv_off, inv_child, inv_a, inv_pos,
       inv_cF, inv_col, at_ptr, at_row, at_src, pcol, at_prow;
   // persistent solve schedule (depends on K and R)
@@ -108,6 +108,8 @@ struct pisp_handle {
   // warp-front list, completion targets, counters and owner release flags
   int32_t n_ftasks = 0, fac_CH = 32, fac_nflags = 0;
   size_t fac_smem = 0;
+  bool fac_single = false;  // the plan is one launch (one_launch), at fac_ctas CTAs per SM
+  int32_t fac_ctas = 0;
   double fac_bytes = 0;
   Buf d_ftasks, d_fwl, d_fneed, fdone, fflags, fticket;
   // numeric state
@@ -242,6 +244,8 @@ int upload(pisp_handle* h, Buf& b, const std::vector<T>& v) {
     if (rc_) return rc_;  \
   } while (0)
 
+constexpr int64_t kManyTasks = 8192;  // (front, shift) pairs beyond which a factorisation has work for every SM
+
 // Factor path of a front of size F > 64: 0 = one CTA with the front in shared
 // memory, C >= 1 = a cluster of C CTAs (distributed shared memory), -1 = the
 // blocked global-memory path.  Policy 0 (default): one CTA while the front
@@ -252,15 +256,40 @@ int factor_path(const pisp_handle* h, int F, int precision) {
   return F <= pisp::small_front_limit(precision) ? 0 : -1;
 }
 
-// Task list of the one-launch factorisation (factor policy 4): per level,
+// Whether the factorisation is one persistent launch: under policy 4, and under
+// policy 0 by what was measured (us level by level / in one launch).  In FP32 it
+// saves the launches and the waits between levels and size classes: 1354 buses
+// 344 / 245, 777 buses 230 / 191, 5 grids 280 / 192, 64 grids 1784 / 897; with a
+// root of 1596 rows the owner tiles are all that counts, and those alone on an SM
+// with 255 registers a thread are ahead (10000 buses 3124 / 3272).  In FP64 one
+// grid's fronts are bound by the FP64 pipe whichever way they are launched, and
+// CTAs for all of them are ahead of segments (300 buses 160 / 168, 1354 buses
+// 703 / 725); many grids' fronts fill the SMs (48 grids 3939 / 2470).
+bool one_launch(const pisp_handle* h, int precision, int32_t K) {
+  if (h->factor_policy != 0) return h->factor_policy == 4;
+  const int64_t tasks = (int64_t)h->sym.sn.size() * K;
+  return precision == PISP_FP32 ? h->sym.max_front <= 1024 : tasks >= kManyTasks;
+}
+
+// Task list of the one-launch factorisation (one_launch): per level,
 // bottom-up, the owner tiles of the fronts wider than the shared-memory
 // limit (in (block, chunk) order, every tile after the ones it waits for),
-// then one task per (front, k) for the shared-memory fronts, then groups of
-// 8 (front, k) warp tasks for the fronts of at most 32.
+// then one task per (front, k) for the shared-memory fronts, then the segment
+// tasks of the fronts of at most 32 rows by size class, 256 / SEG a record.
 int build_persistent_factor(pisp_handle* h, int precision, int32_t K) {
   const pisp::Symbolic& S = h->sym;
-  const int Fc = h->factor_smem_maxF > 0 ? std::min(h->factor_smem_maxF, pisp::persistent_cta_front_limit(precision))
-                                         : pisp::persistent_cta_front_limit(precision);
+  int smem_maxF = h->factor_smem_maxF;
+  h->fac_ctas = h->factor_ctas;
+  if (h->factor_policy == 0) {
+    // many FP32 fronts: three CTAs an SM with the fronts that three can hold
+    // (64 grids 897 us, 993 with two); few: two, the registers are worth more
+    // (2000 buses 334 us, 372 with three)
+    const bool three = precision == PISP_FP32 && (int64_t)S.sn.size() * K >= kManyTasks;
+    smem_maxF = three ? 128 : 0;
+    h->fac_ctas = three ? 3 : 2;
+  }
+  const int Fc = smem_maxF > 0 ? std::min(smem_maxF, pisp::persistent_cta_front_limit(precision))
+                               : pisp::persistent_cta_front_limit(precision);
   int maxBig = 0, maxCta = 0;
   for (const auto& sn : S.sn) {
     if (sn.F() > Fc) maxBig = std::max(maxBig, sn.F());
@@ -268,7 +297,7 @@ int build_persistent_factor(pisp_handle* h, int precision, int32_t K) {
   }
   const int CH = maxBig > 0 ? pisp::owner_chunk_rows(precision, maxBig, h->factor_tc) : 32;
   std::vector<pisp::FactorTask> ft;
-  std::vector<int32_t> wl, need(S.sn.size(), 1);
+  std::vector<int32_t> wl, ntask(S.sn.size(), 1);  // tasks per (front, k)
   int64_t nflags = 0;
   for (int l = 0; l < S.n_levels; ++l) {
     std::vector<int32_t> lst(S.level_sn.begin() + S.level_off[l], S.level_sn.begin() + S.level_off[l + 1]);
@@ -276,10 +305,10 @@ int build_persistent_factor(pisp_handle* h, int precision, int32_t K) {
       const int fa = S.sn[a].F(), fb = S.sn[b].F();
       return fa != fb ? fa > fb : a < b;
     });
-    std::vector<int32_t> big, cta, warp;
+    std::vector<int32_t> big, cta, seg[3];
     for (int32_t sn : lst) {
       const int F = S.sn[sn].F();
-      (F > Fc ? big : (F > 32 ? cta : warp)).push_back(sn);
+      (F > Fc ? big : (F > 32 ? cta : seg[F > 16 ? 2 : (F > 8 ? 1 : 0)])).push_back(sn);
     }
     if (!big.empty()) {
       std::vector<pisp::BigFrontHost> bh;
@@ -290,26 +319,30 @@ int build_persistent_factor(pisp_handle* h, int precision, int32_t K) {
       for (const auto& t : tk)
         ft.push_back({pisp::kFacOwner, big[t.b], t.k, t.p, t.j, (int32_t)(nflags + t.flags)});
       for (size_t b = 0; b < big.size(); ++b)
-        need[big[b]] = ((bh[b].F + 31) / 32) * ((bh[b].F + CH - 1) / CH);
+        ntask[big[b]] = ((bh[b].F + 31) / 32) * ((bh[b].F + CH - 1) / CH);
       nflags += nfl;
       if (nflags >= INT32_MAX) return fail(h, PISP_ERR_UNSUPPORTED, "too many factor flags");
     }
     for (int32_t sn : cta)
       for (int k = 0; k < K; ++k) ft.push_back({pisp::kFacCta, sn, k, 0, 0, 0});
-    if (!warp.empty()) {
-      const int64_t off = (int64_t)wl.size(), tasks = (int64_t)warp.size() * K;
-      if (off + (int64_t)warp.size() >= INT32_MAX || tasks >= INT32_MAX)
+    for (int w = 2; w >= 0; --w) {
+      if (seg[w].empty()) continue;
+      const int64_t off = (int64_t)wl.size(), tasks = (int64_t)seg[w].size() * K;
+      if (off + (int64_t)seg[w].size() >= INT32_MAX || tasks >= INT32_MAX)
         return fail(h, PISP_ERR_UNSUPPORTED, "too many factor tasks");
-      wl.insert(wl.end(), warp.begin(), warp.end());
-      for (int64_t b = 0; b < tasks; b += 8)
-        ft.push_back({pisp::kFacWarp, (int32_t)off, 0, (int32_t)b, (int32_t)tasks, 0});
+      wl.insert(wl.end(), seg[w].begin(), seg[w].end());
+      for (int64_t b = 0; b < tasks; b += 256 / (8 << w))
+        ft.push_back({pisp::kFacSeg8 + w, (int32_t)off, 0, (int32_t)b, (int32_t)tasks, 0});
     }
   }
+  std::vector<int32_t> need(S.sn.size(), 0);
+  for (size_t q = 0; q < S.sn.size(); ++q)
+    if (S.sn[q].parent >= 0) need[S.sn[q].parent] += ntask[q];
   if ((int64_t)ft.size() >= INT32_MAX) return fail(h, PISP_ERR_UNSUPPORTED, "too many factor tasks");
   TRY(upload(h, h->d_ftasks, ft));
   TRY(upload(h, h->d_fwl, wl));
   TRY(upload(h, h->d_fneed, need));
-  if (!h->fdone.ensure(S.sn.size() * (size_t)K * sizeof(int)) || !h->fflags.ensure((size_t)nflags * sizeof(int)) ||
+  if (!h->fdone.ensure(S.sn.size() * (size_t)K * pisp::kCtrStride * sizeof(int)) || !h->fflags.ensure((size_t)nflags * sizeof(int)) ||
       !h->fticket.ensure(sizeof(int)))
     return fail(h, PISP_ERR_OOM, "device allocation failed (factor schedule)");
   h->n_ftasks = (int32_t)ft.size();
@@ -330,6 +363,7 @@ int build_plans(pisp_handle* h, int precision) {
   h->h_bigF.clear();
   h->h_dag.clear();
   h->dag_max_flags = 0;
+  const bool single = one_launch(h, precision, h->K_hint);
   for (int l = 0; l < S.n_levels; ++l) {
     pisp::LevelPlan& lp = h->plans[l];
     std::vector<int32_t> lst(S.level_sn.begin() + S.level_off[l],
@@ -338,10 +372,11 @@ int build_plans(pisp_handle* h, int precision) {
       const int fa = S.sn[a].F(), fb = S.sn[b].F();
       return fa != fb ? fa < fb : a < b;
     });
-    // on-chip fronts: single-CTA classes up to 64, then clusters of 1..8 CTAs
-    const int fcls[3] = {16, 32, 64};
+    // on-chip fronts: segment classes up to 32 (one class of CTAs in FP64),
+    // single-CTA classes up to 64, then clusters of 1..8 CTAs
+    const int fcls[4] = {8, 16, 32, 64};
     int lo = 0;
-    for (int c = 0; c < 3; ++c) {
+    for (int c = precision == PISP_FP32 ? 0 : 2; c < 4; ++c) {
       pisp::LevelPlan::Group G{(int64_t)h->h_small.size(), 0, 0, 0};
       for (int32_t s : lst) {
         const int F = S.sn[s].F();
@@ -397,7 +432,7 @@ int build_plans(pisp_handle* h, int precision) {
     // any front size) or the tile DAG (policy 2, while a panel fits in shared
     // memory); else (and under policies 1 and 3) one panel launch and one
     // update launch per 32 pivots
-    const bool owner = h->factor_policy == 0;
+    const bool owner = h->factor_policy == 0 && !single;
     const bool dag = h->factor_policy == 2 && lp.big_maxF <= pisp::max_dag_front(precision);
     if (lp.big_count > 0 && (owner || dag)) {
       std::vector<pisp::DagTask> tk;
@@ -442,7 +477,8 @@ int build_plans(pisp_handle* h, int precision) {
   TRY(upload(h, h->d_dag, h->h_dag));
   if (!h->dag_ticket.ensure(sizeof(int)) || !h->dag_flags.ensure((size_t)h->dag_max_flags * sizeof(int)))
     return fail(h, PISP_ERR_OOM, "device allocation failed (factor schedule)");
-  if (h->factor_policy == 4) {
+  h->fac_single = single;
+  if (single) {
     TRY(build_persistent_factor(h, precision, h->K_hint));
     h->fac_bytes = 0;
     for (const auto& lp : h->plans) h->fac_bytes += lp.bytes_fsmall + lp.bytes_fbig;
@@ -1135,6 +1171,17 @@ int analyze_impl(pisp_handle* h, int32_t G, const int32_t* n, const int64_t* row
   TRY(upload(h, h->row_off, row_off));
   TRY(upload(h, h->child_off, child_off));
   TRY(upload(h, h->child, S.child));
+  {
+    std::vector<pisp::ChildDesc> cd(S.child.size());
+    for (int s = 0; s < nS; ++s)
+      for (int64_t q = S.child_off[s]; q < S.child_off[s + 1]; ++q) {
+        const pisp::Supernode& c = S.sn[S.child[q]];
+        cd[q] = {S.front_off[S.child[q]], c.ns(), c.F(), 0, {}};
+        if (S.sn[s].F() <= 32)
+          for (int32_t a = 0; a < c.ms; ++a) cd[q].mask |= 1u << S.emap[c.row_off + a];
+      }
+    TRY(upload(h, h->cdesc, cd));
+  }
   TRY(upload(h, h->amap_off, S.amap_off));
   TRY(upload(h, h->amap_src, S.amap_src));
   TRY(upload(h, h->amap_dst, S.amap_dst));
@@ -1193,6 +1240,7 @@ int analyze_impl(pisp_handle* h, int32_t G, const int32_t* n, const int64_t* row
   sd.row_off = h->row_off.as<int64_t>();
   sd.child_off = h->child_off.as<int32_t>();
   sd.child = h->child.as<int32_t>();
+  sd.cdesc = h->cdesc.as<pisp::ChildDesc>();
   sd.amap_off = h->amap_off.as<int64_t>();
   sd.amap_src = h->amap_src.as<int32_t>();
   sd.amap_dst = h->amap_dst.as<int32_t>();
@@ -1320,17 +1368,17 @@ int pisp_factor_perturbed(pisp_handle* h, const double* values, const double* D,
   CK(cudaMemsetAsync(h->serr.p, 0, sizeof(int), h->stream));
   h->launches = 0;
   const pisp::Shifts sh = make_shifts(h, h->beta);
-  if (h->factor_policy == 4) {
+  if (h->fac_single) {
     // every level, every shift and every instance in one persistent launch
     CK(cudaMemsetAsync(h->fticket.p, 0, sizeof(int), h->stream));
-    CK(cudaMemsetAsync(h->fdone.p, 0, S.sn.size() * (size_t)K * sizeof(int), h->stream));
+    CK(cudaMemsetAsync(h->fdone.p, 0, S.sn.size() * (size_t)K * pisp::kCtrStride * sizeof(int), h->stream));
     if (h->fac_nflags) CK(cudaMemsetAsync(h->fflags.p, 0, (size_t)h->fac_nflags * sizeof(int), h->stream));
     const int pb = prof_begin(h);
     const int n = pisp::launch_factor_persistent(
         precision, h->sd, h->d_ftasks.as<pisp::FactorTask>(), h->n_ftasks, h->fticket.as<int>(), h->fdone.as<int>(),
         h->d_fneed.as<int>(), h->fflags.as<int>(), h->serr.as<int>(), h->d_fwl.as<int32_t>(), h->vals.as<double>(),
         h->D.as<double>(), sh, h->fronts.p, h->status.as<int32_t>(), h->badcol.as<int32_t>(), h->fac_CH,
-        h->fac_smem, h->wait_polls, h->factor_tc, h->factor_ctas, h->stream);
+        h->fac_smem, h->factor_policy == 4 ? h->wait_polls : 0, h->factor_tc, h->fac_ctas, h->stream);
     TRY(count(h, n));
     prof_end(h, pb, PISP_PROF_FACTOR, K * h->fac_bytes, n);
     h->factored = true;

@@ -161,134 +161,382 @@ __device__ __forceinline__ void extend_add_columns(const SymDev& sd, int s, int 
   }
 }
 
-// ---------------------------------------------------------------------------
-// Small fronts: whole front in shared memory, one CTA per (front, k).
-// ---------------------------------------------------------------------------
-// One (front s, perturbation k) in the shared-memory buffer f (F*F
-// elements): assembly (original entries, t_k D, children's Schur complements
-// in child order per element), ns steps of pivot-free elimination, write to
-// the front storage.  Any number of threads that is a multiple of 32.
+// One warp: the children's update blocks added into the destination columns
+// [d0, d1) of front s, all its rows, stored at dst[row + col * ld].  The columns'
+// entries of the inverse extend-add map are consecutive; 32 are resolved at a
+// time, one a lane, and four child columns are in flight at a time (two rows a
+// lane), so that a memory latency covers four contributions and not one.  The
+// additions to an element follow a fixed order.
 template <typename T>
-__device__ __forceinline__ void front_cta(const SymDev& sd, int s, int k, const double* __restrict__ vals,
-                                          const double* __restrict__ D, const Shifts& sh,
-                                          T* __restrict__ fronts, int32_t* status, int32_t* badcol, T* f) {
-  const int K = sh.K;
-  const int ns = sd.ns[s], ms = sd.ms[s], F = ns + ms;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int FF = F * F;
-  for (int q = tid; q < FF; q += nt) f[q] = T(0);
-  __syncthreads();
-  // 1a. entries of A owned by this front (duplicates add up)
-  const int64_t a0 = sd.amap_off[s], a1 = sd.amap_off[s + 1];
-  for (int64_t q = a0 + tid; q < a1; q += nt) atomicAdd(&f[sd.amap_dst[q]], (T)vals[sd.amap_src[q]]);
-  // 1b. the perturbation t_k D on the pivot diagonal
-  const double tk = sh.t[k];
+__device__ __forceinline__ void extend_add_flat(const SymDev& sd, int s, int k, int K, const T* __restrict__ fronts,
+                                                T* dst, int ld, int d0, int d1) {
+  constexpr int NE = 4;
+  const int lane = threadIdx.x & 31;
+  const int64_t vo = sd.vec_off[s];
+  const int64_t e1 = sd.inv_off[vo + d1];
+  for (int64_t eb = sd.inv_off[vo + d0]; eb < e1; eb += 32) {
+    const int ne = (int)min((int64_t)32, e1 - eb);
+    int64_t src = 0, ro = 0;
+    int cms = 0, dc = 0;
+    if (lane < ne) {
+      const int ch = sd.inv_child[eb + lane], ca = sd.inv_a[eb + lane];
+      const int cF = sd.inv_cF[eb + lane], col = sd.inv_col[eb + lane];
+      ro = sd.row_off[ch];
+      cms = cF - (col - ca);
+      src = (int64_t)K * sd.front_off[ch] + (int64_t)k * cF * cF + (int64_t)col * cF + (col - ca);
+      dc = sd.emap[ro + ca] * ld;
+    }
+    for (int g = 0; g < ne; g += NE) {
+      const T* p[NE];
+      const int32_t* em[NE];
+      int m[NE], d[NE], most = 0;
+#pragma unroll
+      for (int q = 0; q < NE; ++q) {
+        p[q] = fronts + __shfl_sync(0xffffffffu, src, g + q);
+        em[q] = sd.emap + __shfl_sync(0xffffffffu, ro, g + q);
+        m[q] = __shfl_sync(0xffffffffu, cms, g + q);
+        d[q] = __shfl_sync(0xffffffffu, dc, g + q);
+        most = max(most, m[q]);
+      }
+      for (int a = lane; a < most + lane; a += 64) {  // warp-uniform trips
+        int r0[NE], r1[NE];
+        T v0[NE], v1[NE];
+#pragma unroll
+        for (int q = 0; q < NE; ++q) {
+          r0[q] = a < m[q] ? em[q][a] : -1;
+          v0[q] = a < m[q] ? __ldcg(p[q] + a) : T(0);
+          r1[q] = a + 32 < m[q] ? em[q][a + 32] : -1;
+          v1[q] = a + 32 < m[q] ? __ldcg(p[q] + a + 32) : T(0);
+        }
+#pragma unroll
+        for (int q = 0; q < NE; ++q) {
+          if (r0[q] >= 0) dst[r0[q] + d[q]] += v0[q];
+          if (r1[q] >= 0) dst[r1[q] + d[q]] += v1[q];
+          __syncwarp();  // the next contribution may land on another lane's element
+        }
+      }
+    }
+  }
+}
+
+// leading dimension of a front in shared memory: odd, so that rows and columns
+// both fall on distinct banks
+__host__ __device__ __forceinline__ int front_ld(int F) { return F | 1; }
+
+// Pivot-free LU of ns pivots of the F x F front f (leading dimension ld) in
+// shared memory, by the whole CTA, in panels of NB pivots: one warp factors the
+// panel's diagonal block in registers (lane = row), then threads take the rows
+// below it and the columns beside it, one each, and 4 x 4 register tiles update
+// the rest: three barriers a panel.  (One pivot at a time, two barriers and a
+// pass over the whole front in shared memory each, a 213-row front took 500 us.)
+template <typename T>
+__device__ __forceinline__ void front_lu(T* f, int ld, int F, int ns, T* rinv, const SymDev& sd, int s, int k, int K,
+                                         int32_t* status, int32_t* badcol) {
+  constexpr int NB = 16;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
   const int c0 = sd.c0[s];
-  for (int c = tid; c < ns; c += nt) atomicAdd(&f[c * (F + 1)], (T)(tk * D[sd.perm[c0 + c]]));
-  __syncthreads();
-  // 1c. extend-add of the children's Schur complements, child by child (each
-  // element receives its contributions in child order): the threads take the
-  // entries of one child's update block, which land on distinct elements
-  for (int ci = sd.child_off[s]; ci < sd.child_off[s + 1]; ++ci) {
-    const int c = sd.child[ci];
-    const int cns = sd.ns[c], cms = sd.ms[c], cF = cns + cms;
-    const T* cf = fronts + (int64_t)K * sd.front_off[c] + (int64_t)k * cF * cF;
-    const int32_t* em = sd.emap + sd.row_off[c];
-    const int n2 = cms * cms;
-    for (int q = tid; q < n2; q += nt) {
-      const int a = q % cms, b = q / cms;  // child update row a, column b
-      f[em[a] + em[b] * F] += cf[(cns + a) + (int64_t)(cns + b) * cF];
+  for (int p0 = 0; p0 < ns; p0 += NB) {
+    const int nb = min(NB, ns - p0);
+    T* fd = f + p0 + p0 * ld;  // the diagonal block
+    if (tid < 32) {
+      T d[NB];
+#pragma unroll
+      for (int c = 0; c < NB; ++c) d[c] = lane < nb && c < nb ? fd[lane + c * ld] : T(0);
+#pragma unroll 1
+      for (int c = 0; c < nb; ++c) {  // d[0] is column c: the row moves down a place each step
+        const T piv = __shfl_sync(0xffffffffu, d[0], c);
+        if (lane == 0) check_pivot(piv, sd, s, k, K, c0 + p0 + c, status, badcol);
+        const T rp = T(1) / piv;
+        if (lane == 0) rinv[c] = rp;
+        const T l = lane > c ? d[0] * rp : T(0);
+        if (lane < nb) fd[lane + c * ld] = lane > c ? l : d[0];
+#pragma unroll
+        for (int j = 1; j < NB; ++j) d[j - 1] = d[j] - l * __shfl_sync(0xffffffffu, d[j], c);
+      }
+    }
+    __syncthreads();
+    const int t0 = p0 + nb, m = F - t0;
+    for (int q = tid; q < 2 * m; q += nt) {
+      // a row below, L(i, :) = A(i, :) U^-1, or a column beside, U(:, j) = L^-1 A(:, j)
+      const bool low = q < m;
+      T* v = low ? f + t0 + q + p0 * ld : f + p0 + (t0 + q - m) * ld;
+      const int vs = low ? ld : 1, ds = low ? ld : 1;  // strides of the vector, and of the block's row or column
+      T x[NB];
+#pragma unroll
+      for (int c = 0; c < NB; ++c) x[c] = c < nb ? v[c * vs] : T(0);
+#pragma unroll 1
+      for (int c = 0; c < nb; ++c) {
+        const T y = low ? x[0] * rinv[c] : x[0];
+        v[c * vs] = y;
+        const T* e = fd + c * (ld + 1);  // the pivot; then along its row (U) or column (L)
+#pragma unroll
+        for (int j = 1; j < NB; ++j) x[j - 1] = x[j] - (c + j < nb ? e[j * ds] * y : T(0));
+      }
+    }
+    __syncthreads();
+    // 64 x 64 tiles, 16 x 16 threads, one tile per 256 threads
+    const int tx = tid & 15, ty = (tid >> 4) & 15, tpd = (m + 63) >> 6;
+    for (int t = tid >> 8; t < tpd * tpd; t += nt >> 8) {
+      const int ib = t0 + (t % tpd) * 64 + tx, jb = t0 + (t / tpd) * 64 + ty;
+      T acc[4][4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
+      const T* lp = f + p0 * ld;
+      const T* up = f + p0;
+#pragma unroll 2
+      for (int c = 0; c < nb; ++c) {
+        T l[4], u[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) l[a] = ib + 16 * a < F ? lp[ib + 16 * a + c * ld] : T(0);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) u[b] = jb + 16 * b < F ? up[c + (jb + 16 * b) * ld] : T(0);
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) acc[a][b] += l[a] * u[b];
+      }
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+          if (ib + 16 * a < F && jb + 16 * b < F) f[ib + 16 * a + (jb + 16 * b) * ld] -= acc[a][b];
     }
     __syncthreads();
   }
-  // 2. ns steps of pivot-free elimination
-  for (int p = 0; p < ns; ++p) {
-    const T piv = f[p * (F + 1)];
-    if (tid == 0) check_pivot(piv, sd, s, k, K, c0 + p, status, badcol);
-    const int m = F - p - 1;
-    const T rp = T(1) / piv;
-    for (int i = tid; i < m; i += nt) f[(p + 1 + i) + p * F] *= rp;
-    __syncthreads();
-    {
-      // lanes run down a column (consecutive i), warps take columns
-      const int lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
-      const T* lc = f + p * F;
-      for (int j = p + 1 + wid; j < F; j += nw) {
-        const T u = f[p + j * F];
-        T* col = f + j * F;
-        for (int i = p + 1 + lane; i < F; i += 32) col[i] -= lc[i] * u;
+}
+
+// The same in FP64, where the pipe (2 FMA a clock per SM) bounds the front and
+// every idle lane of an instruction costs as much as a busy one: one pivot at a
+// time, the trailing elements dealt out to the threads one by one, and one
+// barrier a pivot: warp 0 takes the next pivot's column first, inverts the
+// pivot and scales the column while the other warps update the rest (all warps
+// inverting it took as long as a 40-row front's update).
+template <typename T>
+__device__ __forceinline__ void front_lu_flat(T* f, int ld, int F, int ns, const SymDev& sd, int s, int k, int K,
+                                              int32_t* status, int32_t* badcol) {
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const int c0 = sd.c0[s];
+  for (int p = -1; p < ns; ++p) {
+    // column p is scaled; eliminate it from columns p+1 .. F-1, and prepare column p+1
+    const T* lc = f + p * ld;
+    if (tid < 32) {
+      if (p + 1 < ns) {
+        T* col = f + (p + 1) * ld;
+        const T u = p >= 0 ? col[p] : T(0);
+        T piv = col[p + 1];
+        if (p >= 0) piv -= lc[p + 1] * u;
+        if (lane == 0) check_pivot(piv, sd, s, k, K, c0 + p + 1, status, badcol);
+        const T rp = T(1) / piv;
+        __syncwarp();
+        for (int i = p + 1 + lane; i < F; i += 32) {
+          T x = col[i];
+          if (p >= 0) x -= lc[i] * u;
+          col[i] = i == p + 1 ? x : x * rp;
+        }
+      }
+    }
+    if (p >= 0 && p + 1 < F) {
+      const int m = F - p - 1, j0 = p + 1 < ns ? p + 2 : p + 1;  // rows p+1.., columns j0..
+      const int total = m * (F - j0);
+      // warp 0 comes last, after its column
+      const int first = nt > 32 ? (tid + nt - 32) % nt : tid;
+      const int qs = nt / m, rs = nt - qs * m;
+      int c = first / m, r = first - c * m;
+      const T* lp = lc + p + 1;
+      const T* up = f + p + j0 * ld;
+      T* xp = f + p + 1 + j0 * ld;
+      for (int e = first; e < total; e += 4 * nt) {
+        int at[4];
+        T x[4], l[4], u[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const bool in = e + q * nt < total;
+          at[q] = in ? r + c * ld : -1;
+          if (in) {
+            l[q] = lp[r];
+            u[q] = up[c * ld];
+            x[q] = xp[at[q]];
+          }
+          r += rs;
+          c += qs;
+          if (r >= m) {
+            r -= m;
+            ++c;
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (at[q] >= 0) xp[at[q]] = x[q] - l[q] * u[q];
       }
     }
     __syncthreads();
   }
-  T* out = fronts + (int64_t)K * sd.front_off[s] + (int64_t)k * FF;
-  for (int q = tid; q < FF; q += nt) out[q] = f[q];
 }
 
+// ---------------------------------------------------------------------------
+// Fronts in shared memory, one CTA (256 threads, or a multiple) per (front, k):
+// assembly (original entries, t_k D, the children's Schur complements), pivot-
+// free LU, write to the front storage.  f: F x front_ld(F) values.
+// ---------------------------------------------------------------------------
 template <typename T>
-__global__ void k_front_small(SymDev sd, const int32_t* __restrict__ list,
-                              const double* __restrict__ vals, const double* __restrict__ D,
-                              Shifts sh, T* __restrict__ fronts, int32_t* status,
-                              int32_t* badcol) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  front_cta<T>(sd, list[blockIdx.x], blockIdx.y, vals, D, sh, fronts, status, badcol,
-               reinterpret_cast<T*>(smraw));
-}
-
-// One (front s, perturbation k) with F <= 32 by one warp, in its F x F
-// shared-memory area f (column-major): the same assembly and the same
-// per-element sequence of operations as front_cta, with the warp's lanes as
-// rows and no block barrier.
-template <typename T>
-__device__ __forceinline__ void front_warp(const SymDev& sd, int s, int k, const double* __restrict__ vals,
-                                           const double* __restrict__ D, const Shifts& sh,
-                                           T* __restrict__ fronts, int32_t* status, int32_t* badcol, T* f) {
+__device__ __forceinline__ void front_cta(const SymDev& sd, int s, int k, const double* __restrict__ vals,
+                                          const double* __restrict__ D, const Shifts& sh,
+                                          T* __restrict__ fronts, int32_t* status, int32_t* badcol, T* f, T* rinv) {
   const int K = sh.K;
-  const int lane = threadIdx.x & 31;
-  const int ns = sd.ns[s], ms = sd.ms[s], F = ns + ms;
-  const int FF = F * F;
-  for (int q = lane; q < FF; q += 32) f[q] = T(0);
-  __syncwarp();
+  const int ns = sd.ns[s], ms = sd.ms[s], F = ns + ms, ld = front_ld(F);
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
+  for (int q = tid; q < F * ld; q += nt) f[q] = T(0);
+  __syncthreads();
+  // entries of A owned by this front (duplicates add up)
   const int64_t a0 = sd.amap_off[s], a1 = sd.amap_off[s + 1];
-  for (int64_t q = a0 + lane; q < a1; q += 32) atomicAdd(&f[sd.amap_dst[q]], (T)vals[sd.amap_src[q]]);
+  for (int64_t q = a0 + tid; q < a1; q += nt) {
+    const int d = sd.amap_dst[q];
+    atomicAdd(&f[d + d / F * (ld - F)], (T)vals[sd.amap_src[q]]);
+  }
+  // the perturbation t_k D on the pivot diagonal
   const double tk = sh.t[k];
   const int c0 = sd.c0[s];
-  for (int c = lane; c < ns; c += 32) atomicAdd(&f[c * (F + 1)], (T)(tk * D[sd.perm[c0 + c]]));
+  for (int c = tid; c < ns; c += nt) atomicAdd(&f[c * (ld + 1)], (T)(tk * D[sd.perm[c0 + c]]));
+  __syncthreads();
+  // extend-add, every warp its share of the columns
+  extend_add_flat<T>(sd, s, k, K, fronts, f, ld, (int)((int64_t)F * wid / nw), (int)((int64_t)F * (wid + 1) / nw));
+  __syncthreads();
+  if constexpr (sizeof(T) == 8) front_lu_flat<T>(f, ld, F, ns, sd, s, k, K, status, badcol);
+  else front_lu<T>(f, ld, F, ns, rinv, sd, s, k, K, status, badcol);
+  T* out = fronts + (int64_t)K * sd.front_off[s] + (int64_t)k * F * F;
+  for (int j = wid; j < F; j += nw)
+    for (int i = lane; i < F; i += 32) out[i + (int64_t)j * F] = f[i + j * ld];
+}
+
+template <typename T>
+__global__ void __launch_bounds__(512) k_front_small(SymDev sd, const int32_t* __restrict__ list,
+                                                     const double* __restrict__ vals, const double* __restrict__ D,
+                                                     Shifts sh, T* __restrict__ fronts, int32_t* status,
+                                                     int32_t* badcol) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ T rinv[16];
+  front_cta<T>(sd, list[blockIdx.x], blockIdx.y, vals, D, sh, fronts, status, badcol,
+               reinterpret_cast<T*>(smraw), rinv);
+}
+
+// ---------------------------------------------------------------------------
+// Fronts of at most 32 rows: SEG lanes (8, 16 or 32) per (front, k), lane =
+// row, the front in the segment's SEG x SEG shared-memory area f.  A child's
+// update block is added a column at a time, four in flight: the child's rows
+// land on the rows of a 32-bit mask, so lane i reads child row popcount(mask
+// below i), and the columns are the mask's bits in turn.  The elimination takes
+// four columns at a time too, all reads before the writes.  Loops are short and
+// rolled, and run to warp-uniform bounds; all lanes of a warp call together.
+// (The same in registers, unrolled to static indices, is 1500 instructions that
+// a level runs once per SM: fetching them doubled the factorisation of the 118-
+// bus grid.)
+// ---------------------------------------------------------------------------
+template <typename T, int SEG>
+__device__ __forceinline__ void front_seg(const SymDev& sd, int s, int k, bool on, int sl,
+                                          const double* __restrict__ vals, const double* __restrict__ D,
+                                          const Shifts& sh, T* __restrict__ fronts, int32_t* status,
+                                          int32_t* badcol, T* f) {
+  const int K = sh.K;
+  int ns = 0, F = 0, c0 = 0, cb = 0, ce = 0;
+  int64_t a0 = 0, a1 = 0, fo = 0;
+  if (on) {
+    ns = sd.ns[s];
+    F = ns + sd.ms[s];
+    c0 = sd.c0[s];
+    a0 = sd.amap_off[s];
+    a1 = sd.amap_off[s + 1];
+    cb = sd.child_off[s];
+    ce = sd.child_off[s + 1];
+    fo = sd.front_off[s];
+  }
+  const int Fw = __reduce_max_sync(0xffffffffu, F), nsw = __reduce_max_sync(0xffffffffu, ns);
+  for (int j = 0; j < Fw; ++j) f[sl + j * SEG] = T(0);
   __syncwarp();
-  // extend-add, child by child (each element receives its children's
-  // contributions in child order, as in the column-owner form): the lanes
-  // take the entries of the child's cms x cms update block, which land on
-  // distinct elements of this front
-  for (int ci = sd.child_off[s]; ci < sd.child_off[s + 1]; ++ci) {
-    const int c = sd.child[ci];
-    const int cns = sd.ns[c], cms = sd.ms[c], cF = cns + cms;
-    const T* cf = fronts + (int64_t)K * sd.front_off[c] + (int64_t)k * cF * cF;
-    const int32_t* em = sd.emap + sd.row_off[c];
-    const int n2 = cms * cms;
-    for (int q = lane; q < n2; q += 32) {
-      const int a = q % cms, b = q / cms;  // child update row a, column b
-      f[em[a] + em[b] * F] += cf[(cns + a) + (int64_t)(cns + b) * cF];
-    }
-    __syncwarp();
+  for (int64_t q = a0 + sl; q < a1; q += SEG) {
+    const int d = sd.amap_dst[q];
+    atomicAdd(&f[d + d / F * (SEG - F)], (T)vals[sd.amap_src[q]]);
   }
-  for (int p = 0; p < ns; ++p) {
-    const T piv = f[p * (F + 1)];
-    if (lane == 0) check_pivot(piv, sd, s, k, K, c0 + p, status, badcol);
+  if (sl < ns) atomicAdd(&f[sl * (SEG + 1)], (T)(sh.t[k] * D[sd.perm[c0 + sl]]));
+  __syncwarp();
+  // children, SEG records at a time, one a lane
+  const int most = __reduce_max_sync(0xffffffffu, ce - cb);
+  for (int b = 0; b < most; b += SEG) {
+    int64_t cfo = 0;
+    int cns = 0, cF = 0;
+    unsigned cm = 0;
+    if (cb + b + sl < ce) {
+      const ChildDesc cd = sd.cdesc[cb + b + sl];
+      cfo = cd.fo;
+      cns = cd.ns;
+      cF = cd.F;
+      cm = cd.mask;
+    }
+    const int nc = min(SEG, most - b);
+    for (int c = 0; c < nc; ++c) {
+      unsigned mask = __shfl_sync(0xffffffffu, cm, c, SEG);
+      const int eF = __shfl_sync(0xffffffffu, cF, c, SEG), ens = __shfl_sync(0xffffffffu, cns, c, SEG);
+      const int64_t efo = __shfl_sync(0xffffffffu, cfo, c, SEG);
+      const bool mine = (mask >> sl) & 1u;
+      const T* p = fronts + (int64_t)K * efo + (int64_t)k * eF * eF + ens + __popc(mask & ((1u << sl) - 1u)) +
+                   (int64_t)ens * eF;
+      const int cols = __reduce_max_sync(0xffffffffu, __popc(mask));
+      for (int e = 0; e < cols; e += 4) {
+        int j[4];
+        T v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          j[q] = mine && mask ? __ffs(mask) - 1 : -1;
+          mask &= mask - 1;
+          v[q] = j[q] >= 0 ? __ldcg(p) : T(0);
+          p += eF;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (j[q] >= 0) f[sl + j[q] * SEG] += v[q];
+      }
+    }
+  }
+  __syncwarp();
+  for (int p = 0; p < nsw; ++p) {
+    const bool act = p < ns;
+    const T piv = act ? f[p * (SEG + 1)] : T(1);
+    if (act && sl == 0) check_pivot(piv, sd, s, k, K, c0 + p, status, badcol);
     const T rp = T(1) / piv;
-    const int i = p + 1 + lane;  // this lane's row (F <= 32: one row per lane)
-    T l = T(0);
-    if (i < F) {
-      l = f[i + p * F] * rp;
-      f[i + p * F] = l;
-    }
-    for (int j = p + 1; j < F; ++j) {
-      const T u = f[p + j * F];
-      if (i < F) f[i + j * F] -= l * u;
+    const bool below = act && sl > p && sl < F;
+    const T l = below ? f[sl + p * SEG] * rp : T(0);
+    if (below) f[sl + p * SEG] = l;
+    for (int j = p + 1; j < Fw; j += 4) {
+      T u[4], x[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const bool in = below && j + q < F;
+        u[q] = in ? f[p + (j + q) * SEG] : T(0);
+        x[q] = in ? f[sl + (j + q) * SEG] : T(0);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (below && j + q < F) f[sl + (j + q) * SEG] = x[q] - l * u[q];
     }
     __syncwarp();
   }
-  T* out = fronts + (int64_t)K * sd.front_off[s] + (int64_t)k * FF;
-  for (int q = lane; q < FF; q += 32) out[q] = f[q];
+  T* out = fronts + (int64_t)K * fo + (int64_t)k * F * F + sl;
+  for (int j = 0; j < Fw; ++j)
+    if (j < F && sl < F) out[j * F] = f[sl + j * SEG];
+}
+
+template <int SEG>
+__global__ void __launch_bounds__(256) k_front_seg(SymDev sd, const int32_t* __restrict__ list, int ntasks,
+                                                   const double* __restrict__ vals, const double* __restrict__ D,
+                                                   Shifts sh, float* __restrict__ fronts, int32_t* status,
+                                                   int32_t* badcol) {
+  __shared__ float area[256 * SEG];
+  const int q = (int)((blockIdx.x * 256 + threadIdx.x) / SEG);
+  const bool on = q < ntasks;
+  const int s = on ? list[q / sh.K] : 0, k = on ? q % sh.K : 0;
+  front_seg<float, SEG>(sd, s, k, on, threadIdx.x % SEG, vals, D, sh, fronts, status, badcol,
+                        area + threadIdx.x / SEG * SEG * SEG);
 }
 
 // ---------------------------------------------------------------------------
@@ -1373,50 +1621,65 @@ __global__ void __launch_bounds__(kOwnThreads) k_front_owner(SymDev sd, const in
 // assembly forest, all K shifts and all instances of a batch.  Tasks, taken in
 // ticket order (levels bottom-up; within a level the owner tiles first, then
 // the shared-memory fronts, then the warp fronts):
-//   kFacWarp : up to 8 (front, k) pairs with F <= 32, one per warp, each in
-//              its warp's shared-memory area (front_warp);
+//   kFacSeg8/16/32: 256 / SEG (front, k) pairs with F <= SEG, one per segment
+//              of SEG lanes (front_seg);
 //   kFacCta  : one (front, k) pair of a front that fits in shared memory
 //              (front_cta);
 //   kFacOwner: one owner tile of a wider front (owner_tile).
-// Before its assembly a task waits until every child's completion counter
-// for its k, fdone[child * K + k], has reached need[child] (1 for warp and
-// shared-memory fronts, the number of tiles for an owner front); a finished
-// task adds 1 to its own counter after its writes are visible.  Every wait is
+// Before its assembly a task waits until its front's counter for its k,
+// fdone[s * K + k], has reached need[s], the tasks of its children (one each for
+// segment and shared-memory fronts, the tiles of an owner front); a finished task
+// adds 1 to its parent's counter after its writes are visible.  Every wait is
 // on a task with a smaller ticket (a child, or an earlier tile of the same
 // front), which a running CTA already holds, so the schedule cannot deadlock
 // whatever the residency, and every wait is bounded.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void fac_wait_children(const SymDev& sd, const int* fdone, const int* need, int s,
-                                                  int k, int K, int idx, int n, int* err, int64_t polls) {
-  const int cb = sd.child_off[s], ce = sd.child_off[s + 1];
-  for (int ci = cb + idx; ci < ce; ci += n) {
-    const int c = sd.child[ci];
-    const int* f = fdone + (int64_t)c * K + k;
-    const int want = need[c];
+                                                  int k, int K, int* err, int64_t polls) {
+  const int want = need[s];
+  if (want == 0) return;
+  const int* f = fdone + ((int64_t)s * K + k) * kCtrStride;
+  if (dag_ld_acquire(f) >= want) return;
+  // the polls in between are relaxed: an acquiring one drops the SM's L1 lines
+  // under the CTA beside it
+  unsigned ns = 32;
+  for (int64_t i = 0; i < polls; ++i) {
+    __nanosleep(ns);
     int v;
     asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
-    if (v >= want) continue;
-    int64_t i = 0;
-    for (; i < polls; ++i) {
-      __nanosleep(64);
-      asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
-      if (v >= want) break;
-    }
-    if (i == polls) atomicExch(err, 1);
+    if (v >= want) break;
+    ns += ns < 1024 ? ns >> 3 : 0;
   }
-  asm volatile("fence.acq_rel.gpu;" ::: "memory");
+  if (dag_ld_acquire(f) < want) atomicExch(err, 1);
 }
 
-__device__ __forceinline__ void fac_publish(int* fdone, int s, int k, int K) {
-  __threadfence();
-  asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(fdone + (int64_t)s * K + k) : "memory");
+__device__ __forceinline__ void fac_publish(const SymDev& sd, int* fdone, int s, int k, int K) {
+  const int p = sd.parent[s];
+  if (p >= 0)
+    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(fdone + ((int64_t)p * K + k) * kCtrStride) : "memory");
+}
+
+template <typename T, int SEG>
+__device__ __forceinline__ void fac_segments(const SymDev& sd, const FactorTask& t, const int* need, int* fdone,
+                                             int* err, int64_t polls, const int32_t* __restrict__ wlist,
+                                             const double* __restrict__ vals, const double* __restrict__ D,
+                                             const Shifts& sh, T* __restrict__ fronts, int32_t* status,
+                                             int32_t* badcol, T* sm) {
+  const int q = t.q + (int)threadIdx.x / SEG, sl = threadIdx.x % SEG;
+  const bool on = q < t.j;
+  const int s = on ? wlist[t.s + q / sh.K] : 0, k = on ? q % sh.K : 0;
+  if (on && sl == 0) fac_wait_children(sd, fdone, need, s, k, sh.K, err, polls);
+  __syncwarp();
+  front_seg<T, SEG>(sd, s, k, on, sl, vals, D, sh, fronts, status, badcol, sm + threadIdx.x / SEG * SEG * SEG);
+  __syncwarp();
+  if (on && sl == 0) fac_publish(sd, fdone, s, k, sh.K);
 }
 
 template <typename T, bool TC, int MINB>
 __global__ void __launch_bounds__(kOwnThreads, MINB)
 k_factor_persistent(SymDev sd, const FactorTask* __restrict__ tasks, int ntasks, int* ticket, int* fdone,
                     const int* __restrict__ need, int* flags, int* err, const int32_t* __restrict__ wlist,
-                    const double* __restrict__ vals, const double* __restrict__ D, Shifts sh,
+                    const double* __restrict__ vals, const double* __restrict__ D, const __grid_constant__ Shifts sh,
                     T* __restrict__ fronts, int32_t* status, int32_t* badcol, int CH, int64_t polls,
                     size_t tc_off) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -1429,8 +1692,7 @@ k_factor_persistent(SymDev sd, const FactorTask* __restrict__ tasks, int ntasks,
   TcCtx tc{TC ? 1 : 0, tcs, tcs + 2 * 128 * 32, 0, 0, 0};
   if constexpr (TC) tc_setup(tc, &s_taddr, &s_mbar);
   const int K = sh.K;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int lane = tid & 31, wid = tid >> 5;
+  const int tid = threadIdx.x;
   for (;;) {
     __syncthreads();  // the previous task is done with shared memory and s_t
     if (tid == 0) s_t = atomicAdd(ticket, 1);
@@ -1438,26 +1700,22 @@ k_factor_persistent(SymDev sd, const FactorTask* __restrict__ tasks, int ntasks,
     const int u = s_t;
     if (u >= ntasks) break;
     const FactorTask t = tasks[u];
-    if (t.kind == kFacWarp) {
-      const int q = t.q + wid;
-      if (q < t.j) {
-        const int s = wlist[t.s + q / K], k = q % K;
-        fac_wait_children(sd, fdone, need, s, k, K, lane, 32, err, polls);
-        __syncwarp();
-        front_warp<T>(sd, s, k, vals, D, sh, fronts, status, badcol, sm + wid * 32 * 32);
-        __syncwarp();
-        if (lane == 0) fac_publish(fdone, s, k, K);
-      }
+    if (t.kind == kFacSeg8) {
+      fac_segments<T, 8>(sd, t, need, fdone, err, polls, wlist, vals, D, sh, fronts, status, badcol, sm);
+    } else if (t.kind == kFacSeg16) {
+      fac_segments<T, 16>(sd, t, need, fdone, err, polls, wlist, vals, D, sh, fronts, status, badcol, sm);
+    } else if (t.kind == kFacSeg32) {
+      fac_segments<T, 32>(sd, t, need, fdone, err, polls, wlist, vals, D, sh, fronts, status, badcol, sm);
     } else {
-      fac_wait_children(sd, fdone, need, t.s, t.k, K, tid, nt, err, polls);
+      if (tid == 0) fac_wait_children(sd, fdone, need, t.s, t.k, K, err, polls);
       __syncthreads();
       if (t.kind == kFacCta)
-        front_cta<T>(sd, t.s, t.k, vals, D, sh, fronts, status, badcol, sm);
+        front_cta<T>(sd, t.s, t.k, vals, D, sh, fronts, status, badcol, sm, rinv);
       else
         owner_tile<T, TC>(sd, t.s, t.k, t.j, t.q, flags + t.flags, CH, err, vals, D, sh, fronts, status,
                           badcol, sm, sm + 32 * 32, sm + 32 * 32 + 32 * 33, rinv, tc);
       __syncthreads();
-      if (tid == 0) fac_publish(fdone, t.s, t.k, K);
+      if (tid == 0) fac_publish(sd, fdone, t.s, t.k, K);
     }
   }
   if constexpr (TC) tc_teardown(tc);
@@ -1541,14 +1799,6 @@ int owner_impl(const SymDev& sd, const LevelPlan& lp, const int32_t* d_big, cons
 }
 
 template <typename T>
-int small_threads(int maxF) {
-  if (maxF <= 16) return 64;
-  if (maxF <= 32) return 128;
-  if (maxF <= 96) return 256;
-  return 512;
-}
-
-template <typename T>
 void set_smem_attrs() {
   static std::atomic<bool> done_dev[kMaxDevices];
   const int dev = current_device();
@@ -1599,9 +1849,26 @@ int factor_small_group(const SymDev& sd, const LevelPlan& lp, int g, const int32
     const auto& G = lp.groups[g];
     if (G.count == 0) return 0;
     if (G.cluster == 0) {
-      const size_t smem = (size_t)G.maxF * G.maxF * sizeof(T);
-      k_front_small<T><<<dim3(G.count, K), small_threads<T>(G.maxF), smem, st>>>(
-          sd, d_small + G.off, vals, D, sh, fr, status, badcol);
+      const int32_t* lst = d_small + G.off;
+      bool seg_class = false;
+      // FP64 takes a CTA for the narrowest fronts too: its threads are dealt the
+      // elements, where rows as lanes leave some idle (118 buses 114 us against
+      // 136 with segments, 300 buses 168 against 185)
+      if constexpr (sizeof(T) == 4) {
+        const int n = G.count * K;
+        auto seg = [&](auto S) {
+          constexpr int SEG = decltype(S)::value, per = 256 / SEG;
+          k_front_seg<SEG><<<(n + per - 1) / per, 256, 0, st>>>(sd, lst, n, vals, D, sh, fr, status, badcol);
+        };
+        seg_class = G.maxF <= 32;
+        if (G.maxF <= 8) seg(std::integral_constant<int, 8>{});
+        else if (G.maxF <= 16) seg(std::integral_constant<int, 16>{});
+        else if (G.maxF <= 32) seg(std::integral_constant<int, 32>{});
+      }
+      if (!seg_class)
+        k_front_small<T><<<dim3(G.count, K), G.maxF <= 32 ? 128 : (G.maxF <= 96 ? 256 : 512),
+                           (size_t)G.maxF * front_ld(G.maxF) * sizeof(T), st>>>(sd, lst, vals, D, sh, fr, status,
+                                                                               badcol);
     } else {
       const int C = G.cluster;
       cudaLaunchConfig_t cfg = {};
@@ -1803,10 +2070,10 @@ int persistent_cta_front_limit(int precision) { return precision == PISP_FP32 ? 
 
 size_t factor_persistent_smem(int precision, int CH, bool has_owner, int maxCtaF) {
   const size_t es = precision == PISP_FP32 ? 4 : 8;
-  size_t e = (size_t)(kOwnThreads / 32) * 32 * 32;                          // warp fronts
-  e = std::max(e, (size_t)maxCtaF * maxCtaF);                                // shared-memory fronts
+  size_t e = (size_t)(kOwnThreads / 32) * 32 * 32;                          // segments
+  e = std::max(e, (size_t)maxCtaF * front_ld(maxCtaF));                      // shared-memory fronts
   if (has_owner) e = std::max(e, (size_t)(CH + 1) * 32 + 32 * 32 + 32 * 33);  // owner tiles
-  return e * es;
+  return (e * es + 127) / 128 * 128;  // what follows it (the tensor-core staging) stays aligned
 }
 
 int launch_factor_persistent(int precision, const SymDev& sd, const FactorTask* tasks, int ntasks, int* ticket,

@@ -19,6 +19,17 @@ inline int current_device() {
   return d;
 }
 
+constexpr int kCtrStride = 8;  // ints between completion counters: a 32-byte sector each
+
+// A child as its parent's assembly needs it; mask (parents of at most 32 rows):
+// the parent's rows that its update rows land on.
+struct alignas(16) ChildDesc {
+  int64_t fo;  // front_off
+  int32_t ns, F;
+  uint32_t mask;
+  int32_t pad[3];
+};
+
 // Device view of the symbolic structure (all arrays live on the device).
 struct SymDev {
   const int32_t* c0;         // [S] first permuted column of each supernode
@@ -30,6 +41,7 @@ struct SymDev {
   const int64_t* row_off;    // [S] offset into rows/emap
   const int32_t* child_off;  // [S+1]
   const int32_t* child;      // children, ascending
+  const ChildDesc* cdesc;    // [S] their records, in the same order
   const int64_t* amap_off;   // [S+1]
   const int32_t* amap_src;   // A value index
   const int32_t* amap_dst;   // position i + j*F in the front
@@ -73,7 +85,7 @@ struct LevelPlan {
     int32_t maxF;     // largest front in the group
     int32_t cluster;  // 0: one CTA per (front, k); C > 0: clusters of C CTAs
   };
-  Group groups[8];
+  Group groups[9];  // up to 8, 16, 32, 64 rows; clusters of 1, 2, 4, 8; the rest
   int32_t n_groups = 0;
   // big fronts (blocked factorisation in global memory)
   int64_t big_off = 0;
@@ -114,14 +126,14 @@ struct DagTask {
 };
 
 // Tasks of the one-launch factorisation (factor policy 4), all levels:
-//   kFacWarp : s = offset of a group in the warp-front list, q = first task,
-//              j = tasks in the group; task i is (front list[s + i / K],
-//              k = i % K), 8 tasks (one per warp) per record;
+//   kFacSeg8/16/32: s = offset of a group in the list of fronts of at most
+//              32 rows, q = first task, j = tasks in the group; task i is (front
+//              list[s + i / K], k = i % K), 256 / SEG tasks per record;
 //   kFacCta  : front s, perturbation k, factored in shared memory;
 //   kFacOwner: owner tile (column block j, row chunk q) of front s,
 //              perturbation k; flags = offset of the (front, k) pair's
 //              release flags.
-enum FactorKind { kFacWarp = 0, kFacCta = 1, kFacOwner = 2 };
+enum FactorKind { kFacSeg8 = 0, kFacSeg16 = 1, kFacSeg32 = 2, kFacCta = 3, kFacOwner = 4 };
 struct FactorTask {
   int32_t kind, s, k, q, j, flags;
 };
@@ -162,8 +174,8 @@ int launch_factor_big_dag(int precision, const SymDev& sd, const LevelPlan& lp, 
                           const double* vals, const double* D, const Shifts& sh, void* fronts,
                           int32_t* status, int32_t* badcol, int tc, cudaStream_t st);
 // The whole factorisation in one persistent launch (factor policy 4): ticket
-// (1 int), fdone (S*K ints) and flags must be zero; need[s] = 1 for warp and
-// shared-memory fronts, tiles per (front, k) for owner fronts.
+// (1 int), fdone (S*K counters, kCtrStride apart) and flags must be zero; need[s]
+// = the tasks of the children of s (per k).
 int launch_factor_persistent(int precision, const SymDev& sd, const FactorTask* tasks, int ntasks, int* ticket,
                              int* fdone, const int* need, int* flags, int* err, const int32_t* wlist,
                              const double* vals, const double* D, const Shifts& sh, void* fronts,
@@ -220,8 +232,6 @@ struct alignas(16) FrontDesc {
   int32_t flag;   // more than 32 pivots: first of its counters in `wide`
   int32_t whole;  // FrontWhole: counted at group 0 only
 };
-
-constexpr int kCtrStride = 8;  // ints between completion counters: a 32-byte sector each
 
 constexpr int kSolveChunk = 8;  // right-hand sides of a segment task, where there are several
 
