@@ -261,10 +261,10 @@ int factor_path(const pisp_handle* h, int F, int precision) {
 // saves the launches and the waits between levels and size classes: 1354 buses
 // 344 / 245, 777 buses 230 / 191, 5 grids 280 / 192, 64 grids 1784 / 897; with a
 // root of 1596 rows the owner tiles are all that counts, and those alone on an SM
-// with 255 registers a thread are ahead (10000 buses 3124 / 3272).  In FP64 one
-// grid's fronts are bound by the FP64 pipe whichever way they are launched, and
-// CTAs for all of them are ahead of segments (300 buses 160 / 168, 1354 buses
-// 703 / 725); many grids' fronts fill the SMs (48 grids 3939 / 2470).
+// with 255 registers a thread are ahead (10000 buses 2635 / 2999).  In FP64 one
+// grid's fronts are bound by the FP64 pipe whichever way they are launched (118
+// buses 110 / 129, 300 buses 164 / 164, 1354 buses 573 / 567); many grids' fronts
+// fill the SMs (48 grids 3939 / 2470).
 bool one_launch(const pisp_handle* h, int precision, int32_t K) {
   if (h->factor_policy != 0) return h->factor_policy == 4;
   const int64_t tasks = (int64_t)h->sym.sn.size() * K;
@@ -281,11 +281,11 @@ int build_persistent_factor(pisp_handle* h, int precision, int32_t K) {
   int smem_maxF = h->factor_smem_maxF;
   h->fac_ctas = h->factor_ctas;
   if (h->factor_policy == 0) {
-    // many FP32 fronts: three CTAs an SM with the fronts that three can hold
-    // (64 grids 897 us, 993 with two); few: two, the registers are worth more
-    // (2000 buses 334 us, 372 with three)
-    const bool three = precision == PISP_FP32 && (int64_t)S.sn.size() * K >= kManyTasks;
-    smem_maxF = three ? 128 : 0;
+    // many fronts: three CTAs an SM with the fronts that three can hold (64 grids
+    // 871 us, 994 with two; 48 grids in FP64 1914, 2173 with two); few: two, the
+    // registers are worth more (2000 buses 341 us, 364 with three)
+    const bool three = (int64_t)S.sn.size() * K >= kManyTasks;
+    smem_maxF = three ? (precision == PISP_FP32 ? 128 : 64) : 0;
     h->fac_ctas = three ? 3 : 2;
   }
   const int Fc = smem_maxF > 0 ? std::min(smem_maxF, pisp::persistent_cta_front_limit(precision))

@@ -108,11 +108,13 @@ __device__ __forceinline__ void panel_eliminate(T* P, int ld, int Mr, int nb, co
 }
 
 // Children's update columns added into the destination columns [d0, d0 + w)
-// and rows [R0, R1) of front s, stored at dst[(row - R0) + (col - d0) * ld].  Each destination column
-// belongs to one warp (col - d0 = warp, warp + warps, ...), which walks the
-// column's inverse extend-add list in child order: every element receives its
-// contributions in child order, with no barrier between children, and a
-// group of 8 x 32 child rows is loaded before any of them is added.
+// and rows [R0, R1) of front s, stored at dst[(row - R0) + (col - d0) * ld].  Each
+// destination column belongs to one warp (col - d0 = warp, warp + warps, ...),
+// which walks the column's inverse extend-add list in child order: every element
+// receives its contributions in child order, with no barrier between children,
+// and a group of 8 x 32 child rows is loaded before any of them is added.  Owner
+// tiles keep this form: their columns are tall, and the flat form below is no
+// faster there (10000 buses 2401 us of tiles against 2424).
 template <typename T>
 __device__ __forceinline__ void extend_add_columns(const SymDev& sd, int s, int k, int K,
                                                    const T* __restrict__ fronts, T* dst, int ld,
@@ -161,15 +163,41 @@ __device__ __forceinline__ void extend_add_columns(const SymDev& sd, int s, int 
   }
 }
 
+// The CTA: entries [e0, e1) of the assembly map, EB at a time per thread, so that
+// the two dependent reads of an entry are paid once for EB of them (a 486-row
+// dense front's tiles spent 33 us each on them one by one).
+template <typename T, typename Put>
+__device__ __forceinline__ void add_entries(const SymDev& sd, const double* __restrict__ vals, int64_t e0, int64_t e1,
+                                            Put put) {
+  constexpr int EB = 8;
+  const int nt = blockDim.x;
+  for (int64_t e = e0 + threadIdx.x; e < e1; e += (int64_t)EB * nt) {
+    int d[EB], at[EB];
+    double v[EB];
+#pragma unroll
+    for (int q = 0; q < EB; ++q) {
+      const bool in = e + q * nt < e1;
+      d[q] = in ? sd.amap_dst[e + q * nt] : -1;
+      at[q] = in ? sd.amap_src[e + q * nt] : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < EB; ++q) v[q] = d[q] >= 0 ? vals[at[q]] : 0.0;
+#pragma unroll
+    for (int q = 0; q < EB; ++q)
+      if (d[q] >= 0) put(d[q], (T)v[q]);
+  }
+}
+
 // One warp: the children's update blocks added into the destination columns
-// [d0, d1) of front s, all its rows, stored at dst[row + col * ld].  The columns'
+// [d0, d1) of front s, rows [R0, R1), stored at dst[row + col * ld] (dst is
+// where row 0 of column 0 would be).  The columns'
 // entries of the inverse extend-add map are consecutive; 32 are resolved at a
 // time, one a lane, and four child columns are in flight at a time (two rows a
 // lane), so that a memory latency covers four contributions and not one.  The
 // additions to an element follow a fixed order.
 template <typename T>
 __device__ __forceinline__ void extend_add_flat(const SymDev& sd, int s, int k, int K, const T* __restrict__ fronts,
-                                                T* dst, int ld, int d0, int d1) {
+                                                T* dst, int ld, int d0, int d1, int R0, int R1) {
   constexpr int NE = 4;
   const int lane = threadIdx.x & 31;
   const int64_t vo = sd.vec_off[s];
@@ -210,8 +238,8 @@ __device__ __forceinline__ void extend_add_flat(const SymDev& sd, int s, int k, 
         }
 #pragma unroll
         for (int q = 0; q < NE; ++q) {
-          if (r0[q] >= 0) dst[r0[q] + d[q]] += v0[q];
-          if (r1[q] >= 0) dst[r1[q] + d[q]] += v1[q];
+          if (r0[q] >= R0 && r0[q] < R1) dst[r0[q] + d[q]] += v0[q];
+          if (r1[q] >= R0 && r1[q] < R1) dst[r1[q] + d[q]] += v1[q];
           __syncwarp();  // the next contribution may land on another lane's element
         }
       }
@@ -391,17 +419,14 @@ __device__ __forceinline__ void front_cta(const SymDev& sd, int s, int k, const 
   __syncthreads();
   // entries of A owned by this front (duplicates add up)
   const int64_t a0 = sd.amap_off[s], a1 = sd.amap_off[s + 1];
-  for (int64_t q = a0 + tid; q < a1; q += nt) {
-    const int d = sd.amap_dst[q];
-    atomicAdd(&f[d + d / F * (ld - F)], (T)vals[sd.amap_src[q]]);
-  }
+  add_entries<T>(sd, vals, a0, a1, [&](int d, T v) { atomicAdd(&f[d + d / F * (ld - F)], v); });
   // the perturbation t_k D on the pivot diagonal
   const double tk = sh.t[k];
   const int c0 = sd.c0[s];
   for (int c = tid; c < ns; c += nt) atomicAdd(&f[c * (ld + 1)], (T)(tk * D[sd.perm[c0 + c]]));
   __syncthreads();
   // extend-add, every warp its share of the columns
-  extend_add_flat<T>(sd, s, k, K, fronts, f, ld, (int)((int64_t)F * wid / nw), (int)((int64_t)F * (wid + 1) / nw));
+  extend_add_flat<T>(sd, s, k, K, fronts, f, ld, (int)((int64_t)F * wid / nw), (int)((int64_t)F * (wid + 1) / nw), 0, F);
   __syncthreads();
   if constexpr (sizeof(T) == 8) front_lu_flat<T>(f, ld, F, ns, sd, s, k, K, status, badcol);
   else front_lu<T>(f, ld, F, ns, rinv, sd, s, k, K, status, badcol);
@@ -1088,13 +1113,11 @@ int big_dag_impl(const SymDev& sd, const LevelPlan& lp, const int32_t* d_big, co
 //      those U rows and for its own chunk's rows of L21(p), then subtracts
 //      L21(p) U(p, j) from its rows;
 //   3. if the block holds pivots: the tile holding the diagonal block factors
-//      it in shared memory (two pivots per barrier), eliminates its rows below
+//      it in shared memory, eliminates its rows below
 //      it and releases them; the tiles of the chunks below wait for that,
 //      then eliminate their rows with the released U rows and reciprocal
 //      pivots.  Tiles are written to the front storage before their release
 //      flags (st.release.gpu) are set.
-// Every phase runs on all 8 warps with short loop bodies: straight-line code
-// run by a single warp is fetched cold and stalls on instruction fetch.
 // The same per-element sequence of multiply-adds as panel_eliminate is used
 // for the panel, so the pivot block and L21 match the per-panel path.
 // Tasks are taken in ticket order from a list sorted by (block, chunk):
@@ -1134,40 +1157,74 @@ __device__ __forceinline__ void own_trsm(T* Bk, int ld, int r0, int nb, int w, c
   }
 }
 
-// rows [i0, i1) of the tile (stored from row R0): x(i, :) -= L(i, r0..r0+nb-1) U,
-// L read from the front storage (written before its release) straight into
-// registers, U from Us; a work item is one row and 16 columns.
-template <typename T>
-__device__ __forceinline__ void own_update_rows(T* Bt, int ld, int R0, const T* f, int F, int r0, int nb,
-                                                const T* Us, int i0, int i1, int w) {
-  const int m = i1 - i0;
-  for (int q = threadIdx.x; q < 2 * m; q += blockDim.x) {
-    const int g = q >= m ? 1 : 0;
-    const int i = i0 + q - g * m;
-    const int cb = 16 * g;
-    if (cb >= w) continue;
-    T l[32];
+// rows [i0, i1) of an FP64 tile: x(i, :) -= L(i, r0..r0+nb-1) U, L from the front
+// storage, U from Us; lane = row, four columns a warp.
+// A warp has a quarter of the SM's FP64 pipe at most, so all eight take part (two
+// warps of 16 columns took 18 us a panel).
+__device__ __forceinline__ void own_update_few64(double* Bt, int ld, int R0, const double* f, int F, int r0, int nb,
+                                                 const double* Us, int i0, int i1, int w) {
+  const int cb = 4 * (threadIdx.x >> 5);
+  if (cb >= w) return;
+  for (int i = i0 + (threadIdx.x & 31); i < i1; i += 32) {
+    double l[32];
 #pragma unroll
-    for (int c = 0; c < 32; ++c) l[c] = (c < nb) ? __ldcg(f + i + (int64_t)(r0 + c) * F) : T(0);
-    T* row = Bt + (i - R0);
-    T x[16];
+    for (int c = 0; c < 32; ++c) l[c] = c < nb ? __ldcg(f + i + (int64_t)(r0 + c) * F) : 0.0;
+    double* row = Bt + (i - R0) + cb * ld;
+    double x[4];
 #pragma unroll
-    for (int col = 0; col < 16; ++col) x[col] = row[(cb + col) * ld];
+    for (int c = 0; c < 4; ++c) x[c] = row[c * ld];
 #pragma unroll
-    for (int cg = 0; cg < 32; cg += 8) {
-      if (cg < nb) {
+    for (int c = 0; c < 32; ++c)
+      if (c < nb) {
 #pragma unroll
-        for (int c = cg; c < cg + 8; ++c) {
-          const T* ur = Us + c * 32 + cb;
-#pragma unroll
-          for (int col = 0; col < 16; ++col) x[col] -= l[c] * ur[col];
-        }
+        for (int g = 0; g < 4; ++g) x[g] -= l[c] * Us[c * 32 + cb + g];
       }
-    }
 #pragma unroll
-    for (int col = 0; col < 16; ++col)
-      if (cb + col < w) row[(cb + col) * ld] = x[col];
+    for (int c = 0; c < 4; ++c)
+      if (cb + c < w) row[c * ld] = x[c];
   }
+}
+
+// own_eliminate_rows in FP64: the whole CTA takes one pivot column at a time, the
+// elements dealt out one by one (a row a thread, 32 rows were one warp's work, a
+// quarter of the pipe: 19 us)
+__device__ __forceinline__ void own_eliminate_flat(double* Bt, int ld, int R0, int i0, int i1, int np, int w,
+                                                   const double* Us, const double* rinv) {
+  const int m = i1 - i0;
+  if (m <= 0) return;
+  double* t = Bt + (i0 - R0);
+  for (int c = -1; c < np; ++c) {
+    // column c is scaled; its update of the others, and column c + 1 scaled
+    const int j0 = c + 1 < np ? c + 1 : w, n = c >= 0 ? w - c - 1 : 1;
+    const int total = c >= 0 ? m * n : m;
+    for (int e = threadIdx.x; e < total; e += blockDim.x) {
+      const int g = e / m, r = e - g * m, j = c + 1 + g;
+      double x = t[r + j * ld];
+      if (c >= 0) x -= t[r + c * ld] * Us[c * 32 + j];
+      if (j == j0) x *= rinv[j];
+      t[r + j * ld] = x;
+    }
+    __syncthreads();
+  }
+}
+
+// own_trsm in FP64: the warp's four columns stay in the tile and a step's
+// elements, rows below q of the four, are dealt out to the lanes one by one: an
+// FP64 instruction takes its 16 clocks whether its lanes are needed or not.
+__device__ __forceinline__ void own_trsm_flat(double* Bk, int ld, int nb, int w, const double* Ls, double* Us) {
+  const int lane = threadIdx.x & 31, cb = (threadIdx.x >> 5) * 4, wc = min(4, w - cb);
+  for (int q = 0; q + 1 < nb; ++q) {
+    const int m = nb - 1 - q;
+    for (int e = lane; e < m * wc; e += 32) {
+      const int c = e / m, r = q + 1 + e - c * m;
+      double* col = Bk + (cb + c) * ld;
+      col[r] -= Ls[r * 33 + q] * col[q];
+    }
+    __syncwarp();
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    Us[lane * 32 + cb + i] = lane < nb && cb + i < w ? Bk[lane + (cb + i) * ld] : 0.0;
 }
 
 // pivot-free LU of the np x w diagonal block D (rows = the block's pivots) in
@@ -1255,6 +1312,50 @@ __device__ __forceinline__ void own_factor_diag(T* D, int ld, int np, int w, T* 
       if (lane < r) D[r + lane * ld] = v * rinv[lane];
     }
     Us[r * 32 + lane] = (r < np && lane < w && lane >= r) ? v : T(0);
+  }
+}
+
+// The same in FP64: one pivot at a time with one barrier each, the trailing
+// elements dealt out to warps 1 to 7 one by one.  Warp 0 takes the next pivot's
+// column: its update, the one reciprocal, the scaled column.  (Every warp
+// dividing twice a barrier kept the FP64 pipe, 16 clocks an instruction, busy for
+// most of a block's 75 us.)  The operations on an element are the same.
+__device__ __forceinline__ void own_factor_diag_flat(double* D, int ld, int np, int w, double* Us, double* rinv,
+                                                     const SymDev& sd, int s, int k, int K, int colbase,
+                                                     int32_t* status, int32_t* badcol) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  for (int p = -1; p < np; ++p) {
+    const double* lc = D + p * ld;
+    if (tid < 32) {
+      if (p + 1 < np) {
+        double* col = D + (p + 1) * ld;
+        const double u = p >= 0 ? col[p] : 0.0;
+        double piv = col[p + 1];
+        if (p >= 0) piv -= lc[p + 1] * u;
+        if (lane == 0) check_pivot(piv, sd, s, k, K, colbase + p + 1, status, badcol);
+        const double rp = 1.0 / piv;
+        if (lane == 0) rinv[p + 1] = rp;
+        __syncwarp();
+        const int i = p + 1 + lane;
+        if (i < np) {
+          double x = col[i];
+          if (p >= 0) x -= lc[i] * u;
+          col[i] = i == p + 1 ? x : x * rp;
+        }
+      }
+    } else if (p >= 0) {
+      const int m = np - p - 1, j0 = p + 1 < np ? p + 2 : p + 1, total = m * (w - j0);
+      for (int e = tid - 32; e < total; e += blockDim.x - 32) {
+        const int c = e / m, r = e - c * m;
+        double* x = D + (p + 1 + r) + (j0 + c) * ld;
+        *x -= lc[p + 1 + r] * D[p + (j0 + c) * ld];
+      }
+    }
+    __syncthreads();
+  }
+  for (int e = tid; e < 32 * 32; e += blockDim.x) {
+    const int r = e >> 5, c = e & 31;
+    Us[e] = (r < np && c < w && c >= r) ? D[r + c * ld] : 0.0;
   }
 }
 
@@ -1444,11 +1545,258 @@ __device__ __noinline__ void tc_update_rows(float* Bt, int ld, int R0, const flo
   }
 }
 
+// ---------------------------------------------------------------------------
+// FP32 owner tiles on the FP32 pipe.  A tile's rows are worked through in chunks
+// of kOwnChunk, and a panel's flag counts what is final of it: 1 = the pivot
+// rows, 2 + c = also the rows of chunks 0 .. c, kOwnDone = all.  A tile follows
+// the panel before it chunk by chunk, so a panel costs the chain of panels one
+// chunk and the pivot block, not two passes over the column (10000 buses, 1596
+// rows: xx ms of owner tiles, 2.95 before).  U rows are read four values a time,
+// which both of a thread's rows use: read one by one, shared memory took four
+// times as long as the multiply-adds.
+// ---------------------------------------------------------------------------
+constexpr int kOwnChunk = 256;
+constexpr int kOwnDone = 1 << 20;
+
+// waits as dag_wait; returns the value seen
+__device__ __forceinline__ int own_wait(const int* f, int need, int* err) {
+  int v = dag_ld_acquire(f);
+  for (int64_t i = 0; v < need && i < kDagWaitPolls; ++i) {
+    __nanosleep(64);
+    v = dag_ld_acquire(f);
+  }
+  if (v < need) {
+    atomicExch(err, 1);
+    v = need;
+  }
+  return v;
+}
+
+// rows [i0, i1) of the tile: x(i, :) -= L(i, r0..r0+nb-1) U.  A thread takes NR
+// rows, 128 apart, and 16 columns; L comes from the front storage CB columns
+// ahead of their use.
+template <int NR, int CB>
+__device__ __forceinline__ void own_update_rows_of(float* Bt, int ld, int R0, const float* f, int F, int r0, int nb,
+                                                 const float* Us, int i0, int i1, int w) {
+  const int cb = 16 * (threadIdx.x >> 7), pr = threadIdx.x & 127;
+  if (cb >= w) return;
+  const float* lp = f + (int64_t)r0 * F;
+  float l[2][NR][CB];
+  auto fetch = [&](float (&d)[NR][CB], int i, int c0) {
+#pragma unroll
+    for (int h = 0; h < NR; ++h)
+#pragma unroll
+      for (int c = 0; c < CB; ++c)
+        d[h][c] = i + 128 * h < i1 && c0 + c < nb ? __ldcg(lp + i + 128 * h + (int64_t)(c0 + c) * F) : 0.f;
+  };
+  fetch(l[0], i0 + pr, 0);
+  for (int i = i0 + pr; i < i1; i += 128 * NR) {
+    float* row = Bt + (i - R0) + cb * ld;
+    float x[NR][16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+#pragma unroll
+      for (int h = 0; h < NR; ++h) x[h][c] = i + 128 * h < i1 ? row[c * ld + 128 * h] : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < 32 / CB; ++q) {
+      if (q + 1 < 32 / CB) fetch(l[(q + 1) & 1], i, CB * q + CB);
+      else fetch(l[0], i + 128 * NR, 0);
+      if (CB * q < nb) {
+#pragma unroll
+        for (int c = 0; c < CB; ++c) {
+          const float4* u = reinterpret_cast<const float4*>(Us + (CB * q + c) * 32 + cb);
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            const float4 v = u[g];
+#pragma unroll
+            for (int h = 0; h < NR; ++h) {
+              x[h][4 * g] -= l[q & 1][h][c] * v.x;
+              x[h][4 * g + 1] -= l[q & 1][h][c] * v.y;
+              x[h][4 * g + 2] -= l[q & 1][h][c] * v.z;
+              x[h][4 * g + 3] -= l[q & 1][h][c] * v.w;
+            }
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+#pragma unroll
+      for (int h = 0; h < NR; ++h)
+        if (i + 128 * h < i1) row[c * ld + 128 * h] = x[h][c];
+    }
+  }
+}
+
+// by the registers of the kernel: 255 for the tiles alone, 128 or 80 in the one-launch form
+template <int REGS>
+__device__ __forceinline__ void own_update_pairs(float* Bt, int ld, int R0, const float* f, int F, int r0, int nb,
+                                                 const float* Us, int i0, int i1, int w) {
+  own_update_rows_of<(REGS >= 128 ? 2 : 1), (REGS >= 255 ? 16 : 8)>(Bt, ld, R0, f, F, r0, nb, Us, i0, i1, w);
+}
+
+// the same for at most 32 rows: lane = row, four columns a warp (8 warps)
+__device__ __forceinline__ void own_update_few(float* Bt, int ld, int R0, const float* f, int F, int r0, int nb,
+                                               const float* Us, int i0, int i1, int w) {
+  const int i = i0 + (threadIdx.x & 31), cb = 4 * (threadIdx.x >> 5);
+  if (i >= i1 || cb >= w) return;
+  float l[32];
+#pragma unroll
+  for (int c = 0; c < 32; ++c) l[c] = c < nb ? __ldcg(f + i + (int64_t)(r0 + c) * F) : 0.f;
+  float* row = Bt + (i - R0) + cb * ld;
+  float x[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) x[c] = row[c * ld];
+#pragma unroll
+  for (int c = 0; c < 32; ++c) {
+    const float4 v = *reinterpret_cast<const float4*>(Us + c * 32 + cb);
+    x[0] -= l[c] * v.x;
+    x[1] -= l[c] * v.y;
+    x[2] -= l[c] * v.z;
+    x[3] -= l[c] * v.w;
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) row[c * ld] = x[c];
+}
+
+// own_eliminate_rows with the U rows read four at a time
+__device__ __forceinline__ void own_eliminate_quads(float* Bt, int ld, int R0, int i0, int i1, int np,
+                                                    const float* Us, const float* rinv) {
+  for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+    float* row = Bt + (i - R0);
+    float x[32];
+#pragma unroll
+    for (int c = 0; c < 32; ++c) x[c] = row[c * ld];
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      if (c < np) {
+        const float l = x[c] * rinv[c];
+        x[c] = l;
+#pragma unroll
+        for (int g = (c + 1) / 4; g < 8; ++g) {
+          const float4 v = *reinterpret_cast<const float4*>(Us + c * 32 + 4 * g);
+          const float u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (4 * g + e > c) x[4 * g + e] -= l * u[e];
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 32; ++c) row[c * ld] = x[c];
+  }
+}
+
+// The panels' updates and the own pivots of a tile that holds its pivot rows'
+// chunk and is worked through in chunks (Us, Ls: 32 x 32 and 32 x 33 floats,
+// 16-byte aligned).  Returns with every row of the tile from the first pivot
+// down written and released; the U rows above remain to be written.
+template <int REGS>
+__device__ __forceinline__ void own_follow(const SymDev& sd, int s, int k, int K, int j, int q, int CH, int ns, int F,
+                                           int P, int J, int Q, int* Lf, int* Uf, int* err, float* f,
+                                           int32_t* status, int32_t* badcol, float* Us, float* Ls, float* Bt,
+                                           float* rinv) {
+  __shared__ int s_have;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
+  const int ld = CH + 1, j0 = j << 5, w = min(32, F - j0), R0 = q * CH, R1 = min(F, R0 + CH);
+  const int pe = min(j, P), qj = j0 / CH;
+  const bool piv = j < P && q == qj;  // the tile holds its block's diagonal
+  const int np = min(32, ns - j0);
+  const int last = (R1 - 1 - R0) / kOwnChunk;
+  auto release = [&](int v) {
+    __syncthreads();
+    if (tid == 0) dag_st_release(Lf + j * Q + q, v);
+  };
+  auto store = [&](int i0, int i1) {
+    for (int c = wid; c < w; c += nw) {
+      float* dst = f + (int64_t)(j0 + c) * F;
+      const float* src = Bt + c * ld - R0;
+      for (int i = i0 + lane; i < i1; i += 32) dst[i] = src[i];
+    }
+  };
+  auto have = [&](int p, int need) {  // the stage of panel p, at least `need`
+    if (tid == 0) s_have = own_wait(Lf + p * Q + q, need, err);
+    __syncthreads();
+    const int v = s_have;
+    __syncthreads();
+    return v;
+  };
+  int seen = 0;  // stage of panel j - 1
+  for (int p = 0; p < pe; ++p) {
+    const int r0 = p << 5, nb = min(32, ns - r0), qp = r0 / CH;
+    if (q < qp) break;
+    int v = 0;
+    if (q == qp) {
+      v = have(p, 1);
+      for (int e = tid; e < 32 * 32; e += nt) {
+        const int r = e & 31, c = e >> 5;
+        Ls[r * 33 + c] = (r < nb && c < r) ? __ldcg(f + (r0 + r) + (int64_t)(r0 + c) * F) : 0.f;
+      }
+      __syncthreads();
+      own_trsm<float>(Bt + (r0 - R0), ld, 0, nb, w, Ls, Us);
+      __syncthreads();
+      if (qp + 1 < Q) {  // tiles below read these U rows
+        for (int c = wid; c < w; c += nw)
+          for (int r = lane; r < nb; r += 32) f[(r0 + r) + (int64_t)(j0 + c) * F] = Bt[(r0 - R0 + r) + c * ld];
+        __syncthreads();
+        if (tid == 0) dag_st_release(Uf + p * J + j, 1);
+      }
+    } else {
+      if (tid == 0) dag_wait(Uf + p * J + j, 1, err);
+      v = have(p, 2);
+      for (int e = tid; e < 32 * 32; e += nt) {
+        const int r = e >> 5, c = e & 31;
+        Us[e] = (r < nb && c < w) ? __ldcg(f + (r0 + r) + (int64_t)(j0 + c) * F) : 0.f;
+      }
+      __syncthreads();
+    }
+    const int i0 = q == qp ? r0 + nb : R0;  // the rows below the panel's pivots
+    if (piv && p + 1 == pe) {  // goes on below, with the block's own pivots
+      seen = v;
+      break;
+    }
+    for (int c = (i0 - R0) / kOwnChunk; c <= last;) {
+      if (v < 2 + c) v = have(p, 2 + c);
+      const int ce = min(v - 1, last + 1);  // chunks below ce are there
+      own_update_pairs<REGS>(Bt, ld, R0, f, F, r0, nb, Us, max(i0, R0 + c * kOwnChunk), min(R1, R0 + ce * kOwnChunk), w);
+      c = ce;
+    }
+    __syncthreads();
+  }
+  if (!piv) return;
+  // panel j - 1 (32 pivots, its rows below end at j0) and the own pivots: the pivot rows, then chunk by chunk
+  const int p = j - 1, r0 = j0 - 32;
+  if (j > 0) {
+    const int c = (j0 + np - 1 - R0) / kOwnChunk;
+    if (seen < 2 + c) seen = have(p, 2 + c);
+    own_update_few(Bt, ld, R0, f, F, r0, 32, Us, j0, j0 + np, w);
+    __syncthreads();
+  }
+  own_factor_diag<float>(Bt + (j0 - R0), ld, np, w, Ls, rinv, sd, s, k, K, sd.c0[s] + j0, status, badcol);
+  __syncthreads();
+  store(j0, j0 + np);
+  release(1);
+  for (int c = (j0 + np - R0) / kOwnChunk; c <= last; ++c) {
+    const int a = max(j0 + np, R0 + c * kOwnChunk), b = min(R1, R0 + (c + 1) * kOwnChunk);
+    if (j > 0) {
+      if (seen < 2 + c) seen = have(p, 2 + c);
+      own_update_pairs<REGS>(Bt, ld, R0, f, F, r0, 32, Us, a, b, w);
+      __syncthreads();
+    }
+    own_eliminate_quads(Bt, ld, R0, a, b, np, Ls, rinv);
+    __syncthreads();
+    store(a, b);
+    if (c < last) release(2 + c);
+  }
+  release(kOwnDone);
+}
+
 // One owner tile: the 32-column block j of front s, perturbation k,
 // restricted to the row chunk q of CH rows (see above).  `flags` points at
 // the (front, k) pair's release flags.  Needs kOwnThreads threads and the
 // shared memory layout of the owner kernels (Us, Ls, Bt, rinv).
-template <typename T, bool TC>
+template <typename T, bool TC, int REGS>
 __device__ __forceinline__ void owner_tile(const SymDev& sd, int s, int k, int j, int q, int* flags, int CH,
                                            int* err, const double* __restrict__ vals,
                                            const double* __restrict__ D, const Shifts& sh,
@@ -1472,36 +1820,39 @@ __device__ __forceinline__ void owner_tile(const SymDev& sd, int s, int k, int j
   __syncthreads();
   {
     const int64_t a0 = sd.amap_coff[vo + j0], a1 = sd.amap_coff[vo + j0 + w];
-    for (int64_t e = a0 + tid; e < a1; e += nt) {
-      const int d = sd.amap_dst[e];
+    add_entries<T>(sd, vals, a0, a1, [&](int d, T v) {
       const int c = d / F, i = d - c * F;
-      if (i >= R0 && i < R1) atomicAdd(&Bt[(i - R0) + (c - j0) * ld], (T)vals[sd.amap_src[e]]);
-    }
+      if (i >= R0 && i < R1) atomicAdd(&Bt[(i - R0) + (c - j0) * ld], v);
+    });
     const double tk = sh.t[k];
     const int c0 = sd.c0[s];
     for (int c = max(j0, R0) + tid; c < min(min(j0 + w, ns), R1); c += nt)
       atomicAdd(&Bt[(c - R0) + (c - j0) * ld], (T)(tk * D[sd.perm[c0 + c]]));
   }
   __syncthreads();
-  extend_add_columns<T>(sd, s, k, K, fronts, Bt, ld, j0, w, R0, R1, (int)(threadIdx.x >> 5), (int)(blockDim.x >> 5));
+  extend_add_columns<T>(sd, s, k, K, fronts, Bt, ld, j0, w, R0, R1, wid, nw);
   __syncthreads();
 
   // 2. the updates of every earlier panel, in pivot order; panels whose
   //    pivot rows lie below the tile do not touch it
-  const int pe = min(j, P);
+  constexpr bool kFollow = std::is_same<T, float>::value && !TC;
+  if constexpr (kFollow)
+    own_follow<REGS>(sd, s, k, K, j, q, CH, ns, F, P, J, Q, Lf, Uf, err, f, status, badcol, Us, Ls, Bt, rinv);
+  const int pe = kFollow ? 0 : min(j, P);
   for (int p = 0; p < pe; ++p) {
     const int r0 = p << 5, nb = min(32, ns - r0), qp = r0 / CH;
     if (q < qp) break;
     if (q == qp) {
       // the tile holds panel p's pivot rows: solve this block's U rows
-      if (tid == 0) dag_wait(Lf + p * Q + qp, 1, err);
+      if (tid == 0) dag_wait(Lf + p * Q + qp, kOwnDone, err);
       __syncthreads();
       for (int e = tid; e < 32 * 32; e += nt) {
         const int r = e & 31, c = e >> 5;
         Ls[r * 33 + c] = (r < nb && c < r) ? __ldcg(f + (r0 + r) + (int64_t)(r0 + c) * F) : T(0);
       }
       __syncthreads();
-      own_trsm<T>(Bt + (r0 - R0), ld, 0, nb, w, Ls, Us);
+      if constexpr (sizeof(T) == 8) own_trsm_flat(Bt + (r0 - R0), ld, nb, w, Ls, Us);
+      else own_trsm<T>(Bt + (r0 - R0), ld, 0, nb, w, Ls, Us);
       __syncthreads();
       if (qp + 1 < Q) {  // chunks below read these U rows
         for (int c = wid; c < w; c += nw)
@@ -1512,8 +1863,8 @@ __device__ __forceinline__ void owner_tile(const SymDev& sd, int s, int k, int j
       }
       if constexpr (TC && std::is_same<T, float>::value)
         tc_update_rows(Bt, ld, R0, f, F, r0, nb, Us, r0 + nb, R1, w, tc, err);
-      else
-        own_update_rows<T>(Bt, ld, R0, f, F, r0, nb, Us, r0 + nb, R1, w);
+      else if constexpr (sizeof(T) == 8)
+        own_update_few64(Bt, ld, R0, f, F, r0, nb, Us, r0 + nb, R1, w);
       __syncthreads();
     } else {
       // a chunk below panel p: its U rows of this block come from the
@@ -1521,7 +1872,7 @@ __device__ __forceinline__ void owner_tile(const SymDev& sd, int s, int k, int j
       // panel p
       if (tid == 0) {
         dag_wait(Uf + p * J + j, 1, err);
-        dag_wait(Lf + p * Q + q, 1, err);
+        dag_wait(Lf + p * Q + q, kOwnDone, err);
       }
       __syncthreads();
       for (int e = tid; e < 32 * 32; e += nt) {
@@ -1531,8 +1882,8 @@ __device__ __forceinline__ void owner_tile(const SymDev& sd, int s, int k, int j
       __syncthreads();
       if constexpr (TC && std::is_same<T, float>::value)
         tc_update_rows(Bt, ld, R0, f, F, r0, nb, Us, R0, R1, w, tc, err);
-      else
-        own_update_rows<T>(Bt, ld, R0, f, F, r0, nb, Us, R0, R1, w);
+      else if constexpr (sizeof(T) == 8)
+        own_update_few64(Bt, ld, R0, f, F, r0, nb, Us, R0, R1, w);
       __syncthreads();
     }
   }
@@ -1541,10 +1892,14 @@ __device__ __forceinline__ void owner_tile(const SymDev& sd, int s, int k, int j
   const int qj = j0 / CH;
   if (j < P) {
     const int np = min(32, ns - j0);
-    if (q == qj) {
-      own_factor_diag<T>(Bt + (j0 - R0), ld, np, w, Us, rinv, sd, s, k, K, sd.c0[s] + j0, status, badcol);
+    if (q == qj && !kFollow) {
+      if constexpr (sizeof(T) == 8)
+        own_factor_diag_flat(Bt + (j0 - R0), ld, np, w, Us, rinv, sd, s, k, K, sd.c0[s] + j0, status, badcol);
+      else
+        own_factor_diag<T>(Bt + (j0 - R0), ld, np, w, Us, rinv, sd, s, k, K, sd.c0[s] + j0, status, badcol);
       __syncthreads();
-      own_eliminate_rows<T>(Bt, ld, R0, j0 + np, R1, np, w, Us, rinv);
+      if constexpr (sizeof(T) == 8) own_eliminate_flat(Bt, ld, R0, j0 + np, R1, np, w, Us, rinv);
+      else own_eliminate_rows<T>(Bt, ld, R0, j0 + np, R1, np, w, Us, rinv);
       __syncthreads();
     } else if (q > qj) {
       // rows below the diagonal block's chunk: its factored rows come from
@@ -1557,7 +1912,8 @@ __device__ __forceinline__ void owner_tile(const SymDev& sd, int s, int k, int j
       }
       if (tid < np) rinv[tid] = T(1) / __ldcg(f + (int64_t)(j0 + tid) * (F + 1));
       __syncthreads();
-      own_eliminate_rows<T>(Bt, ld, R0, R0, R1, np, w, Us, rinv);
+      if constexpr (sizeof(T) == 8) own_eliminate_flat(Bt, ld, R0, R0, R1, np, w, Us, rinv);
+      else own_eliminate_rows<T>(Bt, ld, R0, R0, R1, np, w, Us, rinv);
       __syncthreads();
     }
   }
@@ -1566,6 +1922,7 @@ __device__ __forceinline__ void owner_tile(const SymDev& sd, int s, int k, int j
   //    (rows from the first pivot down first, then the U rows above)
   const bool rel = j < P && q >= qj;
   const int rs = (rel && q == qj) ? j0 : R0;
+  if (!(kFollow && rel && q == qj)) {
   for (int c = wid; c < w; c += nw) {
     T* dst = f + (int64_t)(j0 + c) * F;
     const T* src = Bt + c * ld;
@@ -1574,7 +1931,8 @@ __device__ __forceinline__ void owner_tile(const SymDev& sd, int s, int k, int j
   if (rel) {
     __threadfence();
     __syncthreads();
-    if (tid == 0) dag_st_release(Lf + j * Q + q, 1);
+    if (tid == 0) dag_st_release(Lf + j * Q + q, kOwnDone);
+  }
   }
   for (int c = wid; c < w; c += nw) {
     T* dst = f + (int64_t)(j0 + c) * F;
@@ -1610,7 +1968,7 @@ __global__ void __launch_bounds__(kOwnThreads) k_front_owner(SymDev sd, const in
     const int u = s_t;
     if (u >= ntasks) break;
     const DagTask t = tasks[u];
-    owner_tile<T, TC>(sd, big[t.b], t.k, t.j, t.p, flags + t.flags, CH, err, vals, D, sh, fronts, status, badcol,
+    owner_tile<T, TC, 255>(sd, big[t.b], t.k, t.j, t.p, flags + t.flags, CH, err, vals, D, sh, fronts, status, badcol,
                   Us, Ls, Bt, rinv, tc);
   }
   if constexpr (TC) tc_teardown(tc);
@@ -1712,7 +2070,7 @@ k_factor_persistent(SymDev sd, const FactorTask* __restrict__ tasks, int ntasks,
       if (t.kind == kFacCta)
         front_cta<T>(sd, t.s, t.k, vals, D, sh, fronts, status, badcol, sm, rinv);
       else
-        owner_tile<T, TC>(sd, t.s, t.k, t.j, t.q, flags + t.flags, CH, err, vals, D, sh, fronts, status,
+        owner_tile<T, TC, MINB >= 3 ? 80 : 128>(sd, t.s, t.k, t.j, t.q, flags + t.flags, CH, err, vals, D, sh, fronts, status,
                           badcol, sm, sm + 32 * 32, sm + 32 * 32 + 32 * 33, rinv, tc);
       __syncthreads();
       if (tid == 0) fac_publish(sd, fdone, t.s, t.k, K);
@@ -1977,10 +2335,10 @@ int owner_chunk_rows(int precision, int maxF, int tc) {
   // Rows per tile.  FP64 elimination runs at a small fraction of the FP32
   // rate on this part, so one SM per 32-column block is the bottleneck of a
   // panel step: 32-row tiles spread a block's update and elimination over
-  // its chunks (1354-bus root: 0.66 ms against 0.82 with whole columns).  In
-  // FP32 the extra hand-offs and reloads of row chunks cost more than they
-  // save (10000-bus: 3.2-5.1 ms with 256- to 96-row tiles against 3.0), so a
-  // tile is a whole column block while it fits in shared memory.
+  // its chunks (1354-bus root: 0.66 ms against 0.82 with whole columns, when the
+  // kernels inside were slower; 0.40 with 32-row tiles now).  In FP32 a tile is a
+  // whole column block while it fits in shared memory: row chunks are handed
+  // over from inside it (own_follow), without their reloads.
   const int full = (maxF + 31) / 32 * 32;
   if (precision != PISP_FP32) return std::min(32, full);
   // (CH + 1) * 32 + 2080 floats, plus the tensor-core staging when it is on

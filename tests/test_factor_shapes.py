@@ -100,3 +100,33 @@ def test_many_children(precision, sweeps, policy):
         s.close()
         scale = float(sum(abs(w) for w in oracle.weights(t)))
         assert entrywise_err(x, oracle.x_hat(A, D, t, b)) <= 1e-10 * scale, (hub, arms)
+
+
+@pytest.mark.parametrize("policy", [0, 3, 4])
+@pytest.mark.parametrize("hub,arms", [(230, (27, 33, 70)), (250, (6, 40)), (480, (32, 64)), (530, (1, 95))])
+def test_owner_tiles(hub, arms, policy):
+    """Wide fronts around a chunk of 256 rows and a block of 32 columns: a dense hub
+    and dense blocks tied to all of it, a front of (block + hub) rows each."""
+    import torch
+    import paper_2311_11833_gb300 as pisp
+    r = np.random.default_rng(hub)
+    n = hub + sum(arms)
+    M = np.zeros((n, n))
+    M[:hub, :] = r.standard_normal((hub, n))
+    M[:, :hub] = r.standard_normal((n, hub))
+    at = hub
+    for a in arms:
+        M[at:at + a, at:at + a] = r.standard_normal((a, a))
+        at += a
+    M[np.arange(n), np.arange(n)] = 2.0 * np.sqrt(n) + abs(M[np.arange(n), np.arange(n)])
+    A, D = sp.csr_matrix(M), r.uniform(0.5, 1.5, n)
+    t = pfgen.symmetric_shifts(2, 1e-3)
+    s = pisp.Solver([n], A.indptr.astype(np.int64), A.indices.astype(np.int32), factor_policy=policy)
+    dev = lambda a: torch.tensor(np.asarray(a), dtype=torch.float64, device="cuda")  # noqa: E731
+    s.factor(dev(A.data), dev(D), t, "fp32")
+    assert s.stats()["max_front"] >= hub + 1
+    b = pfgen.rhs(n, 2, 1)
+    x = s.solve(dev(b), sweeps=5).cpu().numpy()
+    assert s.status()[0] == 0
+    s.close()
+    assert entrywise_err(x, oracle.x_hat(A, D, t, b)) <= 1e-10 * float(sum(abs(w) for w in oracle.weights(t)))
