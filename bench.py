@@ -46,13 +46,7 @@ L2_BYTES = 129 * 1024 * 1024
 # to the full workload where the capture ran a reduced batch); an entry is
 # removed when its kernel changes.
 # Keys: (workload, family, instances, library options as sorted (name, value) pairs).
-BATCH_TUNED = (("factor_ctas_per_sm", 3), ("factor_policy", 4), ("factor_smem_maxF", 128), ("relax_small", 16),
-               ("relax_zeros", 0.1), ("solve_ctas_per_sm", 4), ("solve_kfuse", 1), ("solve_schedule", 0),
-               ("solve_warp_maxF", 64))
-TRAFFIC_PER_LAUNCH = {
-    ("batching", "backward", 256, BATCH_TUNED): 670.31e6,            # 586.72 MB read + 83.59 MB written
-    ("batching", "factor_persistent", 256, BATCH_TUNED): 1378.02e6,  # 619.55 MB read + 758.47 MB written
-}
+TRAFFIC_PER_LAUNCH = {}
 
 # factor precision and FP64 residual sweeps per workload; refine_tol > 0:
 # adaptive sweeps (pisp_set_refinement), `sweeps` is then the maximum
@@ -84,7 +78,7 @@ def parse():
     ap.add_argument("--eps", type=float, default=1e-2)
     ap.add_argument("--no-graph", action="store_true", help="launch eagerly instead of a CUDA graph")
     ap.add_argument("--factor-policy", type=int, default=0, choices=[0, 1, 2, 3, 4],
-                    help="fronts wider than 64: 0 single CTA / column-block owners (default), "
+                    help="0 by size: one launch, or per level with single CTA / column-block owners (default), "
                          "1 CTA clusters, 2 single CTA / tile DAG, 3 single CTA / per-panel launches, "
                          "4 one persistent launch for the whole factorisation")
     ap.add_argument("--schedule", type=int, default=0, choices=[0, 1],
@@ -510,7 +504,7 @@ def run_pisp(args, rank, world, local_rank):
                                    if refine_tol > 0 and sweeps else "fixed"),
                    "graph": "library (pisp_graph_capture)" if use_graph else None,
                    "solve_schedule": ["persistent", "per-level"][args.schedule],
-                   "factor_policy": ["single-CTA/column-block-owners", "clusters", "single-CTA/tile-DAG",
+                   "factor_policy": ["by size: one launch, or single-CTA/column-block-owners", "clusters", "single-CTA/tile-DAG",
                                      "single-CTA/per-panel", "one-launch-persistent"][
                        (tuned["options"].get("factor_policy", 0) if tuned else args.factor_policy)], "l2": "flushed between steps (256 MB write outside the events)",
                    "parallelism": f"replicas x{world}"},
