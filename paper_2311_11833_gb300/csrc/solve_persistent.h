@@ -543,6 +543,12 @@ __device__ __forceinline__ void stage_block(T* B, T* rd, const T* f, int F, int 
   if (!UNIT && tid < 32) rd[tid] = tid < ns ? T(1) / dg : T(1);
 }
 
+// Shared memory of a front of the two kinds below, in elements: the diagonal
+// block, its reciprocal pivots, then the pivots' values (forward) or the warps'
+// partial sums (backward)
+constexpr int kThinRd = 32 * kBS, kThinV = kThinRd + 32;
+constexpr int thin_smem(bool fwd, int nr) { return kThinV + (fwd ? 32 * nr : kSolveWarps * 32); }
+
 // Wider fronts with at most 32 pivots, one (front, shift, chunk) a CTA: every
 // thread keeps its row's values and coefficients in registers; only the pivot
 // rows meet in shared memory.
@@ -552,8 +558,8 @@ __device__ __forceinline__ void thin_forward(const SolveArgs<T>& a, const FrontD
   const int ns = d.ns, F = d.F;
   const bool vec = a.vec && (r0 % Vec16<T>::N == 0);
   T* B = sm;                    // 32 x kBS
-  T* rdv = B + 32 * kBS;        // 32
-  T* y = rdv + 32;              // 32 x NR
+  T* rdv = B + kThinRd;         // 32
+  T* y = B + kThinV;            // 32 x NR
   const T* f = a.fronts + a.K * d.fo + (int64_t)k * F * F;
   stage_block<T, true, !TRANS, TRANS>(B, rdv, f, F, ns, tid);
   Gather g = gather_begin<T>(a, d, tid, tid < F);
@@ -618,8 +624,8 @@ __device__ __forceinline__ void thin_backward1(const SolveArgs<T>& a, const Fron
   const int ns = d.ns, F = d.F, ms = F - ns;
   const int64_t K = a.K;
   T* B = sm;                    // 32 x kBS
-  T* rdv = B + 32 * kBS;        // 32
-  T* part = rdv + 32;           // 8 warps x 32
+  T* rdv = B + kThinRd;         // 32
+  T* part = B + kThinV;         // 8 warps x 32
   const T* f = a.fronts + K * d.fo + (int64_t)k * F * F;
   stage_block<T, false, TRANS, TRANS>(B, rdv, f, F, ns, tid);
   const int lp = ns <= 1 ? 0 : 32 - __clz(ns - 1);  // log2 of the pivots rounded up
@@ -1385,8 +1391,8 @@ int launch_solve_dir(bool trans, const SolveArgs<T>& a0, int32_t nunits, int32_t
   SolveArgs<T> a = a0;
   size_t e;
   if (FWD || a.R == 1) {
-    const size_t nr = a.R == 1 ? 1 : 8;
-    e = std::max((size_t)32 * kBS + 32 + 32 * nr, (size_t)kSolveWarps * 32 * nr);
+    const int nr = a.R == 1 ? 1 : 8;
+    e = std::max(thin_smem(FWD, nr), kSolveWarps * 32 * nr);
   } else {
     // most shifts among 32 columns
     a.stage = col_stage<T>(std::min(a.K, (31 + a.RV - 1) / a.RV + 1));

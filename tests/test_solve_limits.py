@@ -1,0 +1,94 @@
+"""Solves at the limits of their launches: what a task may use of shared memory,
+schedules rebuilt under work in flight, waits that run out, and calls that fail."""
+import numpy as np
+import pytest
+import scipy.sparse as sp
+
+import oracle
+import pfgen
+from _parity import entrywise_err, grad_entrywise_err
+from test_abi import HostSymbolic
+
+TOL = 1e-10  # the repository's entry-wise bound (FP64 factors, or FP32 with FP64 sweeps)
+HUB = 32
+ARMS = (2, 3, 5, 8, 9, 17, 32)
+
+
+def _thin(p):
+    """Two dense blocks of p unknowns, each tied to all of a dense hub of 32 but one:
+    two fronts of p pivots and p + 31 rows under a root of 32 pivots."""
+    r = np.random.default_rng(p)
+    n = 2 * p + HUB
+    M = np.zeros((n, n))
+    M[2 * p:, 2 * p:] = r.standard_normal((HUB, HUB))
+    for a in range(2):
+        at = np.arange(a * p, a * p + p)
+        hub = 2 * p + np.delete(np.arange(HUB), a)
+        M[np.ix_(at, at)] = r.standard_normal((p, p))
+        M[np.ix_(at, hub)] = r.standard_normal((p, HUB - 1))
+        M[np.ix_(hub, at)] = r.standard_normal((HUB - 1, p))
+    d = np.arange(n)
+    M[d, d] = 2.0 * np.sqrt(n) + abs(M[d, d])
+    A = sp.csr_matrix(M)
+    return pfgen.Instance(n=n, row_ptr=A.indptr.astype(np.int64), col=A.indices.astype(np.int32), val=A.data,
+                          D=r.uniform(0.5, 1.5, n), meta={})
+
+
+def _concat(insts):
+    rp, cols, off = [0], [], 0
+    for I in insts:
+        rp.extend((I.row_ptr[1:] + rp[-1]).tolist())
+        cols.append(I.col + off)
+        off += I.n
+    return ([I.n for I in insts], np.array(rp, np.int64), np.concatenate(cols).astype(np.int32),
+            np.concatenate([I.val for I in insts]), np.concatenate([I.D for I in insts]))
+
+
+def _dev(a):
+    import torch
+    return torch.tensor(np.asarray(a), dtype=torch.float64, device="cuda")
+
+
+def test_thin_fronts_and_no_wider_pivot_blocks():
+    """The systems of the next test are what it says: fronts of more than 32 rows,
+    none with more than 32 pivots."""
+    import paper_2311_11833_gb300._lib as L
+    insts = [_thin(p) for p in ARMS]
+    sizes, rp, col, _, _ = _concat(insts)
+    hs = HostSymbolic(L.load(), sizes, rp, col, ordering=1, relax_small=1, relax_zeros=0.0)
+    assert hs.rc == 0
+    ns = hs.c1 - hs.c0
+    assert ns.max() == HUB and set(ns[ns + hs.ms > 32]) == set(ARMS)
+    hs.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision,sweeps", [("fp64", 0), ("fp32", 4)])
+@pytest.mark.parametrize("K", [1, 4])
+def test_thin_fronts_one_right_hand_side(precision, sweeps, K):
+    """Fronts of more than 32 rows solved by a CTA while no front has more than 32
+    pivots, whose tasks would ask for far more shared memory: the backward solve of
+    one right-hand side once asked for less than its partial sums take."""
+    import paper_2311_11833_gb300 as pisp
+    insts = [_thin(p) for p in ARMS]
+    sizes, rp, col, val, D = _concat(insts)
+    t = pfgen.one_sided_shifts(K, 1e-3) if K % 2 else pfgen.symmetric_shifts(K, 1e-3)
+    N = sum(sizes)
+    b, g = pfgen.rhs(N, 1, 5), pfgen.rhs(N, 1, 6)
+    s = pisp.Solver(sizes, rp, col, ordering=1, relax_small=1, relax_zeros=0.0)
+    s.factor(_dev(val), _dev(D), t, precision)
+    x = s.solve(_dev(b), sweeps=sweeps).cpu().numpy()
+    gb, gv = (v.cpu().numpy() for v in s.adjoint(_dev(g), sweeps=sweeps))
+    assert s.status()[0] == 0
+    s.close()
+    scale = float(sum(abs(w) for w in oracle.weights(t)))
+    r0 = e0 = 0
+    for I in insts:
+        rows, ent = slice(r0, r0 + I.n), slice(e0, e0 + I.nnz)
+        A = oracle.to_scipy(I)
+        assert entrywise_err(x[rows], oracle.x_hat(A, I.D, t, b[rows])) <= TOL * scale, I.n
+        rb, rv = oracle.adjoint(A, I.D, t, b[rows], g[rows])
+        assert entrywise_err(gb[rows], rb) <= TOL * scale, I.n
+        assert grad_entrywise_err(gv[ent], rv) <= TOL * scale, I.n
+        r0 += I.n
+        e0 += I.nnz
