@@ -30,7 +30,10 @@ constexpr int kSolveThreads = 256;
 constexpr int kSolveWarps = kSolveThreads / 32;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kBS = 33;                              // padded row of a staged 32 x 32 block
-constexpr int kSolveSmemMax = 128 * 1024;
+// Shared memory a launch may ask for.  The most is asked for by column tasks of
+// FP64 factors with two right-hand sides, whose 32 columns are 16 shifts (K = 16:
+// 158720 bytes, one CTA an SM); checked at compile time with the layouts below.
+constexpr int kSolveSmemMax = 160 * 1024;
 
 __device__ __forceinline__ int ld_relaxed(const int* p) {
   int v;
@@ -694,7 +697,7 @@ template <typename T> struct Stage { static constexpr int LD = sizeof(T) == 4 ? 
 
 // per-warp stage: two buffers of nk sets, the reciprocal pivots of a block (nk x 9)
 template <typename T>
-__host__ __device__ __forceinline__ int col_stage(int nk) { return 2 * nk * Stage<T>::LD + (nk * 9 + 3) / 4 * 4; }
+__host__ __device__ constexpr int col_stage(int nk) { return 2 * nk * Stage<T>::LD + (nk * 9 + 3) / 4 * 4; }
 
 template <typename T>
 struct Cols {
@@ -1385,6 +1388,15 @@ int launch_one(const SolveArgs<T>& a, int nunits, size_t smem, cudaStream_t st) 
 
 }  // namespace
 
+// elements of a launch's column tasks (8 warps' stages and partial sums), and of
+// its tasks of fronts with more than 32 pivots, `wide` right-hand sides each
+template <typename T>
+constexpr size_t col_smem(int nk) { return (size_t)kSolveWarps * col_stage<T>(nk) + (size_t)(kSolveWarps - 1) * 8 * 32; }
+template <typename T>
+constexpr size_t wide_smem(int wide, bool trans) {
+  return (size_t)kWideRows * wide + (size_t)kSolveWarps * kTri + (trans ? (size_t)kSolveWarps * 32 * WideTile<T>::LD : 0);
+}
+
 template <typename T, bool FWD>
 int launch_solve_dir(bool trans, const SolveArgs<T>& a0, int32_t nunits, int32_t wide, int32_t ctas, cudaStream_t st) {
   if (nunits <= 0) return 0;
@@ -1395,14 +1407,15 @@ int launch_solve_dir(bool trans, const SolveArgs<T>& a0, int32_t nunits, int32_t
     e = std::max(thin_smem(FWD, nr), kSolveWarps * 32 * nr);
   } else {
     // most shifts among 32 columns
-    a.stage = col_stage<T>(std::min(a.K, (31 + a.RV - 1) / a.RV + 1));
-    e = (size_t)kSolveWarps * a.stage + (size_t)(kSolveWarps - 1) * 8 * 32;
+    const int nk = std::min(a.K, (31 + a.RV - 1) / a.RV + 1);
+    a.stage = col_stage<T>(nk);
+    e = col_smem<T>(nk);
   }
-  if (wide > 0)
-    e = std::max(e, (size_t)kWideRows * wide + (size_t)kSolveWarps * kTri +
-                        (trans ? (size_t)kSolveWarps * 32 * WideTile<T>::LD : 0));
+  if (wide > 0) e = std::max(e, wide_smem<T>(wide, trans));
   const size_t smem = e * sizeof(T);
-  if (smem > (size_t)kSolveSmemMax) return -1;
+  static_assert(col_smem<T>(PISP_K_MAX) * sizeof(T) <= kSolveSmemMax && wide_smem<T>(wide_chunk<T>(), true) * sizeof(T) <= kSolveSmemMax &&
+                    std::max(thin_smem(FWD, 8), kSolveWarps * 32 * 8) * sizeof(T) <= kSolveSmemMax,
+                "every launch of a solve fits");
   if (a.R == 1)
     return trans ? launch_one<T, FWD, true, 2, true>(a, nunits, smem, st)
                  : launch_one<T, FWD, false, 2, true>(a, nunits, smem, st);

@@ -92,3 +92,14 @@ def test_thin_fronts_one_right_hand_side(precision, sweeps, K):
         assert grad_entrywise_err(gv[ent], rv) <= TOL * scale, I.n
         r0 += I.n
         e0 += I.nnz
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision,sweeps", [("fp64", 0), ("fp32", 4)])
+@pytest.mark.parametrize("K", [12, 13, 16])
+def test_two_right_hand_sides_many_shifts(precision, sweeps, K):
+    """Two right-hand sides put up to 16 shifts into a group of 32 columns, each with
+    coefficients of its own in shared memory: with FP64 factors 13 shifts and more
+    were once refused."""
+    import test_solve_shapes as shapes
+    shapes.test_solve_and_adjoint_shapes(precision, sweeps, K, 2, {})
