@@ -231,10 +231,24 @@ int set_device(pisp_handle* h, DeviceScope& scope) {
   return PISP_OK;
 }
 
+// Copies v to b, which keeps its allocation when it is large enough: on the
+// handle's stream, so that work in flight there reads the old contents to its end
+// and what is queued next reads the new ones (a copy on the legacy stream is
+// ordered with neither when the handle's stream is a non-blocking one).  v may be
+// freed afterwards.  While the stream is being captured the copy is not to become
+// part of the graph.
 template <typename T>
 int upload(pisp_handle* h, Buf& b, const std::vector<T>& v) {
   if (!b.ensure(v.size() * sizeof(T))) return fail(h, PISP_ERR_OOM, "device allocation failed");
-  if (!v.empty()) CK(cudaMemcpy(b.p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
+  if (v.empty()) return PISP_OK;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  CK(cudaStreamIsCapturing(h->stream, &cs));
+  if (cs != cudaStreamCaptureStatusNone) {
+    CK(cudaMemcpy(b.p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
+    return PISP_OK;
+  }
+  CK(cudaMemcpyAsync(b.p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, h->stream));
+  CK(cudaStreamSynchronize(h->stream));
   return PISP_OK;
 }
 

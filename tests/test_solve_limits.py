@@ -103,3 +103,43 @@ def test_two_right_hand_sides_many_shifts(precision, sweeps, K):
     were once refused."""
     import test_solve_shapes as shapes
     shapes.test_solve_and_adjoint_shapes(precision, sweeps, K, 2, {})
+
+
+@pytest.mark.gpu
+def test_schedules_rebuilt_under_work_in_flight():
+    """Other numbers of right-hand sides and of shifts rebuild the task lists while
+    solves and factorisations that read the old ones wait behind a long kernel on a
+    stream that the legacy stream does not wait for."""
+    import torch
+    import paper_2311_11833_gb300 as pisp
+    insts = [pfgen.grid_jacobian(n, None, n) for n in (60, 140, 200)]
+    sizes, rp, col, val, D = _concat(insts)
+    N = sum(sizes)
+    s = pisp.Solver(sizes, rp, col)
+    vals_d, D_d = _dev(val), _dev(D)
+    steps = [(K, R) for K in (4, 2) for R in (12, 1, 5, 2)] + [(4, 3)]
+    rhs = [_dev(pfgen.rhs(N, R, R)) for _, R in steps]
+    st = torch.cuda.Stream()
+    st.wait_stream(torch.cuda.current_stream())
+    got, want = [], []
+    with torch.cuda.stream(st):
+        for out, busy in ((want, False), (got, True)):
+            for (K, R), b in zip(steps, rhs):
+                if busy:
+                    torch.cuda._sleep(20_000_000)  # about 10 ms
+                s.factor(vals_d, D_d, pfgen.symmetric_shifts(K), "fp64")
+                out.append(s.solve(b))
+                if not busy:
+                    st.synchronize()
+    st.synchronize()
+    assert s.status()[0] == 0
+    s.close()
+    r0 = 0
+    for I in insts:
+        rows = slice(r0, r0 + I.n)
+        A = oracle.to_scipy(I)
+        for (K, R), b, x, w in zip(steps, rhs, got, want):
+            assert torch.equal(x, w), (K, R)
+            t = pfgen.symmetric_shifts(K)
+            assert entrywise_err(x[rows].cpu().numpy(), oracle.x_hat(A, I.D, t, b[rows].cpu().numpy())) <= TOL, (K, R)
+        r0 += I.n
