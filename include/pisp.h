@@ -315,18 +315,19 @@ int pisp_graph_capture(pisp_handle* h, const double* values, const double* D, co
 int pisp_graph_launch(pisp_handle* h);
 
 /* The bounded device waits (no counterpart in the paper).  Every dependency
- * wait of the persistent solves polls a completion counter at most `polls`
- * times (32 ns apart at first, up to 1 us in a long wait) and then gives up: it
- * records the failure, the task goes on with whatever data is there, the launch
- * ends normally, and
- * pisp_get_status returns PISP_ERR_TIMEOUT until the next
- * pisp_factor_perturbed clears the record.  polls = 0 restores the default
- * (2^22 polls, a few seconds per wait).  unreachable != 0 is a test
- * hook: the next solves also wait on one completion target raised by one, which
- * no task ever reaches, so that a wait runs out on purpose (results of those
- * solves are not valid); unreachable = 0 restores the true targets.  Applies
- * from the next pisp_solve / pisp_refine.  Returns PISP_ERR_INVALID_ARG for
- * polls < 0. */
+ * wait of the persistent solves, plain and transposed, and of the one-launch
+ * factorisation under factor_policy 4 polls a completion counter for the time of
+ * `polls` polls 64 ns apart (the polls grow apart from 32 ns to 1 us in a long wait)
+ * and then gives up: it records the failure, the task goes on with whatever data
+ * is there, the launch ends normally, and pisp_get_status returns
+ * PISP_ERR_TIMEOUT until the next pisp_factor_perturbed clears the record.
+ * polls = 0 restores the default (2^22 polls, a few tenths of a second per wait),
+ * which the other waits of a factorisation always have.  unreachable != 0 is a
+ * test hook: the next solves also wait on one completion target raised by one,
+ * which no task ever reaches, so that a wait runs out on purpose (results of
+ * those solves are not valid); unreachable = 0 restores the true targets.
+ * Applies from the next pisp_factor_perturbed / pisp_solve / pisp_refine /
+ * pisp_adjoint.  Returns PISP_ERR_INVALID_ARG for polls < 0. */
 int pisp_set_wait_limit(pisp_handle* h, int64_t polls, int32_t unreachable);
 
 /* Adaptive FP64 residual sweeps (no counterpart in the paper, which solves

@@ -780,7 +780,7 @@ int solve_pass_t(pisp_handle* h, bool trans, const SolveIO& io, int32_t R, const
   a.perm = h->sd.perm;
   a.act = act;
   a.err = h->serr.as<int>();
-  a.polls = h->wait_polls > 0 ? h->wait_polls : (int64_t)1 << 22;
+  a.wait_ns = pisp::wait_limit_ns(h->wait_polls);
   a.fronts = h->fronts.as<T>();
   a.b = io.b;
   a.rk = (const T*)io.rk;

@@ -913,7 +913,7 @@ __global__ void __launch_bounds__(256) k_front_cluster(SymDev sd, const int32_t*
 // tasks in ticket order and wait only for tasks with smaller tickets; every
 // wait is bounded and sets *err when it gives up.
 // ---------------------------------------------------------------------------
-constexpr int64_t kDagWaitPolls = 1 << 22;
+constexpr int64_t kDagWaitPolls = kWaitPolls;
 
 __device__ __forceinline__ int dag_ld_acquire(const int* p) {
   int v;
@@ -1993,7 +1993,7 @@ __global__ void __launch_bounds__(kOwnThreads) k_front_owner(SymDev sd, const in
 // whatever the residency, and every wait is bounded.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void fac_wait_children(const SymDev& sd, const int* fdone, const int* need, int s,
-                                                  int k, int K, int* err, int64_t polls) {
+                                                  int k, int K, int* err, int64_t wait_ns) {
   const int want = need[s];
   if (want == 0) return;
   const int* f = fdone + ((int64_t)s * K + k) * kCtrStride;
@@ -2001,11 +2001,12 @@ __device__ __forceinline__ void fac_wait_children(const SymDev& sd, const int* f
   // the polls in between are relaxed: an acquiring one drops the SM's L1 lines
   // under the CTA beside it
   unsigned ns = 32;
-  for (int64_t i = 0; i < polls; ++i) {
+  for (int64_t left = wait_ns; left > 0;) {
     __nanosleep(ns);
     int v;
     asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
     if (v >= want) break;
+    left -= ns;
     ns += ns < 1024 ? ns >> 3 : 0;
   }
   if (dag_ld_acquire(f) < want) atomicExch(err, 1);
@@ -2019,14 +2020,14 @@ __device__ __forceinline__ void fac_publish(const SymDev& sd, int* fdone, int s,
 
 template <typename T, int SEG>
 __device__ __forceinline__ void fac_segments(const SymDev& sd, const FactorTask& t, const int* need, int* fdone,
-                                             int* err, int64_t polls, const int32_t* __restrict__ wlist,
+                                             int* err, int64_t wait_ns, const int32_t* __restrict__ wlist,
                                              const double* __restrict__ vals, const double* __restrict__ D,
                                              const Shifts& sh, T* __restrict__ fronts, int32_t* status,
                                              int32_t* badcol, T* sm) {
   const int q = t.q + (int)threadIdx.x / SEG, sl = threadIdx.x % SEG;
   const bool on = q < t.j;
   const int s = on ? wlist[t.s + q / sh.K] : 0, k = on ? q % sh.K : 0;
-  if (on && sl == 0) fac_wait_children(sd, fdone, need, s, k, sh.K, err, polls);
+  if (on && sl == 0) fac_wait_children(sd, fdone, need, s, k, sh.K, err, wait_ns);
   __syncwarp();
   front_seg<T, SEG>(sd, s, k, on, sl, vals, D, sh, fronts, status, badcol, sm + threadIdx.x / SEG * SEG * SEG);
   __syncwarp();
@@ -2038,7 +2039,7 @@ __global__ void __launch_bounds__(kOwnThreads, MINB)
 k_factor_persistent(SymDev sd, const FactorTask* __restrict__ tasks, int ntasks, int* ticket, int* fdone,
                     const int* __restrict__ need, int* flags, int* err, const int32_t* __restrict__ wlist,
                     const double* __restrict__ vals, const double* __restrict__ D, const __grid_constant__ Shifts sh,
-                    T* __restrict__ fronts, int32_t* status, int32_t* badcol, int CH, int64_t polls,
+                    T* __restrict__ fronts, int32_t* status, int32_t* badcol, int CH, int64_t wait_ns,
                     size_t tc_off) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int s_t;
@@ -2059,13 +2060,13 @@ k_factor_persistent(SymDev sd, const FactorTask* __restrict__ tasks, int ntasks,
     if (u >= ntasks) break;
     const FactorTask t = tasks[u];
     if (t.kind == kFacSeg8) {
-      fac_segments<T, 8>(sd, t, need, fdone, err, polls, wlist, vals, D, sh, fronts, status, badcol, sm);
+      fac_segments<T, 8>(sd, t, need, fdone, err, wait_ns, wlist, vals, D, sh, fronts, status, badcol, sm);
     } else if (t.kind == kFacSeg16) {
-      fac_segments<T, 16>(sd, t, need, fdone, err, polls, wlist, vals, D, sh, fronts, status, badcol, sm);
+      fac_segments<T, 16>(sd, t, need, fdone, err, wait_ns, wlist, vals, D, sh, fronts, status, badcol, sm);
     } else if (t.kind == kFacSeg32) {
-      fac_segments<T, 32>(sd, t, need, fdone, err, polls, wlist, vals, D, sh, fronts, status, badcol, sm);
+      fac_segments<T, 32>(sd, t, need, fdone, err, wait_ns, wlist, vals, D, sh, fronts, status, badcol, sm);
     } else {
-      if (tid == 0) fac_wait_children(sd, fdone, need, t.s, t.k, K, err, polls);
+      if (tid == 0) fac_wait_children(sd, fdone, need, t.s, t.k, K, err, wait_ns);
       __syncthreads();
       if (t.kind == kFacCta)
         front_cta<T>(sd, t.s, t.k, vals, D, sh, fronts, status, badcol, sm, rinv);
@@ -2097,7 +2098,7 @@ int factor_persistent_launch(const SymDev& sd, const FactorTask* tasks, int ntas
   const int grid = std::max(1, std::min(ntasks, std::max(1, occ) * std::max(nsm, 1)));
   k_factor_persistent<T, TC, M><<<grid, kOwnThreads, smem, st>>>(sd, tasks, ntasks, ticket, fdone, need, flags,
                                                                  err, wlist, vals, D, sh, (T*)fronts, status,
-                                                                 badcol, CH, polls > 0 ? polls : kDagWaitPolls,
+                                                                 badcol, CH, wait_limit_ns(polls),
                                                                  tc_off);
   return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }

@@ -19,6 +19,14 @@ inline int current_device() {
   return d;
 }
 
+// Limit of a bounded wait on the device, stated in polls 64 ns apart (0: the
+// default).  The polls of a long wait grow apart, so the limit is kept as the time
+// asleep between them; with the polls themselves the default is about 0.4 s.
+constexpr int64_t kWaitPolls = 1 << 22;
+inline int64_t wait_limit_ns(int64_t polls) {
+  return 64 * (polls <= 0 ? kWaitPolls : polls < INT64_MAX / 64 ? polls : INT64_MAX / 64);
+}
+
 constexpr int kCtrStride = 8;  // ints between completion counters: a 32-byte sector each
 
 // A child as its parent's assembly needs it; mask (parents of at most 32 rows):
@@ -252,7 +260,7 @@ struct SolveArgs {
   int* done;              // [S][NG] finished tasks, zero; nullptr (one launch per stage): nothing to wait for
   int* wide;              // solved blocks per (front with more than 32 pivots, shift, chunk), zero
   int* err;               // set if a wait gave up
-  int64_t polls;
+  int64_t wait_ns;        // most time asleep in one wait
   const T* fronts;
   const double* b;        // broadcast right-hand side, or nullptr: rk
   const T* rk;

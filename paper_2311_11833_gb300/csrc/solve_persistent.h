@@ -47,8 +47,8 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
   return v;
 }
 
-// One thread waits until *f >= need, at most `polls` polls; then gives up and
-// records it.  Returns the count seen.  Whatever thread group continues is
+// One thread waits until *f >= need, asleep between polls for at most wait_ns in
+// all; then gives up and records it.  Returns the count seen.  Whatever thread group continues is
 // ordered after the acquiring load by the caller's barrier; the data themselves
 // are read past L1.  The polls in between are relaxed (an acquiring one drops
 // the SM's L1 lines each time, under the CTAs at work beside it) and end with an
@@ -57,13 +57,14 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 // waited up to 1 us, and every counter has a sector of its own (kCtrStride):
 // hundreds of pollers on a few lines fill the L2 slices that hold them, ahead of
 // the results and the counts they wait for.
-__device__ __forceinline__ int wait_count(const int* f, int need, int* err, int64_t polls) {
+__device__ __forceinline__ int wait_count(const int* f, int need, int* err, int64_t wait_ns) {
   int v = ld_acquire(f);
   if (v >= need) return v;
   unsigned ns = 32;
-  for (int64_t i = 0; i < polls; ++i) {
+  for (int64_t left = wait_ns; left > 0;) {
     __nanosleep(ns);
     if (ld_relaxed(f) >= need) break;
+    left -= ns;
     ns += ns < 1024 ? ns >> 3 : 0;
   }
   v = ld_acquire(f);
@@ -86,7 +87,7 @@ __device__ __forceinline__ void publish(int* f) {
 // counts all its tasks together (at group 0).
 template <typename T>
 __device__ __forceinline__ void wait_children(const SolveArgs<T>& a, const FrontDesc& d, int g) {
-  if (a.done && d.needF > 0) wait_count(a.done + ((int64_t)d.s * a.NG + g) * kCtrStride, d.needF, a.err, a.polls);
+  if (a.done && d.needF > 0) wait_count(a.done + ((int64_t)d.s * a.NG + g) * kCtrStride, d.needF, a.err, a.wait_ns);
 }
 template <typename T>
 __device__ __forceinline__ void publish_up(const SolveArgs<T>& a, const FrontDesc& d, int g) {
@@ -98,10 +99,10 @@ template <typename T>
 __device__ __forceinline__ void wait_parent(const SolveArgs<T>& a, const FrontDesc& d, int g) {
   if (!a.done || d.parent < 0) return;
   const int* c = a.done + (int64_t)d.parent * a.NG * kCtrStride;
-  if (d.whole & kParentWhole) wait_count(c, d.needB, a.err, a.polls);
+  if (d.whole & kParentWhole) wait_count(c, d.needB, a.err, a.wait_ns);
   else if (d.whole & kSelfWhole)
-    for (int q = 0; q < a.NG; ++q) wait_count(c + q * kCtrStride, d.needB, a.err, a.polls);
-  else wait_count(c + g * kCtrStride, d.needB, a.err, a.polls);
+    for (int q = 0; q < a.NG; ++q) wait_count(c + q * kCtrStride, d.needB, a.err, a.wait_ns);
+  else wait_count(c + g * kCtrStride, d.needB, a.err, a.wait_ns);
 }
 template <typename T>
 __device__ __forceinline__ void publish_self(const SolveArgs<T>& a, const FrontDesc& d, int g) {
@@ -1117,7 +1118,7 @@ __device__ __forceinline__ void wide_forward(const SolveArgs<T>& a, const FrontD
   // blocks solved by other CTAs
   const int next = min(b0, nblk);
   for (int p = 0; p < next;) {
-    if (tid == 0) s_seen = wait_count(flag, p + 1, a.err, a.polls);
+    if (tid == 0) s_seen = wait_count(flag, p + 1, a.err, a.wait_ns);
     __syncthreads();  // also: the blocks before are taken in
     const int m = min(next, min(max(s_seen, p + 1), p + kSolveWarps)) - p;
     if (tid < m * 32) {
@@ -1228,7 +1229,7 @@ __device__ __forceinline__ void wide_backward(const SolveArgs<T>& a, const Front
   const int top = nblk - 1;
   if (rows && mine < top) load_panel<T, TRANS>(L, f, F, i, ns, top * 32, ns - top * 32, tile, lane);
   for (int p = top; p > hi;) {
-    if (tid == 0) s_seen = wait_count(flag, nblk - p, a.err, a.polls);
+    if (tid == 0) s_seen = wait_count(flag, nblk - p, a.err, a.wait_ns);
     __syncthreads();
     const int m = min(p - hi, min(max(s_seen, nblk - p) - (top - p), kSolveWarps));
     const int lo = p - m + 1;

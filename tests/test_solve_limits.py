@@ -143,3 +143,26 @@ def test_schedules_rebuilt_under_work_in_flight():
             t = pfgen.symmetric_shifts(K)
             assert entrywise_err(x[rows].cpu().numpy(), oracle.x_hat(A, I.D, t, b[rows].cpu().numpy())) <= TOL, (K, R)
         r0 += I.n
+
+
+@pytest.mark.gpu
+def test_default_wait_limit_is_a_few_tenths_of_a_second():
+    """2^22 polls 64 ns apart are 0.27 s of sleep, however far apart the polls of a
+    long wait really are (1 us: 4.3 s); a task that gives up lets the next ones on."""
+    import time
+    import torch
+    import paper_2311_11833_gb300 as pisp
+    inst = pfgen.make_instance("plain")
+    s = pisp.Solver(inst.n, inst.row_ptr, inst.col)
+    s.factor(_dev(inst.val), _dev(inst.D), pfgen.symmetric_shifts(2), "fp64")
+    b = _dev(pfgen.rhs(inst.n, 2, 3))
+    s.solve(b)
+    s.set_wait_limit(0, True)
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    s.solve(b)
+    torch.cuda.synchronize()
+    waited = time.perf_counter() - t0
+    assert s.status()[0] == 6  # PISP_ERR_TIMEOUT
+    s.close()
+    assert 0.05 < waited < 2.5
