@@ -371,6 +371,8 @@ int build_persistent_factor(pisp_handle* h, int precision, int32_t K) {
 // solve classes.
 int build_plans(pisp_handle* h, int precision) {
   const pisp::Symbolic& S = h->sym;
+  h->plan_precision = 0;  // until all of it is in place
+  h->units_K = h->units_R = 0;
   h->plans.assign(S.n_levels, pisp::LevelPlan());
   h->h_small.clear();
   h->h_big.clear();
@@ -498,7 +500,6 @@ int build_plans(pisp_handle* h, int precision) {
     for (const auto& lp : h->plans) h->fac_bytes += lp.bytes_fsmall + lp.bytes_fbig;
   }
   h->plan_precision = precision;
-  h->units_K = h->units_R = 0;
   return PISP_OK;
 }
 
@@ -612,6 +613,7 @@ int build_unit_list(pisp_handle* h, int32_t K, int32_t R, const std::vector<int3
 }
 
 int build_units(pisp_handle* h, int32_t K, int32_t R) {
+  h->units_K = h->units_R = 0;  // until all of it is in place
   const pisp::Symbolic& S = h->sym;
   const size_t nS = S.sn.size();
   // parents have larger numbers than their children
@@ -1468,6 +1470,9 @@ int pisp_solve(pisp_handle* h, const double* b, int32_t R, const double* w, doub
   DeviceScope dev_scope_;
   TRY(set_device(h, dev_scope_));
   TRY(set_weights(h, w, h->w_last));
+  // from here on the kept solutions go, and with more right-hand sides than fit
+  // the workspace too: until this solve is queued nothing may be made of them
+  h->solved = false;
   TRY(ensure_solve_buffers(h, R));
   const pisp::Shifts sh = make_shifts(h, h->w_last);
   TRY(solve_core(h, b, h->X.as<double>(), R, sweeps, sh));

@@ -166,3 +166,39 @@ def test_default_wait_limit_is_a_few_tenths_of_a_second():
     assert s.status()[0] == 6  # PISP_ERR_TIMEOUT
     s.close()
     assert 0.05 < waited < 2.5
+
+
+@pytest.mark.gpu
+def test_solve_that_cannot_be_set_up_leaves_nothing_to_differentiate():
+    """A solve whose workspace does not fit the card (front vectors of 2^21 right-hand
+    sides and 16 shifts) has given up the workspace of the solve before it: combining
+    or differentiating that one is refused, and the next solve is correct."""
+    import torch
+    import paper_2311_11833_gb300 as pisp
+    from paper_2311_11833_gb300._lib import PispError
+    inst = pfgen.make_instance("plain")
+    t = pfgen.symmetric_shifts(16, 1e-3)
+    b, g = pfgen.rhs(inst.n, 3, 5), pfgen.rhs(inst.n, 3, 6)
+    s = pisp.Solver(inst.n, inst.row_ptr, inst.col)
+    c0, c1, ms = s.supernodes()[:3]
+    R = 1 << 21
+    assert 16 * R * 8 * int((c1 - c0 + ms).sum()) > torch.cuda.get_device_properties(0).total_memory
+    s.factor(_dev(inst.val), _dev(inst.D), t, "fp64")
+    s.solve(_dev(b))
+    wide = torch.zeros((inst.n, R), dtype=torch.float64, device="cuda")
+    with pytest.raises(PispError, match="OOM"):
+        s.solve(wide)
+    del wide
+    torch.cuda.empty_cache()
+    with pytest.raises(PispError, match="NOT_FACTORED"):
+        s.adjoint(_dev(g))
+    with pytest.raises(PispError, match="NOT_FACTORED"):
+        s.combine()
+    x = s.solve(_dev(b)).cpu().numpy()
+    gb = s.adjoint(_dev(g))[0].cpu().numpy()
+    assert s.status()[0] == 0
+    s.close()
+    A = oracle.to_scipy(inst)
+    scale = float(sum(abs(w) for w in oracle.weights(t)))
+    assert entrywise_err(x, oracle.x_hat(A, inst.D, t, b)) <= TOL * scale
+    assert entrywise_err(gb, oracle.adjoint(A, inst.D, t, b, g)[0]) <= TOL * scale
