@@ -258,31 +258,54 @@ int upload(pisp_handle* h, Buf& b, const std::vector<T>& v) {
     if (rc_) return rc_;  \
   } while (0)
 
-constexpr int64_t kManyTasks = 8192;  // (front, shift) pairs beyond which a factorisation has work for every SM
-
-// Factor path of a front of size F > 64: 0 = one CTA with the front in shared
-// memory, C >= 1 = a cluster of C CTAs (distributed shared memory), -1 = the
-// blocked global-memory path.  Policy 0 (default): one CTA while the front
-// fits, else the global path.  Policy 1: clusters wherever the front fits in
-// at most 8 CTAs' shared memory.
+// Level by level, the path of a front of size F > 64: 0 = one CTA with the front in
+// shared memory, C >= 1 = a cluster of C CTAs (distributed shared memory), -1 = the
+// global-memory path.  Policy 1: clusters wherever the front fits in at most 8 CTAs'
+// shared memory; the others: one CTA while the front fits.
 int factor_path(const pisp_handle* h, int F, int precision) {
   if (h->factor_policy == 1) return pisp::front_cluster_size(F, precision);
   return F <= pisp::small_front_limit(precision) ? 0 : -1;
 }
 
+// Routing of policy 0, by (front, shift) pairs: beyond kManyTasks a factorisation
+// has work for every SM.
+constexpr int64_t kManyTasks = 8192;
+
+// CTAs of the one-launch factorisation that an SM holds (at most 3) beside the
+// shared memory of the owner tiles, which grows with the widest front in FP32.
+int tile_ctas(const pisp_handle* h, int precision) {
+  const int F = h->sym.max_front;
+  if (F <= pisp::persistent_cta_front_limit(precision)) return 3;
+  const size_t smem = pisp::factor_persistent_smem(precision, pisp::owner_chunk_rows(precision, F, h->factor_tc), true, 0) +
+                      (precision == PISP_FP32 && h->factor_tc ? pisp::tc_staging_bytes() : 0);
+  return (int)std::min<size_t>(3, 228 * 1024 / (smem + 1536));  // an SM's, and what a CTA takes beside
+}
+
 // Whether the factorisation is one persistent launch: under policy 4, and under
-// policy 0 by what was measured (us level by level / in one launch).  In FP32 it
+// policy 0 by what was measured (us level by level / in one launch, K 4).  In FP32 it
 // saves the launches and the waits between levels and size classes: 1354 buses
 // 344 / 245, 777 buses 230 / 191, 5 grids 280 / 192, 64 grids 1784 / 897; with a
 // root of 1596 rows the owner tiles are all that counts, and those alone on an SM
-// with 255 registers a thread are ahead (10000 buses 2635 / 2999).  In FP64 one
-// grid's fronts are bound by the FP64 pipe whichever way they are launched (118
-// buses 110 / 129, 300 buses 164 / 164, 1354 buses 573 / 567); many grids' fronts
-// fill the SMs (48 grids 3939 / 2470).
+// with 255 registers a thread are ahead (10000 buses 1671 / 1786).  The owner tiles'
+// shared memory bounds the CTAs an SM holds for all the other fronts too, so a batch
+// with one wide front goes level by level from some number of pairs on.  With room
+// for three CTAs one launch was ahead or even wherever it was measured (150 grids of
+// 200 buses and one of 3000, 55 k pairs: 600 / 521; 600 and one, 206 k: 935 / 880).
+// For two, the other grids decide (one of 5000 buses, with 150 of 200 buses, 58 k:
+// 855 / 771; with 100 of 1000, 170 k: 1907 / 1574; with 600 of 200, 210 k: 1134 /
+// 1323; with 1500, 513 k: 1694 / 2513).  For one, few pairs do (one of 6000 buses:
+// 10 k 919 / 897; with 150 of 200 buses, 59 k: 1008 / 1066; with 600, 211 k: 1244 /
+// 2043; with 100 of 1000, 171 k: 1941 / 2510).
+// In FP64 tiles are small.  One grid's fronts are bound by the FP64 pipe whichever
+// way they are launched (300 buses 164 / 164, 1354 buses 573 / 567; 118 buses 110 /
+// 129, of which 22 are the segments that the one-launch form takes for fronts of at
+// most 32 rows); many grids' fronts fill the SMs (48 grids 3939 / 2470).
 bool one_launch(const pisp_handle* h, int precision, int32_t K) {
   if (h->factor_policy != 0) return h->factor_policy == 4;
   const int64_t tasks = (int64_t)h->sym.sn.size() * K;
-  return precision == PISP_FP32 ? h->sym.max_front <= 1024 : tasks >= kManyTasks;
+  if (precision != PISP_FP32) return tasks >= kManyTasks;
+  const int room = tile_ctas(h, precision);
+  return h->sym.max_front <= 1024 && tasks < (room >= 3 ? INT64_MAX : room == 2 ? 24 * kManyTasks : 4 * kManyTasks);
 }
 
 // Task list of the one-launch factorisation (one_launch): per level,
@@ -296,9 +319,11 @@ int build_persistent_factor(pisp_handle* h, int precision, int32_t K) {
   h->fac_ctas = h->factor_ctas;
   if (h->factor_policy == 0) {
     // many fronts: three CTAs an SM with the fronts that three can hold (64 grids
-    // 871 us, 994 with two; 48 grids in FP64 1914, 2173 with two); few: two, the
-    // registers are worth more (2000 buses 341 us, 364 with three)
-    const bool three = (int64_t)S.sn.size() * K >= kManyTasks;
+    // 871 us, 994 with two; 48 grids in FP64 1914, 2173 with two); few fronts, or
+    // tiles that leave no room for three: two, the registers are worth more (2000
+    // buses 341 us, 364 with three; 6000 buses 749, 887 with three; 150 grids of 200
+    // buses and one of 5000: 771, 850 with three)
+    const bool three = (int64_t)S.sn.size() * K >= kManyTasks && tile_ctas(h, precision) >= 3;
     smem_maxF = three ? (precision == PISP_FP32 ? 128 : 64) : 0;
     h->fac_ctas = three ? 3 : 2;
   }

@@ -2435,6 +2435,8 @@ size_t factor_persistent_smem(int precision, int CH, bool has_owner, int maxCtaF
   return (e * es + 127) / 128 * 128;  // what follows it (the tensor-core staging) stays aligned
 }
 
+size_t tc_staging_bytes() { return (size_t)kTcSmemFloats * sizeof(float); }
+
 int launch_factor_persistent(int precision, const SymDev& sd, const FactorTask* tasks, int ntasks, int* ticket,
                              int* fdone, const int* need, int* flags, int* err, const int32_t* wlist,
                              const double* vals, const double* D, const Shifts& sh, void* fronts,

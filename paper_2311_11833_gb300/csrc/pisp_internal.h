@@ -193,6 +193,7 @@ int launch_factor_persistent(int precision, const SymDev& sd, const FactorTask* 
 // owner tiles), and its dynamic shared memory per CTA
 int persistent_cta_front_limit(int precision);
 size_t factor_persistent_smem(int precision, int CH, bool has_owner, int maxCtaF);
+size_t tc_staging_bytes();  // more of it for the tensor-core form
 // largest front the tile-DAG path takes (its panel must fit in shared memory)
 int max_dag_front(int precision);
 // rows per owner tile for a level whose widest front is maxF (tc != 0: leave
