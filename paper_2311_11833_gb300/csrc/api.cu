@@ -7,6 +7,7 @@
 #include <climits>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <stdexcept>
 #include <string>
@@ -84,6 +85,8 @@ struct pisp_handle {
   int32_t loop_kernels = 0;     // kernels per iteration of that loop
   cudaStream_t body_stream = nullptr;  // captures the loop's body
   std::vector<double> inst_w;  // solve work of each instance (front entries)
+  // supernodes by level, and by instance, the widest fronts of each first
+  std::vector<int32_t> by_level, by_inst;
   Buf rng_f, rng_b, units_fc, units_bc, ucount, r_act, r_pre, r_dmax, r_xmax, r_prevd, r_nsw, d_inst_off;
   Buf r_nact, r_ai, r_arow, r_ccnt, r_sweep;
   // bounded waits of the persistent solves: polls before giving up (0 = the
@@ -238,18 +241,37 @@ int set_device(pisp_handle* h, DeviceScope& scope) {
 // freed afterwards.  While the stream is being captured the copy is not to become
 // part of the graph.
 template <typename T>
-int upload(pisp_handle* h, Buf& b, const std::vector<T>& v) {
-  if (!b.ensure(v.size() * sizeof(T))) return fail(h, PISP_ERR_OOM, "device allocation failed");
-  if (v.empty()) return PISP_OK;
+int upload(pisp_handle* h, Buf& b, const T* v, size_t n) {
+  if (!b.ensure(n * sizeof(T))) return fail(h, PISP_ERR_OOM, "device allocation failed");
+  if (n == 0) return PISP_OK;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   CK(cudaStreamIsCapturing(h->stream, &cs));
   if (cs != cudaStreamCaptureStatusNone) {
-    CK(cudaMemcpy(b.p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(b.p, v, n * sizeof(T), cudaMemcpyHostToDevice));
     return PISP_OK;
   }
-  CK(cudaMemcpyAsync(b.p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, h->stream));
+  CK(cudaMemcpyAsync(b.p, v, n * sizeof(T), cudaMemcpyHostToDevice, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   return PISP_OK;
+}
+template <typename T>
+int upload(pisp_handle* h, Buf& b, const std::vector<T>& v) {
+  return upload(h, b, v.data(), v.size());
+}
+
+// The schedules are built inside the first factorisation and the first solve of a
+// pattern (and when K, the precision or R change), so they cost a user with one
+// pattern a call what they cost: linear passes over the supernodes, no sorts.
+// list stably sorted by key in [0, n); start[v] = the first entry of key v, start[n]
+// their number.
+template <typename Key>
+std::vector<int32_t> sorted_by(const std::vector<int32_t>& list, size_t n, std::vector<int32_t>& start, Key key) {
+  std::vector<int32_t> at(n + 1, 0), out(list.size());
+  for (int32_t s : list) ++at[key(s) + 1];
+  for (size_t v = 0; v < n; ++v) at[v + 1] += at[v];
+  start = at;
+  for (int32_t s : list) out[at[key(s)]++] = s;
+  return out;
 }
 
 #define TRY(x)            \
@@ -339,16 +361,11 @@ int build_persistent_factor(pisp_handle* h, int precision, int32_t K) {
   std::vector<int32_t> wl, ntask(S.sn.size(), 1);  // tasks per (front, k)
   int64_t nflags = 0;
   for (int l = 0; l < S.n_levels; ++l) {
-    std::vector<int32_t> lst(S.level_sn.begin() + S.level_off[l], S.level_sn.begin() + S.level_off[l + 1]);
-    std::sort(lst.begin(), lst.end(), [&](int32_t a, int32_t b) {
-      const int fa = S.sn[a].F(), fb = S.sn[b].F();
-      return fa != fb ? fa > fb : a < b;
-    });
-    std::vector<int32_t> big, cta, seg[3];
-    for (int32_t sn : lst) {
-      const int F = S.sn[sn].F();
-      (F > Fc ? big : (F > 32 ? cta : seg[F > 16 ? 2 : (F > 8 ? 1 : 0)])).push_back(sn);
-    }
+    // the level's fronts from the widest down: owner tiles, CTAs, segments
+    const auto at = h->by_level.begin() + S.level_off[l], end = h->by_level.begin() + S.level_off[l + 1];
+    auto past = [&](auto from, int F) { return std::find_if(from, end, [&](int32_t q) { return S.sn[q].F() <= F; }); };
+    const auto cta = past(at, Fc), seg32 = past(cta, 32), seg16 = past(seg32, 16), seg8 = past(seg16, 8);
+    const std::vector<int32_t> big(at, cta);
     if (!big.empty()) {
       std::vector<pisp::BigFrontHost> bh;
       for (int32_t sn : big) bh.push_back({S.sn[sn].F(), S.sn[sn].ns()});
@@ -362,14 +379,14 @@ int build_persistent_factor(pisp_handle* h, int precision, int32_t K) {
       nflags += nfl;
       if (nflags >= INT32_MAX) return fail(h, PISP_ERR_UNSUPPORTED, "too many factor flags");
     }
-    for (int32_t sn : cta)
-      for (int k = 0; k < K; ++k) ft.push_back({pisp::kFacCta, sn, k, 0, 0, 0});
+    for (auto q = cta; q != seg32; ++q)
+      for (int k = 0; k < K; ++k) ft.push_back({pisp::kFacCta, *q, k, 0, 0, 0});
     for (int w = 2; w >= 0; --w) {
-      if (seg[w].empty()) continue;
-      const int64_t off = (int64_t)wl.size(), tasks = (int64_t)seg[w].size() * K;
-      if (off + (int64_t)seg[w].size() >= INT32_MAX || tasks >= INT32_MAX)
+      const auto from = w == 2 ? seg32 : (w == 1 ? seg16 : seg8), to = w == 2 ? seg16 : (w == 1 ? seg8 : end);
+      const int64_t off = (int64_t)wl.size(), tasks = (to - from) * K;
+      if (off + (to - from) >= INT32_MAX || tasks >= INT32_MAX)
         return fail(h, PISP_ERR_UNSUPPORTED, "too many factor tasks");
-      wl.insert(wl.end(), seg[w].begin(), seg[w].end());
+      wl.insert(wl.end(), from, to);
       for (int64_t b = 0; b < tasks; b += 256 / (8 << w))
         ft.push_back({pisp::kFacSeg8 + w, (int32_t)off, 0, (int32_t)b, (int32_t)tasks, 0});
     }
@@ -391,89 +408,88 @@ int build_persistent_factor(pisp_handle* h, int precision, int32_t K) {
   return PISP_OK;
 }
 
-// Groups the supernodes of every level by front size: small fronts into
-// shared-memory classes, big fronts into the blocked path, and all fronts into
-// solve classes.
+// The factorisation's schedule: one launch (build_persistent_factor), or level by
+// level, its fronts grouped by size: fronts factored in shared memory into classes,
+// wider ones into the global-memory paths.  Either way the algorithmic bytes per
+// level and perturbation: what each kernel family must read and write at least
+// (values, indices, factor entries, vectors).
 int build_plans(pisp_handle* h, int precision) {
   const pisp::Symbolic& S = h->sym;
   h->plan_precision = 0;  // until all of it is in place
   h->units_K = h->units_R = 0;
   h->plans.assign(S.n_levels, pisp::LevelPlan());
+  auto path = [&](int F) { return F > 64 ? factor_path(h, F, precision) : 0; };
+  const double p = (double)esize(precision);
+  for (const pisp::Supernode& sn : S.sn) {
+    pisp::LevelPlan& lp = h->plans[sn.level];
+    const size_t s = &sn - S.sn.data();
+    const double F = sn.F(), ns = sn.ns(), ms = sn.ms;
+    const double amap = (double)(S.amap_off[s + 1] - S.amap_off[s]);
+    const double fac = amap * 16 + ns * 12 + F * F * p;
+    if (path(sn.F()) < 0) lp.bytes_fbig += fac + 2 * F * F * p;
+    else lp.bytes_fsmall += fac;
+    lp.bytes_fwd_a += ns * 4 + (ns * F - ns * (ns + 1) / 2) * p;
+    lp.bytes_fwd_b += ns * 8 + F * p;
+    lp.bytes_bwd_a += ms * 4 + (ns * (ns + 1) / 2 + ns * ms) * p;
+    lp.bytes_bwd_b += ms * 8 + ns * p + ns * 8;
+    if (sn.parent < 0) continue;
+    // as a child of its parent
+    const pisp::Supernode& up = S.sn[sn.parent];
+    pisp::LevelPlan& lq = h->plans[up.level];
+    (path(up.F()) < 0 ? lq.bytes_fbig : lq.bytes_fsmall) += ms * ms * p + ms * 4;
+    lq.bytes_fwd_a += ms * 4;
+    lq.bytes_fwd_b += ms * p;
+  }
+  h->fac_single = one_launch(h, precision, h->K_hint);
+  if (h->fac_single) {
+    TRY(build_persistent_factor(h, precision, h->K_hint));
+    h->fac_bytes = 0;
+    for (const auto& lp : h->plans) h->fac_bytes += lp.bytes_fsmall + lp.bytes_fbig;
+    h->plan_precision = precision;
+    return PISP_OK;
+  }
   h->h_small.clear();
   h->h_big.clear();
   h->h_bigF.clear();
   h->h_dag.clear();
   h->dag_max_flags = 0;
-  const bool single = one_launch(h, precision, h->K_hint);
   for (int l = 0; l < S.n_levels; ++l) {
     pisp::LevelPlan& lp = h->plans[l];
-    std::vector<int32_t> lst(S.level_sn.begin() + S.level_off[l],
-                             S.level_sn.begin() + S.level_off[l + 1]);
-    std::sort(lst.begin(), lst.end(), [&](int32_t a, int32_t b) {
-      const int fa = S.sn[a].F(), fb = S.sn[b].F();
-      return fa != fb ? fa < fb : a < b;
-    });
-    // on-chip fronts: segment classes up to 32 (one class of CTAs in FP64),
-    // single-CTA classes up to 64, then clusters of 1..8 CTAs
-    const int fcls[4] = {8, 16, 32, 64};
-    int lo = 0;
-    for (int c = precision == PISP_FP32 ? 0 : 2; c < 4; ++c) {
-      pisp::LevelPlan::Group G{(int64_t)h->h_small.size(), 0, 0, 0};
-      for (int32_t s : lst) {
-        const int F = S.sn[s].F();
-        if (F > lo && F <= fcls[c]) {
-          h->h_small.push_back(s);
-          ++G.count;
-          G.maxF = std::max(G.maxF, F);
-        }
-      }
-      if (G.count) lp.groups[lp.n_groups++] = G;
-      lo = fcls[c];
-    }
-    // fronts above 64: the factor path of each front (single CTA in shared
-    // memory, a cluster of C CTAs in distributed shared memory, or the blocked
-    // global-memory path) comes from the handle's factor policy
-    auto path = [&](int F) { return factor_path(h, F, precision); };
-    for (int C = 1; C <= 8; C *= 2) {
-      pisp::LevelPlan::Group G{(int64_t)h->h_small.size(), 0, 0, C};
-      for (int32_t s : lst) {
-        const int F = S.sn[s].F();
-        if (F > 64 && path(F) == C) {
-          h->h_small.push_back(s);
-          ++G.count;
-          G.maxF = std::max(G.maxF, F);
-        }
-      }
-      if (G.count) lp.groups[lp.n_groups++] = G;
-    }
-    {
-      pisp::LevelPlan::Group G{(int64_t)h->h_small.size(), 0, 0, 0};
-      for (int32_t s : lst) {
-        const int F = S.sn[s].F();
-        if (F > 64 && path(F) == 0) {
-          h->h_small.push_back(s);
-          ++G.count;
-          G.maxF = std::max(G.maxF, F);
-        }
-      }
-      if (G.count) lp.groups[lp.n_groups++] = G;
-    }
     lp.big_off = (int64_t)h->h_big.size();
-    for (int32_t s : lst) {
-      const int F = S.sn[s].F();
-      if (F > 64 && path(F) < 0) {
-        h->h_big.push_back(s);
-        h->h_bigF.push_back({F, S.sn[s].ns()});
-        ++lp.big_count;
-        lp.big_maxF = std::max(lp.big_maxF, F);
-        lp.big_maxns = std::max(lp.big_maxns, S.sn[s].ns());
+    // from the narrowest front up, in the order of their numbers among equals
+    int last = 0;
+    for (int64_t hi = S.level_off[l + 1]; hi > S.level_off[l];) {
+      int64_t lo = hi - 1;
+      const int F = S.sn[h->by_level[lo]].F();
+      while (lo > S.level_off[l] && S.sn[h->by_level[lo - 1]].F() == F) --lo;
+      const int C = path(F);
+      if (C < 0) {
+        for (int64_t q = lo; q < hi; ++q) {
+          const int32_t s = h->by_level[q];
+          h->h_big.push_back(s);
+          h->h_bigF.push_back({F, S.sn[s].ns()});
+          lp.big_maxns = std::max(lp.big_maxns, S.sn[s].ns());
+        }
+        lp.big_count += (int32_t)(hi - lo);
+        lp.big_maxF = F;
+      } else {
+        // on-chip fronts: segment classes up to 32 (one class of CTAs in FP64), a
+        // class of CTAs up to 64, then clusters of 1..8 CTAs or single CTAs
+        const int cls = F > 64 ? 100 + C : F > 32 ? 64 : precision != PISP_FP32 ? 32 : F > 16 ? 32 : F > 8 ? 16 : 8;
+        if (cls != last) lp.groups[lp.n_groups++] = {(int64_t)h->h_small.size(), 0, 0, C};
+        last = cls;
+        pisp::LevelPlan::Group& G = lp.groups[lp.n_groups - 1];
+        h->h_small.insert(h->h_small.end(), h->by_level.begin() + lo, h->by_level.begin() + hi);
+        G.count += (int32_t)(hi - lo);
+        G.maxF = F;
       }
+      hi = lo;
     }
     // big fronts as one persistent launch per level: owner tiles (policy 0,
     // any front size) or the tile DAG (policy 2, while a panel fits in shared
     // memory); else (and under policies 1 and 3) one panel launch and one
     // update launch per 32 pivots
-    const bool owner = h->factor_policy == 0 && !single;
+    const bool owner = h->factor_policy == 0;
     const bool dag = h->factor_policy == 2 && lp.big_maxF <= pisp::max_dag_front(precision);
     if (lp.big_count > 0 && (owner || dag)) {
       std::vector<pisp::DagTask> tk;
@@ -491,39 +507,12 @@ int build_plans(pisp_handle* h, int precision) {
       h->h_dag.insert(h->h_dag.end(), tk.begin(), tk.end());
       h->dag_max_flags = std::max(h->dag_max_flags, nfl);
     }
-    // algorithmic bytes per perturbation: what each kernel family must read
-    // and write at least (values, indices, factor entries, vectors)
-    const double p = (double)esize(precision);
-    for (int32_t s : lst) {
-      const pisp::Supernode& sn = S.sn[s];
-      const double F = sn.F(), ns = sn.ns(), ms = sn.ms;
-      double child = 0, childv = 0;
-      for (int64_t q = S.child_off[s]; q < S.child_off[s + 1]; ++q) {
-        const double cms = S.sn[S.child[q]].ms;
-        child += cms * cms * p + cms * 4;
-        childv += cms;
-      }
-      const double amap = (double)(S.amap_off[s + 1] - S.amap_off[s]);
-      const double fac = amap * 16 + ns * 12 + child + F * F * p;
-      if (sn.F() > 64 && path(sn.F()) < 0) lp.bytes_fbig += fac + 2 * F * F * p;
-      else lp.bytes_fsmall += fac;
-      lp.bytes_fwd_a += ns * 4 + childv * 4 + (ns * F - ns * (ns + 1) / 2) * p;
-      lp.bytes_fwd_b += ns * 8 + childv * p + F * p;
-      lp.bytes_bwd_a += ms * 4 + (ns * (ns + 1) / 2 + ns * ms) * p;
-      lp.bytes_bwd_b += ms * 8 + ns * p + ns * 8;
-    }
   }
   TRY(upload(h, h->d_small, h->h_small));
   TRY(upload(h, h->d_big, h->h_big));
   TRY(upload(h, h->d_dag, h->h_dag));
   if (!h->dag_ticket.ensure(sizeof(int)) || !h->dag_flags.ensure((size_t)h->dag_max_flags * sizeof(int)))
     return fail(h, PISP_ERR_OOM, "device allocation failed (factor schedule)");
-  h->fac_single = single;
-  if (single) {
-    TRY(build_persistent_factor(h, precision, h->K_hint));
-    h->fac_bytes = 0;
-    for (const auto& lp : h->plans) h->fac_bytes += lp.bytes_fsmall + lp.bytes_fbig;
-  }
   h->plan_precision = precision;
   return PISP_OK;
 }
@@ -556,7 +545,7 @@ struct UnitList {
 };
 
 // tasks[s]: tasks of front s per completion counter
-int build_unit_list(pisp_handle* h, int32_t K, int32_t R, const std::vector<int32_t>& stage,
+int build_unit_list(pisp_handle* h, int32_t K, int32_t R, const std::vector<int32_t>& stage, int32_t stages,
                     const std::vector<int32_t>& left, bool fwd, std::vector<int32_t>& tasks, int32_t& wide,
                     UnitList& out) {
   const pisp::Symbolic& S = h->sym;
@@ -564,24 +553,25 @@ int build_unit_list(pisp_handle* h, int32_t K, int32_t R, const std::vector<int3
   const bool cols = !fwd && R > 1;
   const int kf = std::max(1, std::min(h->kfuse, (int)K));
   const int rchunks = R == 1 ? 1 : (R + pisp::kSolveChunk - 1) / pisp::kSolveChunk;
-  std::vector<std::vector<int32_t>> at;
-  for (size_t q = 0; q < S.sn.size(); ++q) {
-    if ((size_t)stage[q] >= at.size()) at.resize(stage[q] + 1);
-    at[stage[q]].push_back((int32_t)q);
-  }
+  // by stage, within it by instance and from the widest front down
+  std::vector<int32_t> at;
+  const std::vector<int32_t> lst = sorted_by(h->by_inst, stages, at, [&](int32_t q) { return stage[q]; });
   out.order.reserve(S.sn.size());
   auto cta_unit = [&](int32_t sn, const pisp::SolveUnit& u) {
     out.units.push_back(u);
     out.rng.push_back(S.sn[sn].instance);
     out.rng.push_back(S.sn[sn].instance);
   };
-  for (auto& lst : at) {
+  std::vector<int32_t> cta, seg[4];  // segments of 8, 16, 32 lanes; warps
+  for (int32_t st = 0; st < stages; ++st) {
     out.start.push_back((int32_t)out.units.size());
-    std::vector<int32_t> cta, seg[4];  // segments of 8, 16, 32 lanes; warps
+    cta.clear();
+    for (auto& g : seg) g.clear();
     auto wide_rows = [&](int32_t sn) {  // tasks of 256 rows
       return ((fwd ? S.sn[sn].F() : S.sn[sn].ns()) + pisp::kWideUnitRows - 1) / pisp::kWideUnitRows;
     };
-    for (int32_t sn : lst) {
+    for (int32_t e = at[st]; e < at[st + 1]; ++e) {
+      const int32_t sn = lst[e];
       const int F = S.sn[sn].F(), ns = S.sn[sn].ns();
       if (ns > 32 || F > std::max(32, h->warp_maxF)) cta.push_back(sn);
       else seg[cols ? 3 : (F > 16 ? 2 : (F > 8 ? 1 : 0))].push_back(sn);
@@ -616,11 +606,6 @@ int build_unit_list(pisp_handle* h, int32_t K, int32_t R, const std::vector<int3
       const int kind = w == 3 ? pisp::kUnitCol : (w == 2 ? pisp::kUnitSeg32 : (w == 1 ? pisp::kUnitSeg16 : pisp::kUnitSeg8));
       const int per_unit = w == 3 ? 8 : 256 / (8 << w);
       const int64_t per_front = w == 3 ? NG : (int64_t)((K + kf - 1) / kf) * rchunks;
-      std::sort(g.begin(), g.end(), [&](int32_t a, int32_t b) {
-        if (S.sn[a].instance != S.sn[b].instance) return S.sn[a].instance < S.sn[b].instance;
-        const int fa = S.sn[a].F(), fb = S.sn[b].F();
-        return fa != fb ? fa > fb : a < b;
-      });
       const int32_t off = (int32_t)out.order.size();
       const int64_t n = (int64_t)g.size() * per_front;
       if (n >= INT32_MAX) return fail(h, PISP_ERR_UNSUPPORTED, "too many solve tasks");
@@ -644,13 +629,16 @@ int build_units(pisp_handle* h, int32_t K, int32_t R) {
   // parents have larger numbers than their children
   std::vector<int32_t> height(nS), depth(nS, 0);
   for (size_t q = 0; q < nS; ++q) height[q] = S.sn[q].level;
-  for (size_t q = nS; q-- > 0;)
+  int32_t deepest = -1;
+  for (size_t q = nS; q-- > 0;) {
     if (S.sn[q].parent >= 0) depth[q] = depth[S.sn[q].parent] + 1;
+    deepest = std::max(deepest, depth[q]);
+  }
   UnitList f, b;
   std::vector<int32_t> nf(nS, 1), nb(nS, 1);
   int32_t wide = 0;
-  TRY(build_unit_list(h, K, R, height, depth, true, nf, wide, f));
-  TRY(build_unit_list(h, K, R, depth, height, false, nb, wide, b));
+  TRY(build_unit_list(h, K, R, height, S.n_levels, depth, true, nf, wide, f));
+  TRY(build_unit_list(h, K, R, depth, deepest + 1, height, false, nb, wide, b));
   // completion targets: forward, every task of a front's children; backward,
   // every task of its parent, as the counters count them
   const int NG = std::max(counter_groups(h, K, R, true), counter_groups(h, K, R, false));
@@ -678,19 +666,26 @@ int build_units(pisp_handle* h, int32_t K, int32_t R) {
       nflags += (int64_t)K * R;
       if (nflags >= INT32_MAX) return fail(h, PISP_ERR_UNSUPPORTED, "too many solve tasks");
     }
-  std::vector<pisp::FrontDesc> desc(2 * nS);  // forward order, then backward order
-  for (size_t q = 0; q < 2 * nS; ++q) {
-    const int32_t sn = q < nS ? f.order[q] : b.order[q - nS];
-    const pisp::Supernode& n = S.sn[sn];
-    desc[q] = {n.c0, n.ns(), n.F(), n.instance, S.front_off[sn], S.vec_off[sn], n.row_off, n.parent, sn, need[sn],
-               n.parent >= 0 ? nb[n.parent] : 0, flag[sn],
-               (whole(sn) ? pisp::kSelfWhole : 0) | (n.parent >= 0 && whole(n.parent) ? pisp::kParentWhole : 0)};
+  // the records, forward order, then backward order; read in the fronts' own order
+  std::unique_ptr<pisp::FrontDesc[]> desc(new pisp::FrontDesc[2 * nS]);
+  std::vector<int32_t> at_f(nS), at_b(nS);
+  for (size_t q = 0; q < nS; ++q) {
+    at_f[f.order[q]] = (int32_t)q;
+    at_b[b.order[q]] = (int32_t)q;
+  }
+  for (size_t q = 0; q < nS; ++q) {
+    const int32_t sn = (int32_t)q;
+    const pisp::Supernode& n = S.sn[q];
+    desc[at_f[q]] = desc[nS + at_b[q]] = {
+        n.c0, n.ns(), n.F(), n.instance, S.front_off[q], S.vec_off[q], n.row_off, n.parent, sn, need[q],
+        n.parent >= 0 ? nb[n.parent] : 0, flag[q],
+        (whole(sn) ? pisp::kSelfWhole : 0) | (n.parent >= 0 && whole(n.parent) ? pisp::kParentWhole : 0)};
   }
   TRY(upload(h, h->units_f, f.units));
   TRY(upload(h, h->units_b, b.units));
   TRY(upload(h, h->rng_f, f.rng));
   TRY(upload(h, h->rng_b, b.rng));
-  TRY(upload(h, h->desc, desc));
+  TRY(upload(h, h->desc, desc.get(), 2 * nS));
   if (!h->units_fc.ensure(f.units.size() * sizeof(pisp::SolveUnit)) ||
       !h->units_bc.ensure(b.units.size() * sizeof(pisp::SolveUnit)) || !h->ucount.ensure(2 * sizeof(int32_t)) ||
       !h->serr.ensure(sizeof(int)) || !h->ctr.ensure(2 * (f.start.size() + b.start.size() + 8 + (nS * (size_t)NG + (size_t)nflags) * pisp::kCtrStride) * sizeof(int)))
@@ -1235,6 +1230,13 @@ int analyze_impl(pisp_handle* h, int32_t G, const int32_t* n, const int64_t* row
   TRY(upload(h, h->d_inst_off, S.inst_off));
   h->inst_w.assign(G, 0.0);
   for (int s = 0; s < nS; ++s) h->inst_w[S.sn[s].instance] += (double)S.sn[s].F() * S.sn[s].F();
+  {
+    std::vector<int32_t> order(nS), start;
+    for (int s = 0; s < nS; ++s) order[s] = s;
+    order = sorted_by(order, (size_t)S.max_front + 1, start, [&](int32_t s) { return S.max_front - S.sn[s].F(); });
+    h->by_level = sorted_by(order, S.n_levels, start, [&](int32_t s) { return S.sn[s].level; });
+    h->by_inst = sorted_by(order, G, start, [&](int32_t s) { return S.sn[s].instance; });
+  }
   TRY(upload(h, h->row_ptr, rp));
   TRY(upload(h, h->col, cl));
   TRY(upload(h, h->parent, par));
