@@ -274,6 +274,18 @@ std::vector<int32_t> sorted_by(const std::vector<int32_t>& list, size_t n, std::
   return out;
 }
 
+// Runs a step that allocates host memory: no C++ exception may cross the C boundary.
+template <typename Step>
+int no_throw(pisp_handle* h, Step step) {
+  try {
+    return step();
+  } catch (const std::bad_alloc&) {
+    return fail(h, PISP_ERR_OOM, "out of host memory");
+  } catch (const std::exception& e) {
+    return fail(h, PISP_ERR_INVALID_ARG, e.what());
+  }
+}
+
 #define TRY(x)            \
   do {                    \
     int rc_ = (x);        \
@@ -856,7 +868,7 @@ int solve_pass_t(pisp_handle* h, bool trans, const SolveIO& io, int32_t R, const
 // Adaptive sweeps (persistent schedule): act skips the fronts of instances
 // that have stopped and the compacted unit lists are walked.
 int solve_pass(pisp_handle* h, bool trans, const SolveIO& io, int32_t R, const uint8_t* act = nullptr) {
-  if (h->units_K != h->K || h->units_R != R) TRY(build_units(h, h->K, R));
+  if (h->units_K != h->K || h->units_R != R) TRY(no_throw(h, [&] { return build_units(h, h->K, R); }));
   return h->precision == PISP_FP32 ? solve_pass_t<float>(h, trans, io, R, act)
                                    : solve_pass_t<double>(h, trans, io, R, act);
 }
@@ -1320,17 +1332,7 @@ extern "C" {
 int pisp_analyze(pisp_handle* h, int32_t G, const int32_t* n, const int64_t* row_ptr,
                  const int32_t* col_idx, const pisp_options* opt) {
   if (!h) return fail(h, PISP_ERR_INVALID_ARG, "null handle");
-  // no C++ exception may cross the C boundary: host allocation failures of
-  // the analysis (or of its staging vectors) become error codes
-  try {
-    return analyze_impl(h, G, n, row_ptr, col_idx, opt);
-  } catch (const std::bad_alloc&) {
-    h->analyzed = false;
-    return fail(h, PISP_ERR_OOM, "out of host memory in pisp_analyze");
-  } catch (const std::exception& e) {
-    h->analyzed = false;
-    return fail(h, PISP_ERR_INVALID_ARG, std::string("pisp_analyze failed: ") + e.what());
-  }
+  return no_throw(h, [&] { return analyze_impl(h, G, n, row_ptr, col_idx, opt); });
 }
 
 int pisp_match_rows(int32_t n, const int64_t* row_ptr, const int32_t* col_idx, int32_t* row_perm) {
@@ -1390,7 +1392,7 @@ int pisp_factor_perturbed(pisp_handle* h, const double* values, const double* D,
   TRY(set_device(h, dev_scope_));
   h->factored = h->solved = false;
   h->K_hint = K;
-  if (h->plan_precision != precision || h->plan_K != K) TRY(build_plans(h, precision));
+  if (h->plan_precision != precision || h->plan_K != K) TRY(no_throw(h, [&] { return build_plans(h, precision); }));
   h->plan_K = K;
   h->K = K;
   h->precision = precision;
