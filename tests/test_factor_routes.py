@@ -45,3 +45,81 @@ def test_one_launch_or_level_by_level(n, ones, single):
         assert entrywise_err(x[:n], oracle.x_hat(oracle.to_scipy(I), I.D, t, b[:n])) <= TOL * scale
         want = sum(w * b[n:] / (a + tk * d)[:, None] for w, tk in zip(oracle.weights(t), t))
         assert (abs(x[n:] - want) <= TOL * scale * abs(want).max()).all()
+
+
+def _unit(precision):
+    return 2.0 ** -24 if precision == "fp32" else 2.0 ** -53
+
+
+# sizes of test_factor_shapes, which the default routing factors in one launch with FP32
+# factors, and the widest fronts of a CTA level by level (224 rows, FP64: 160)
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("policy", [2, 3])
+def test_dense_fronts_level_by_level(precision, policy):
+    import test_factor_shapes as shapes
+    ns = shapes.DENSE + (162, 191, 223, 224, 225)
+    insts = [pfgen.random_sparse(n, 1.0, seed=n, diag_boost=2.0 * np.sqrt(n)) for n in ns]
+    s, t, _ = shapes._factor(insts, 2, precision, factor_policy=policy)
+    assert s.stats()["gpu_launches"] > 1
+    perm, first = s.perm(), s.supernodes()[0].tolist()
+    r0 = 0
+    for I in insts:
+        p = perm[r0:r0 + I.n] - r0
+        A = oracle.to_scipy(I).toarray()
+        for k in range(2):
+            f = s.front(first.index(r0), k).astype(np.float64)
+            L, U = np.tril(f, -1) + np.eye(I.n), np.triu(f)
+            B = (A + t[k] * np.diag(I.D))[np.ix_(p, p)]
+            # the bound of test_factor_shapes: any order of summation
+            assert (abs(L @ U - B) <= (I.n + 6) * _unit(precision) * (abs(L) @ abs(U) + abs(B))).all(), (I.n, k)
+        r0 += I.n
+    s.close()
+
+
+@pytest.mark.parametrize("precision,sweeps", [("fp32", 4), ("fp64", 0)])
+def test_many_children_level_by_level(precision, sweeps):
+    import test_factor_shapes as shapes
+    shapes.test_many_children(precision, sweeps, 2)
+
+
+def _hub(hub, arms, seed):
+    """A dense hub and dense blocks tied to all of it: a front of (block + hub) rows each."""
+    r = np.random.default_rng(seed)
+    n = hub + sum(arms)
+    M = np.zeros((n, n))
+    M[:hub, :] = r.standard_normal((hub, n))
+    M[:, :hub] = r.standard_normal((n, hub))
+    at = hub
+    for a in arms:
+        M[at:at + a, at:at + a] = r.standard_normal((a, a))
+        at += a
+    M[np.arange(n), np.arange(n)] = 2.0 * np.sqrt(n) + abs(M[np.arange(n), np.arange(n)])
+    return sp.csr_matrix(M), r.uniform(0.5, 1.5, n)
+
+
+HUBS = [(120, (31, 65)), (250, (6, 40)), (480, (32, 64)), (1010, (33, 95))]
+
+
+@pytest.mark.parametrize("precision,sweeps,policy,hub,arms", [("fp64", 0, p, *h) for p in (0, 4) for h in HUBS] +
+                         [("fp32", 5, 0, *HUBS[-1])])
+def test_owner_tiles_by_themselves(precision, sweeps, policy, hub, arms):
+    """Owner tiles of FP64 factors, level by level and in one launch, and of FP32 factors
+    in launches of their own (fronts of more than 1024 rows)."""
+    import paper_2311_11833_gb300 as pisp
+    A, D = _hub(hub, arms, hub)
+    n = A.shape[0]
+    t = pfgen.symmetric_shifts(2, 1e-3)
+    s = pisp.Solver([n], A.indptr.astype(np.int64), A.indices.astype(np.int32), factor_policy=policy)
+    s.profile(True)
+    s.factor(_dev(A.data), _dev(D), t, precision)
+    s.profile_collect()
+    s.profile(False)
+    ran = {f for f, v in s.profile_read().items() if v["launches"]}
+    assert ("factor_persistent" in ran) == (policy == 4)
+    # level by level owner tiles take the fronts that a CTA's shared memory does not hold
+    assert policy == 4 or ("factor_big" in ran) == (s.stats()["max_front"] > (224 if precision == "fp32" else 160))
+    b = pfgen.rhs(n, 2, 1)
+    x = s.solve(_dev(b), sweeps=sweeps).cpu().numpy()
+    assert s.status()[0] == 0
+    s.close()
+    assert entrywise_err(x, oracle.x_hat(A, D, t, b)) <= TOL * float(sum(abs(w) for w in oracle.weights(t)))
