@@ -68,7 +68,6 @@ struct SymDev {
   const int64_t* row_ptr;    // [N+1] CSR of A (original order)
   const int32_t* col;        // [nnz]
   const int64_t* at_ptr;     // [N+1] CSC of A: entries of column j at at_ptr[j]..at_ptr[j+1]
-  const int32_t* at_row;     //   their rows
   const int32_t* at_src;     //   their CSR entry indices
   const int64_t* inv_pos;    // inverse extend-add map as positions: vec_off[child] + inv_col
   const int32_t* pcol;       // [nnz] permuted column of every CSR entry
@@ -207,7 +206,7 @@ int small_front_limit(int precision);
 int front_cluster_size(int F, int precision);
 // largest front the blocked path can take (its panel must fit in shared memory)
 int max_big_front(int precision);
-// largest front the solve kernels can take
+// widest front a solve takes
 int max_solve_front(int precision);
 
 // ---- solve (solve_persistent.h; solve.cu) ----
@@ -282,8 +281,9 @@ inline int32_t rhs_stride(int precision, int32_t R) {
 inline int32_t rhs_stride64(int32_t R) { return R == 1 ? 1 : (R + 1) / 2 * 2; }
 
 // One launch of the forward (L, or U^T with trans) or backward (U, L^T) solve;
-// ctas = resident CTAs per SM it is compiled for (2, 3, 4; <= 0: 3 for FP32,
-// 2 for FP64); wide = the largest chunk of a front with more than 32 pivots.  Returns the kernels launched or -1.
+// ctas = resident CTAs per SM it is compiled for with several right-hand sides
+// (2, 3, 4; <= 0, or transposed: 2); wide = the largest chunk of a front with more
+// than 32 pivots, 0 if there is none.  Returns the kernels launched or -1.
 template <typename T, bool FWD>
 int launch_solve_dir(bool trans, const SolveArgs<T>& a, int32_t nunits, int32_t wide, int32_t ctas, cudaStream_t st);
 // right-hand sides and rows of a task of a front with more than 32 pivots

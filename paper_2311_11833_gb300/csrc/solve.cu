@@ -19,7 +19,6 @@ namespace pisp {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kSolveSmem = 96 * 1024;  // one value per row of the widest front the solves take
 
 // x[perm[i]][r] = sum_k w_k X[i][k][r]   (Eq. x_star; FP64, k ascending)
 __global__ void k_combine(SymDev sd, const double* __restrict__ X, Shifts sh, int R, int RX,
@@ -450,7 +449,9 @@ unsigned sm_count() {
 
 }  // namespace
 
-int max_solve_front(int precision) { return kSolveSmem / (precision == PISP_FP32 ? 4 : 8); }
+// The kernels hold no vector of a whole front; these are the widths accepted when
+// they held one in 96 KB of shared memory, and no wider front has been run since.
+int max_solve_front(int precision) { return precision == PISP_FP32 ? 24576 : 12288; }
 
 int wide_chunk(int precision, int R) { return R == 1 ? 1 : (precision == PISP_FP32 ? 4 : 2); }
 
