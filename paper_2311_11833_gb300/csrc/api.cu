@@ -326,10 +326,11 @@ int tile_ctas(const pisp_handle* h, int precision) {
 // for three CTAs one launch was ahead or even wherever it was measured (150 grids of
 // 200 buses and one of 3000, 55 k pairs: 600 / 521; 600 and one, 206 k: 935 / 880).
 // For two, the other grids decide (one of 5000 buses, with 150 of 200 buses, 58 k:
-// 855 / 771; with 100 of 1000, 170 k: 1907 / 1574; with 600 of 200, 210 k: 1134 /
+// 855 / 784; with 100 of 1000, 170 k: 1907 / 1746; with 600 of 200, 210 k: 1134 /
 // 1323; with 1500, 513 k: 1694 / 2513).  For one, few pairs do (one of 6000 buses:
-// 10 k 919 / 897; with 150 of 200 buses, 59 k: 1008 / 1066; with 600, 211 k: 1244 /
-// 2043; with 100 of 1000, 171 k: 1941 / 2510).
+// 10 k 919 / 765; with 150 of 200 buses, 59 k: 1008 / 1066; with 600, 211 k: 1244 /
+// 2043; with 100 of 1000, 171 k: 1941 / 2510; the one-launch figures past the lines
+// are with fronts of up to 160 rows by CTAs).
 // In FP64 tiles are small.  One grid's fronts are bound by the FP64 pipe whichever
 // way they are launched (300 buses 164 / 164, 1354 buses 573 / 567; 118 buses 110 /
 // 129, of which 22 are the segments that the one-launch form takes for fronts of at
@@ -353,13 +354,13 @@ int build_persistent_factor(pisp_handle* h, int precision, int32_t K) {
   h->fac_ctas = h->factor_ctas;
   if (h->factor_policy == 0) {
     // many fronts: three CTAs an SM with the fronts that three can hold (64 grids
-    // 871 us, 994 with two; 48 grids in FP64 1914, 2173 with two); few fronts, or
-    // tiles that leave no room for three: two, the registers are worth more (2000
-    // buses 341 us, 364 with three; 6000 buses 749, 887 with three; 150 grids of 200
-    // buses and one of 5000: 771, 850 with three)
-    const bool three = (int64_t)S.sn.size() * K >= kManyTasks && tile_ctas(h, precision) >= 3;
-    smem_maxF = three ? (precision == PISP_FP32 ? 128 : 64) : 0;
-    h->fac_ctas = three ? 3 : 2;
+    // 871 us, 994 with two; 48 grids in FP64 1914, 2173 with two), but compiled for
+    // two, with more registers, where the tiles leave no room for three (one of 6000
+    // buses, K 8: 1051 us, 1182 compiled for three; 150 grids of 200 buses and one of
+    // 5000, K 4: 784, 851); few: two (2000 buses 341 us, 364 with three)
+    const bool many = (int64_t)S.sn.size() * K >= kManyTasks;
+    smem_maxF = many ? (precision == PISP_FP32 ? 128 : 64) : 0;
+    h->fac_ctas = many && tile_ctas(h, precision) >= 3 ? 3 : 2;
   }
   const int Fc = smem_maxF > 0 ? std::min(smem_maxF, pisp::persistent_cta_front_limit(precision))
                                : pisp::persistent_cta_front_limit(precision);
