@@ -335,12 +335,37 @@ __device__ __forceinline__ void front_lu(T* f, int ld, int F, int ns, T* rinv, c
   }
 }
 
-// The same in FP64, where the pipe (2 FMA a clock per SM) bounds the front and
-// every idle lane of an instruction costs as much as a busy one: one pivot at a
-// time, the trailing elements dealt out to the threads one by one, and one
-// barrier a pivot: warp 0 takes the next pivot's column first, inverts the
-// pivot and scales the column while the other warps update the rest (all warps
-// inverting it took as long as a 40-row front's update).
+// The same one pivot at a time: the column scaled by all threads, then the trailing
+// columns dealt out to the warps, two barriers a pivot.  The form of FP64, whose pipe
+// (2 FMA a clock per SM) gains nothing from panels: a 40-row front 40 us, a 160-row
+// one 509.
+template <typename T>
+__device__ __forceinline__ void front_lu_columns(T* f, int ld, int F, int ns, const SymDev& sd, int s, int k, int K,
+                                                 int32_t* status, int32_t* badcol) {
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
+  const int c0 = sd.c0[s];
+  for (int p = 0; p < ns; ++p) {
+    T* lc = f + p * ld;
+    const T piv = lc[p];
+    if (tid == 0) check_pivot(piv, sd, s, k, K, c0 + p, status, badcol);
+    const T rp = T(1) / piv;
+    for (int i = p + 1 + tid; i < F; i += nt) lc[i] *= rp;
+    __syncthreads();
+    for (int j = p + 1 + wid; j < F; j += nw) {
+      T* col = f + j * ld;
+      const T u = col[p];
+      for (int i = p + 1 + lane; i < F; i += 32) col[i] -= lc[i] * u;
+    }
+    __syncthreads();
+  }
+}
+
+// The same with the trailing elements dealt out to the threads one by one, where
+// three CTAs share an SM's FP64 pipe and every idle lane of an instruction costs as
+// much as a busy one: one barrier a pivot: warp 0 takes the next pivot's column
+// first, inverts the pivot and scales the column while the other warps update the
+// rest (48 grids 1983 us, 2015 by columns).  A CTA by itself is slower this way (a
+// 40-row front 46 us against 40, a 160-row one 540 against 509).
 template <typename T>
 __device__ __forceinline__ void front_lu_flat(T* f, int ld, int F, int ns, const SymDev& sd, int s, int k, int K,
                                               int32_t* status, int32_t* badcol) {
@@ -408,7 +433,7 @@ __device__ __forceinline__ void front_lu_flat(T* f, int ld, int F, int ns, const
 // assembly (original entries, t_k D, the children's Schur complements), pivot-
 // free LU, write to the front storage.  f: F x front_ld(F) values.
 // ---------------------------------------------------------------------------
-template <typename T>
+template <typename T, bool FLAT>
 __device__ __forceinline__ void front_cta(const SymDev& sd, int s, int k, const double* __restrict__ vals,
                                           const double* __restrict__ D, const Shifts& sh,
                                           T* __restrict__ fronts, int32_t* status, int32_t* badcol, T* f, T* rinv) {
@@ -428,7 +453,8 @@ __device__ __forceinline__ void front_cta(const SymDev& sd, int s, int k, const 
   // extend-add, every warp its share of the columns
   extend_add_flat<T>(sd, s, k, K, fronts, f, ld, (int)((int64_t)F * wid / nw), (int)((int64_t)F * (wid + 1) / nw), 0, F);
   __syncthreads();
-  if constexpr (sizeof(T) == 8) front_lu_flat<T>(f, ld, F, ns, sd, s, k, K, status, badcol);
+  if constexpr (sizeof(T) == 8 && FLAT) front_lu_flat<T>(f, ld, F, ns, sd, s, k, K, status, badcol);
+  else if constexpr (sizeof(T) == 8) front_lu_columns<T>(f, ld, F, ns, sd, s, k, K, status, badcol);
   else front_lu<T>(f, ld, F, ns, rinv, sd, s, k, K, status, badcol);
   T* out = fronts + (int64_t)K * sd.front_off[s] + (int64_t)k * F * F;
   for (int j = wid; j < F; j += nw)
@@ -442,7 +468,7 @@ __global__ void __launch_bounds__(512) k_front_small(SymDev sd, const int32_t* _
                                                      int32_t* badcol) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ T rinv[16];
-  front_cta<T>(sd, list[blockIdx.x], blockIdx.y, vals, D, sh, fronts, status, badcol,
+  front_cta<T, false>(sd, list[blockIdx.x], blockIdx.y, vals, D, sh, fronts, status, badcol,
                reinterpret_cast<T*>(smraw), rinv);
 }
 
@@ -2069,7 +2095,7 @@ k_factor_persistent(SymDev sd, const FactorTask* __restrict__ tasks, int ntasks,
       if (tid == 0) fac_wait_children(sd, fdone, need, t.s, t.k, K, err, wait_ns);
       __syncthreads();
       if (t.kind == kFacCta)
-        front_cta<T>(sd, t.s, t.k, vals, D, sh, fronts, status, badcol, sm, rinv);
+        front_cta<T, (MINB >= 3)>(sd, t.s, t.k, vals, D, sh, fronts, status, badcol, sm, rinv);
       else
         owner_tile<T, TC, MINB >= 3 ? 80 : 128>(sd, t.s, t.k, t.j, t.q, flags + t.flags, CH, err, vals, D, sh, fronts, status,
                           badcol, sm, sm + 32 * 32, sm + 32 * 32 + 32 * 33, rinv, tc);
