@@ -335,9 +335,14 @@ int tile_ctas(const pisp_handle* h, int precision) {
 // way they are launched (300 buses 164 / 164, 1354 buses 573 / 567; 118 buses 110 /
 // 129, of which 22 are the segments that the one-launch form takes for fronts of at
 // most 32 rows); many grids' fronts fill the SMs (48 grids 3939 / 2470).
+// Fronts that wait for no others (dense systems) need no more than a launch a size
+// class, and no counters, while a CTA holds each: FP32, K 4, 16 systems of 40 rows
+// 36 / 39, of 97 81 / 90, of 160 139 / 156, of 200 (owner tiles) 191 / 144, of 9 to 137
+// 110 / 122; 100 systems, K 10, of 40 rows 73 / 118; FP64, of 128 rows 2065 / 2490.
 bool one_launch(const pisp_handle* h, int precision, int32_t K) {
   if (h->factor_policy != 0) return h->factor_policy == 4;
   const int64_t tasks = (int64_t)h->sym.sn.size() * K;
+  if (h->sym.n_levels == 1 && h->sym.max_front <= 160) return false;
   if (precision != PISP_FP32) return tasks >= kManyTasks;
   const int room = tile_ctas(h, precision);
   return h->sym.max_front <= 1024 && tasks < (room >= 3 ? INT64_MAX : room == 2 ? 24 * kManyTasks : 4 * kManyTasks);

@@ -123,3 +123,27 @@ def test_owner_tiles_by_themselves(precision, sweeps, policy, hub, arms):
     assert s.status()[0] == 0
     s.close()
     assert entrywise_err(x, oracle.x_hat(A, D, t, b)) <= TOL * float(sum(abs(w) for w in oracle.weights(t)))
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("sizes,persistent", [((40, 40, 7), False), ((160, 33), False), ((200, 40), True)])
+def test_fronts_that_wait_for_no_others(precision, sizes, persistent):
+    """Dense systems: level by level while a CTA holds each front, whatever their number."""
+    import test_factor_shapes as shapes
+    G = 1000 if max(sizes) <= 40 else 1
+    insts = [pfgen.random_sparse(n, 1.0, seed=n, diag_boost=2.0 * np.sqrt(n)) for n in sizes] * G
+    s, t, dev = shapes._factor(insts, 4, precision)
+    s.profile(True)
+    s.factor(dev(np.concatenate([I.val for I in insts])), dev(np.concatenate([I.D for I in insts])), t, precision)
+    s.profile_collect()
+    s.profile(False)
+    assert bool(s.profile_read()["factor_persistent"]["launches"]) == (persistent and precision == "fp32")
+    b = pfgen.rhs(sum(I.n for I in insts), 2, 1)
+    x = s.solve(dev(b), sweeps=4 if precision == "fp32" else 0).cpu().numpy()
+    assert s.status()[0] == 0
+    s.close()
+    r0 = 0
+    scale = float(sum(abs(w) for w in oracle.weights(t)))
+    for I in insts[:len(sizes)]:
+        assert entrywise_err(x[r0:r0 + I.n], oracle.x_hat(oracle.to_scipy(I), I.D, t, b[r0:r0 + I.n])) <= TOL * scale
+        r0 += I.n
