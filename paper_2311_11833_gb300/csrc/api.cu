@@ -562,6 +562,20 @@ struct UnitList {
   std::vector<int32_t> start;  // first unit of each stage, and the number of units
 };
 
+// Whether the backward solve of R > 1 right-hand sides takes a front of ns <= 32
+// pivots by segments and not by columns: a warp's 32 columns share n^2 / 2 steps on
+// it, a segment's 8 right-hand sides n steps each, so that few columns, or many
+// pivots, leave the columns behind (dense systems, K 4, FP64, columns / segments: 32 rows,
+// R 2 55 / 18 us, R 8 56 / 45, R 32 56 / 46, and with 1000 pairs 58 / 158; 16 rows, R 4 22
+// / 18; FP32, 32 rows, R 2 28 / 14, R 8 29 / 18; 24 rows, R 8 20 / 20).
+bool few_columns(int ns, int32_t R) { return ns > std::max(8, 3 * R); }
+
+// Whether a front counts its tasks of a backward solve of R > 1 right-hand sides
+// together, because they are cut by shift.
+bool whole_front(const pisp::Supernode& n, const pisp_handle* h, int32_t R) {
+  return n.ns() > 32 || (few_columns(n.ns(), R) && n.F() <= std::max(32, h->warp_maxF));
+}
+
 // tasks[s]: tasks of front s per completion counter
 int build_unit_list(pisp_handle* h, int32_t K, int32_t R, const std::vector<int32_t>& stage, int32_t stages,
                     const std::vector<int32_t>& left, bool fwd, std::vector<int32_t>& tasks, int32_t& wide,
@@ -592,8 +606,8 @@ int build_unit_list(pisp_handle* h, int32_t K, int32_t R, const std::vector<int3
       const int32_t sn = lst[e];
       const int F = S.sn[sn].F(), ns = S.sn[sn].ns();
       if (ns > 32 || F > std::max(32, h->warp_maxF)) cta.push_back(sn);
-      else seg[cols ? 3 : (F > 16 ? 2 : (F > 8 ? 1 : 0))].push_back(sn);
-      tasks[sn] = cols ? 1 : rchunks;
+      else seg[cols && !few_columns(ns, R) ? 3 : (F > 16 ? 2 : (F > 8 ? 1 : 0))].push_back(sn);
+      tasks[sn] = !cols ? rchunks : whole_front(S.sn[sn], h, R) ? K * rchunks : 1;
     }
     std::sort(cta.begin(), cta.end(), [&](int32_t a, int32_t b) {
       if (left[a] != left[b]) return left[a] > left[b];
@@ -660,7 +674,7 @@ int build_units(pisp_handle* h, int32_t K, int32_t R) {
   // completion targets: forward, every task of a front's children; backward,
   // every task of its parent, as the counters count them
   const int NG = std::max(counter_groups(h, K, R, true), counter_groups(h, K, R, false));
-  auto whole = [&](int32_t q) { return R > 1 && S.sn[q].ns() > 32; };  // backward
+  auto whole = [&](int32_t q) { return R > 1 && whole_front(S.sn[q], h, R); };  // backward
   std::vector<int32_t> need(nS, 0);
   for (size_t q = 0; q < nS; ++q)
     if (S.sn[q].parent >= 0) need[S.sn[q].parent] += nf[q];

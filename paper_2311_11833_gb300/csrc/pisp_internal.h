@@ -211,8 +211,8 @@ int max_solve_front(int precision);
 
 // ---- solve (solve_persistent.h; solve.cu) ----
 // Work unit of the solves: 16 bytes, read at once.  x = kind | d << 4.
-//   kUnitSeg8/16/32 (forward, and backward with one right-hand side): 256 / SEG
-//     consecutive segment tasks of one group (a task = one front, a group of d
+//   kUnitSeg8/16/32 (forward, and backward with one right-hand side, or with many
+//     pivots to few right-hand sides): 256 / SEG consecutive segment tasks of one group (a task = one front, a group of d
 //     consecutive shifts, one chunk of 8 right-hand sides or the only one): a =
 //     the group's first front record, b = first task, c = tasks in the group;
 //   kUnitCol (backward, several right-hand sides): 8 consecutive warp tasks of

@@ -83,8 +83,8 @@ __device__ __forceinline__ void publish(int* f) {
 // counts per group, so that the groups run through the tree independently.
 // Forward, a front waits for the tasks of its children, counted at itself;
 // backward, for those of its parent, counted at the parent.  Backward with
-// several right-hand sides a front with more than 32 pivots is cut by shift, and
-// counts all its tasks together (at group 0).
+// several right-hand sides a front solved by segments or with more than 32 pivots is
+// cut by shift, and counts all its tasks together (at group 0).
 template <typename T>
 __device__ __forceinline__ void wait_children(const SolveArgs<T>& a, const FrontDesc& d, int g) {
   if (a.done && d.needF > 0) wait_count(a.done + ((int64_t)d.s * a.NG + g) * kCtrStride, d.needF, a.err, a.wait_ns);
@@ -511,6 +511,77 @@ __device__ __forceinline__ void seg_backward(const SolveArgs<T>& a, const SegTas
   }
 }
 
+// The same for several right-hand sides, eight columns of coefficients at a time.
+template <typename T, int SEG, bool TRANS, int NR>
+__device__ __forceinline__ void seg_backward_rhs(const SolveArgs<T>& a, const SegTask& t, const FrontDesc& d, int sl) {
+  const int ns = d.ns, F = d.F;
+  const int nr = t.active ? t.nr : 0;
+  const bool vec = a.vec;
+  const int Fw = min(SEG, __reduce_max_sync(kFull, F)), top = (Fw - 1) & ~7;
+  const int nkw = __reduce_max_sync(kFull, t.k1 - t.k0);
+  const int nrw = __reduce_max_sync(kFull, nr);
+  const int64_t row = sl < ns ? d.c0 + sl : ld_early(a.rows + d.ro + sl - ns, sl < F);
+  for (int kk = 0; kk < nkw; ++kk) {
+    const int k = min(t.k0 + kk, max(t.k1 - 1, 0));
+    const bool kon = t.k0 + kk < t.k1 && t.active;
+    const T* f = a.fronts + a.K * d.fo + (int64_t)k * F * F;
+    T C[8], v[NR];
+    auto load8 = [&](int jb) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int j = jb + q;
+        C[q] = coef<T, TRANS>(f, F, sl, j, kon && sl < ns && j > sl && j < F);
+      }
+    };
+    load8(top);
+    T rd = T(1);
+    if (!TRANS && kon && sl < ns) rd = T(1) / __ldg(f + (int64_t)sl * (F + 1));
+    const int n = (kon && sl < F) ? nr : 0;
+    ld_row<T, NR>(a.V + ((d.vo + sl) * a.K + k) * a.RV + t.r0, sl < ns ? n : 0, vec, v);
+    if (!TRANS) settle(rd);
+    if (kon && sl == 0) wait_parent(a, d, 0);
+    __syncwarp();
+    T* x = a.xt + (row * a.K + k) * a.RV + t.r0;
+    if (n && sl >= ns) ld_row<T, NR>(x, n, vec, v);
+    if (SEG == 32) {
+      // positions beyond the first 32 (one front a warp): ancestors' solutions, 32 at a time
+      for (int j0 = 32; j0 < F; j0 += 32) {
+        const int j = j0 + sl, m = min(32, F - j0);
+        const bool in = kon && j < F;
+        const int64_t rj = ld_early(a.rows + d.ro + j - ns, in);
+        T y[NR];
+        ld_row<T, NR>(a.xt + (rj * a.K + k) * a.RV + t.r0, in ? nr : 0, vec, y);
+        for (int jj = 0; jj < m; ++jj) {
+          const T u = coef<T, TRANS>(f, F, sl, j0 + jj, kon && sl < ns);
+#pragma unroll
+          for (int r = 0; r < NR; ++r)
+            if (r < nrw) v[r] -= u * __shfl_sync(kFull, y[r], jj);
+        }
+      }
+    }
+    for (int jb = top; jb >= 0; jb -= 8) {
+      if (jb != top) load8(jb);
+#pragma unroll
+      for (int q = 7; q >= 0; --q) {
+        const int j = jb + q;
+        if (j >= Fw) continue;
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+          if (r < nrw) {
+            if (!TRANS && sl == j) v[r] *= rd;  // rd = 1 beyond the pivots
+            v[r] -= C[q] * __shfl_sync(kFull, v[r], j, SEG);
+          }
+      }
+    }
+    if (n && sl < ns) {
+      st_row<T, NR>(x, n, vec, v);
+      if (a.xd) st_xd_row<T, NR>(a.xd + (row * a.K + k) * a.RX + t.r0, n, a.vecd, a.xd_mode, v);
+    }
+    __syncwarp();
+    if (kon && sl == 0) publish_self(a, d, 0);
+  }
+}
+
 // One warp, lane = row of a staged 32 x 32 triangle B (zero outside it, rd =
 // reciprocal diagonal, 1 where unit): v becomes the solution.
 template <typename T, bool LOWER, bool UNIT>
@@ -681,7 +752,8 @@ __device__ __forceinline__ void thin_backward1(const SolveArgs<T>& a, const Fron
 }
 
 // ---------------------------------------------------------------------------
-// Backward solves of several right-hand sides, fronts with at most 32 pivots: a
+// Backward solves of several right-hand sides, fronts with at most 32 pivots (but for
+// those with many pivots to few right-hand sides, kUnitSeg16/32): a
 // warp takes one front for 32 of its K x RV columns (k, r), one a lane.
 // Structure is read once for the 32 columns, V and xt a whole row segment at a
 // time, and no lane idles on a front's shape; the columns of the front are
@@ -1345,6 +1417,15 @@ __global__ void __launch_bounds__(kSolveThreads, MINB) k_solve(const __grid_cons
         const SegTask t = seg_task<T>(a, U, (unsigned)U.b + tid / 32, NR, d);
         if constexpr (FWD) seg_forward<T, 32, TRANS, NR>(a, t, d, tid % 32, sm + wid * 32 * NR);
         else seg_backward<T, 32, TRANS>(a, t, d, tid % 32);
+      }
+    } else if (kind == kUnitSeg16 || kind == kUnitSeg32) {
+      FrontDesc d;
+      if (kind == kUnitSeg16) {
+        const SegTask t = seg_task<T>(a, U, (unsigned)U.b + tid / 16, 8, d);
+        seg_backward_rhs<T, 16, TRANS, 8>(a, t, d, tid % 16);
+      } else {
+        const SegTask t = seg_task<T>(a, U, (unsigned)U.b + tid / 32, 8, d);
+        seg_backward_rhs<T, 32, TRANS, 8>(a, t, d, tid % 32);
       }
     } else {
       // a CTA task, its 8 warps sharing the front, or per warp task q of the

@@ -202,3 +202,41 @@ def test_solve_that_cannot_be_set_up_leaves_nothing_to_differentiate():
     scale = float(sum(abs(w) for w in oracle.weights(t)))
     assert entrywise_err(x, oracle.x_hat(A, inst.D, t, b)) <= TOL * scale
     assert entrywise_err(gb, oracle.adjoint(A, inst.D, t, b, g)[0]) <= TOL * scale
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision,sweeps", [("fp64", 0), ("fp32", 4)])
+@pytest.mark.parametrize("K,R,opts", [
+    (1, 2, {}), (4, 2, dict(solve_kfuse=3)), (3, 3, dict(solve_schedule=1)), (2, 4, dict(solve_warp_maxF=64)),
+    (2, 5, dict(solve_warp_maxF=64, solve_ctas_per_sm=4)), (4, 8, {}), (2, 9, {}), (16, 7, {}), (16, 12, {})])
+def test_pivots_to_right_hand_sides(precision, sweeps, K, R, opts):
+    """Fronts of 9 to 32 pivots around the numbers of right-hand sides where their
+    backward solve changes from segments to columns (3 R pivots), alone and under other
+    fronts, and fronts with more pivots at 1, 2 and 4 right-hand sides a task (FP64)."""
+    import paper_2311_11833_gb300 as pisp
+    dense = [pfgen.random_sparse(n, 1.0, seed=n, diag_boost=2.0 * np.sqrt(n))
+             for n in (6, 9, 10, 12, 13, 15, 16, 17, 24, 25, 27, 28, 32, 65, 257, 300)]
+    insts = dense + [_thin(p) for p in (2, 9, 12, 17, 32)] + [pfgen.grid_jacobian(140, None, 9)]
+    sizes, rp, col, val, D = _concat(insts)
+    t = pfgen.one_sided_shifts(K, 1e-3) if K % 2 else pfgen.symmetric_shifts(K, 1e-3)
+    N = sum(sizes)
+    b, g = pfgen.rhs(N, R, 5), pfgen.rhs(N, R, 6)
+    s = pisp.Solver(sizes, rp, col, ordering=1, relax_small=1, relax_zeros=0.0, **opts)
+    s.factor(_dev(val), _dev(D), t, precision)
+    x = s.solve(_dev(b), sweeps=sweeps).cpu().numpy()
+    again = s.solve(_dev(b), sweeps=sweeps).cpu().numpy()
+    gb, gv = (v.cpu().numpy() for v in s.adjoint(_dev(g), sweeps=sweeps))
+    assert s.status()[0] == 0
+    s.close()
+    assert (x == again).all()
+    scale = float(sum(abs(w) for w in oracle.weights(t)))
+    r0 = e0 = 0
+    for I in insts:
+        rows, ent = slice(r0, r0 + I.n), slice(e0, e0 + I.nnz)
+        A = oracle.to_scipy(I)
+        assert entrywise_err(x[rows], oracle.x_hat(A, I.D, t, b[rows])) <= TOL * scale, I.n
+        rb, rv = oracle.adjoint(A, I.D, t, b[rows], g[rows])
+        assert entrywise_err(gb[rows], rb) <= TOL * scale, I.n
+        assert grad_entrywise_err(gv[ent], rv) <= TOL * scale, I.n
+        r0 += I.n
+        e0 += I.nnz
