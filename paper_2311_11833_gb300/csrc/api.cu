@@ -67,7 +67,7 @@ struct pisp_handle {
   int32_t factor_policy = 0;
   int32_t units_K = 0, units_R = 0;
   int32_t n_units_f = 0, n_units_b = 0;
-  int32_t units_wide = 0;                     // largest chunk of a front with more than 32 pivots
+  int32_t units_wide[2] = {};                 // right-hand sides of a task of a front with more than 32 pivots, per direction
   size_t ctr_tickets = 0, ctr_half = 0;       // tickets, and all counters, of one direction
   std::vector<int32_t> lvl_units_f, lvl_units_b;  // first unit of each stage (one launch per stage)
   // front records in unit-list order; counters, forward then backward: the
@@ -562,18 +562,40 @@ struct UnitList {
   std::vector<int32_t> start;  // first unit of each stage, and the number of units
 };
 
-// Whether the backward solve of R > 1 right-hand sides takes a front of ns <= 32
-// pivots by segments and not by columns: a warp's 32 columns share n^2 / 2 steps on
+// Right-hand sides of a task of a front with more than 32 pivots, by the most such
+// tasks that a stage would have with one each.  FP32: four, whose chains of steps
+// overlap in the warp that solves a block, or eight, a warp each, where such tasks fill
+// the SMs (two CTAs each) and the kernel has the registers: 100 dense systems of 97
+// rows, K 10, R 8, forward + backward, 50 + 48 us, 74 + 70 with four; 4 of 97, K 6, R 4,
+// 15 + 15.  FP64, whose pipe is what the columns of a task wait for: one while those
+// fill the SMs (4 systems of 97 rows, K 6, R 4: 22 + 25 us, 33 + 40 with two in one
+// warp), then two and four, a warp each (40 grids to 1500 buses, K 4, R 8: 208 + 208, 197
+// + 213 with one, 228 + 245 with four; 128 to 3000: 1014 + 784, 1025 + 831, 941 + 710),
+// and eight where even those fill them many times (100 of 64 rows, K 10, R 32: 343 + 485
+// us, 400 + 531 with four; 712 + 973 with two in one warp).
+int wide_rhs(const pisp_handle* h, int64_t tasks, int32_t R) {
+  if (R == 1) return 1;
+  constexpr int64_t kCtas = 2 * 152;
+  if (h->precision == PISP_FP32) return R > 4 && h->solve_ctas <= 2 && tasks * ((R + 7) / 8) >= kCtas ? 8 : 4;
+  const int64_t n = tasks * R;
+  return n <= kCtas ? 1 : (n <= 4 * kCtas ? 2 : (n <= 32 * kCtas ? 4 : 8));
+}
+
+// Whether the backward solve of R > 1 right-hand sides takes a front of at most 32
+// rows by segments and not by columns: a warp's 32 columns share n^2 / 2 steps on
 // it, a segment's 8 right-hand sides n steps each, so that few columns, or many
 // pivots, leave the columns behind (dense systems, K 4, FP64, columns / segments: 32 rows,
 // R 2 55 / 18 us, R 8 56 / 45, R 32 56 / 46, and with 1000 pairs 58 / 158; 16 rows, R 4 22
-// / 18; FP32, 32 rows, R 2 28 / 14, R 8 29 / 18; 24 rows, R 8 20 / 20).
-bool few_columns(int ns, int32_t R) { return ns > std::max(8, 3 * R); }
+// / 18; FP32, 32 rows, R 2 28 / 14, R 8 29 / 18; 24 rows, R 8 20 / 20).  Compiled for
+// more than two CTAs an SM the kernel has no registers for both.
+bool few_columns(const pisp_handle* h, const pisp::Supernode& n, int32_t R) {
+  return h->solve_ctas <= 2 && n.F() <= 32 && n.ns() > std::max(8, 3 * R);
+}
 
 // Whether a front counts its tasks of a backward solve of R > 1 right-hand sides
 // together, because they are cut by shift.
-bool whole_front(const pisp::Supernode& n, const pisp_handle* h, int32_t R) {
-  return n.ns() > 32 || (few_columns(n.ns(), R) && n.F() <= std::max(32, h->warp_maxF));
+bool whole_front(const pisp_handle* h, const pisp::Supernode& n, int32_t R) {
+  return n.ns() > 32 || few_columns(h, n, R);
 }
 
 // tasks[s]: tasks of front s per completion counter
@@ -594,27 +616,34 @@ int build_unit_list(pisp_handle* h, int32_t K, int32_t R, const std::vector<int3
     out.rng.push_back(S.sn[sn].instance);
     out.rng.push_back(S.sn[sn].instance);
   };
+  auto wide_rows = [&](int32_t sn) {  // tasks of 256 rows
+    return ((fwd ? S.sn[sn].F() : S.sn[sn].ns()) + pisp::kWideUnitRows - 1) / pisp::kWideUnitRows;
+  };
+  int64_t most = 0;
+  for (int32_t st = 0; st < stages; ++st) {
+    int64_t n = 0;
+    for (int32_t e = at[st]; e < at[st + 1]; ++e)
+      if (S.sn[lst[e]].ns() > 32) n += (int64_t)wide_rows(lst[e]) * K;
+    most = std::max(most, n);
+  }
+  const int rc = wide_rhs(h, most, R);
   std::vector<int32_t> cta, seg[4];  // segments of 8, 16, 32 lanes; warps
   for (int32_t st = 0; st < stages; ++st) {
     out.start.push_back((int32_t)out.units.size());
     cta.clear();
     for (auto& g : seg) g.clear();
-    auto wide_rows = [&](int32_t sn) {  // tasks of 256 rows
-      return ((fwd ? S.sn[sn].F() : S.sn[sn].ns()) + pisp::kWideUnitRows - 1) / pisp::kWideUnitRows;
-    };
     for (int32_t e = at[st]; e < at[st + 1]; ++e) {
       const int32_t sn = lst[e];
       const int F = S.sn[sn].F(), ns = S.sn[sn].ns();
       if (ns > 32 || F > std::max(32, h->warp_maxF)) cta.push_back(sn);
-      else seg[cols && !few_columns(ns, R) ? 3 : (F > 16 ? 2 : (F > 8 ? 1 : 0))].push_back(sn);
-      tasks[sn] = !cols ? rchunks : whole_front(S.sn[sn], h, R) ? K * rchunks : 1;
+      else seg[cols ? (few_columns(h, S.sn[sn], R) ? 2 : 3) : (F > 16 ? 2 : (F > 8 ? 1 : 0))].push_back(sn);
+      tasks[sn] = !cols ? rchunks : whole_front(h, S.sn[sn], R) ? K * rchunks : 1;
     }
     std::sort(cta.begin(), cta.end(), [&](int32_t a, int32_t b) {
       if (left[a] != left[b]) return left[a] > left[b];
       const int fa = S.sn[a].F(), fb = S.sn[b].F();
       return fa != fb ? fa > fb : a < b;
     });
-    const int rc = pisp::wide_chunk(h->precision, R);
     for (int32_t sn : cta) {
       const int32_t slot = (int32_t)out.order.size();
       out.order.push_back(sn);
@@ -624,13 +653,13 @@ int build_unit_list(pisp_handle* h, int32_t K, int32_t R, const std::vector<int3
         continue;
       }
       const int ch = (R + rc - 1) / rc, nq = wide_rows(sn);
-      wide = std::max(wide, rc);
+      wide = rc;
       tasks[sn] = cols ? nq * K * ch : nq * ch;
       // the rows solved first, first: a task waits only for tasks before it
       for (int q = 0; q < nq; ++q)
         for (int k = 0; k < K; ++k)
           for (int c = 0; c < ch; ++c)
-            cta_unit(sn, {pisp::kUnitWide | rc << 4, slot, k | (fwd ? q : nq - 1 - q) << 8, c});
+            cta_unit(sn, {pisp::kUnitWide, slot, k | rc << 4 | (fwd ? q : nq - 1 - q) << 8, c});
     }
     for (int w = 3; w >= 0; --w) {
       std::vector<int32_t>& g = seg[w];
@@ -668,13 +697,13 @@ int build_units(pisp_handle* h, int32_t K, int32_t R) {
   }
   UnitList f, b;
   std::vector<int32_t> nf(nS, 1), nb(nS, 1);
-  int32_t wide = 0;
-  TRY(build_unit_list(h, K, R, height, S.n_levels, depth, true, nf, wide, f));
-  TRY(build_unit_list(h, K, R, depth, deepest + 1, height, false, nb, wide, b));
+  int32_t wide[2] = {};
+  TRY(build_unit_list(h, K, R, height, S.n_levels, depth, true, nf, wide[0], f));
+  TRY(build_unit_list(h, K, R, depth, deepest + 1, height, false, nb, wide[1], b));
   // completion targets: forward, every task of a front's children; backward,
   // every task of its parent, as the counters count them
   const int NG = std::max(counter_groups(h, K, R, true), counter_groups(h, K, R, false));
-  auto whole = [&](int32_t q) { return R > 1 && whole_front(S.sn[q], h, R); };  // backward
+  auto whole = [&](int32_t q) { return R > 1 && whole_front(h, S.sn[q], R); };  // backward
   std::vector<int32_t> need(nS, 0);
   for (size_t q = 0; q < nS; ++q)
     if (S.sn[q].parent >= 0) need[S.sn[q].parent] += nf[q];
@@ -726,7 +755,8 @@ int build_units(pisp_handle* h, int32_t K, int32_t R) {
   h->n_units_b = (int32_t)b.units.size();
   h->lvl_units_f = f.start;
   h->lvl_units_b = b.start;
-  h->units_wide = wide;
+  h->units_wide[0] = wide[0];
+  h->units_wide[1] = wide[1];
   h->ctr_tickets = (f.start.size() + b.start.size()) / 8 * 8 + 8;  // more than one per stage
   h->ctr_half = h->ctr_tickets + (nS * (size_t)NG + (size_t)nflags) * pisp::kCtrStride;
   h->units_K = K;
@@ -854,8 +884,8 @@ int solve_pass_t(pisp_handle* h, bool trans, const SolveIO& io, int32_t R, const
     const int pb = prof_begin(h);
     int n = 0;
     auto go = [&](int count) {
-      return dir == 0 ? pisp::launch_solve_dir<T, true>(trans, a, count, h->units_wide, h->solve_ctas, h->stream)
-                      : pisp::launch_solve_dir<T, false>(trans, a, count, h->units_wide, h->solve_ctas, h->stream);
+      return dir == 0 ? pisp::launch_solve_dir<T, true>(trans, a, count, h->units_wide[dir], h->solve_ctas, h->stream)
+                      : pisp::launch_solve_dir<T, false>(trans, a, count, h->units_wide[dir], h->solve_ctas, h->stream);
     };
     const int total = dir == 0 ? h->n_units_f : h->n_units_b;
     a.NG = counter_groups(h, h->K, R, dir == 0);

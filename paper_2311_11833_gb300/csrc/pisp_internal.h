@@ -220,8 +220,9 @@ int max_solve_front(int precision);
 //     above;
 //   kUnitCta: one front (record a) with at most 32 pivots, for the shift b and
 //     RHS chunk c, or for the column group b;
-//   kUnitWide: a front (record a) with more than 32 pivots, b = shift | q << 8
-//     with q the 256 rows taken, RHS chunk c of d right-hand sides.
+//   kUnitWide: a front (record a) with more than 32 pivots, b = shift | d << 4 |
+//     q << 8 with q the 256 rows taken, RHS chunk c of d right-hand sides (as many
+//     in all units of a direction).
 enum UnitKind { kUnitSeg8 = 0, kUnitSeg16 = 1, kUnitSeg32 = 2, kUnitCol = 3, kUnitCta = 4, kUnitWide = 5 };
 struct SolveUnit {
   int32_t x, a, b, c;
@@ -282,13 +283,11 @@ inline int32_t rhs_stride64(int32_t R) { return R == 1 ? 1 : (R + 1) / 2 * 2; }
 
 // One launch of the forward (L, or U^T with trans) or backward (U, L^T) solve;
 // ctas = resident CTAs per SM it is compiled for with several right-hand sides
-// (2, 3, 4; <= 0, or transposed: 2); wide = the largest chunk of a front with more
-// than 32 pivots, 0 if there is none.  Returns the kernels launched or -1.
+// (2, 3, 4; <= 0, or transposed: 2); wide = the most right-hand sides of a task of a
+// front with more than 32 pivots, 0 if there is none.  Returns the kernels launched or -1.
 template <typename T, bool FWD>
 int launch_solve_dir(bool trans, const SolveArgs<T>& a, int32_t nunits, int32_t wide, int32_t ctas, cudaStream_t st);
-// right-hand sides and rows of a task of a front with more than 32 pivots
-int wide_chunk(int precision, int R);
-constexpr int kWideUnitRows = 256;
+constexpr int kWideUnitRows = 256;  // rows of a task of a front with more than 32 pivots
 int launch_combine(const SymDev& sd, const double* X, const Shifts& sh, int32_t R, double* x,
                    cudaStream_t st);
 // The instances still iterating in the adaptive sweeps (device arrays

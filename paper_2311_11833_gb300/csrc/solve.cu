@@ -453,8 +453,6 @@ unsigned sm_count() {
 // they held one in 96 KB of shared memory, and no wider front has been run since.
 int max_solve_front(int precision) { return precision == PISP_FP32 ? 24576 : 12288; }
 
-int wide_chunk(int precision, int R) { return R == 1 ? 1 : (precision == PISP_FP32 ? 4 : 2); }
-
 int launch_combine(const SymDev& sd, const double* X, const Shifts& sh, int32_t R, double* x,
                    cudaStream_t st) {
   const int64_t n = sd.N * R;

@@ -511,65 +511,47 @@ __device__ __forceinline__ void seg_backward(const SolveArgs<T>& a, const SegTas
   }
 }
 
-// The same for several right-hand sides, eight columns of coefficients at a time.
-template <typename T, int SEG, bool TRANS, int NR>
+// The same for several right-hand sides and a front of at most 32 rows a warp, eight
+// columns of coefficients at a time.
+template <typename T, bool TRANS, int NR>
 __device__ __forceinline__ void seg_backward_rhs(const SolveArgs<T>& a, const SegTask& t, const FrontDesc& d, int sl) {
   const int ns = d.ns, F = d.F;
-  const int nr = t.active ? t.nr : 0;
+  const int nr = t.nr;
   const bool vec = a.vec;
-  const int Fw = min(SEG, __reduce_max_sync(kFull, F)), top = (Fw - 1) & ~7;
-  const int nkw = __reduce_max_sync(kFull, t.k1 - t.k0);
-  const int nrw = __reduce_max_sync(kFull, nr);
+  const int top = (F - 1) & ~7;
   const int64_t row = sl < ns ? d.c0 + sl : ld_early(a.rows + d.ro + sl - ns, sl < F);
-  for (int kk = 0; kk < nkw; ++kk) {
-    const int k = min(t.k0 + kk, max(t.k1 - 1, 0));
-    const bool kon = t.k0 + kk < t.k1 && t.active;
+  if (!t.active) return;
+  for (int k = t.k0; k < t.k1; ++k) {
     const T* f = a.fronts + a.K * d.fo + (int64_t)k * F * F;
     T C[8], v[NR];
     auto load8 = [&](int jb) {
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         const int j = jb + q;
-        C[q] = coef<T, TRANS>(f, F, sl, j, kon && sl < ns && j > sl && j < F);
+        C[q] = coef<T, TRANS>(f, F, sl, j, sl < ns && j > sl && j < F);
       }
     };
     load8(top);
     T rd = T(1);
-    if (!TRANS && kon && sl < ns) rd = T(1) / __ldg(f + (int64_t)sl * (F + 1));
-    const int n = (kon && sl < F) ? nr : 0;
+    if (!TRANS && sl < ns) rd = T(1) / __ldg(f + (int64_t)sl * (F + 1));
+    const int n = sl < F ? nr : 0;
     ld_row<T, NR>(a.V + ((d.vo + sl) * a.K + k) * a.RV + t.r0, sl < ns ? n : 0, vec, v);
     if (!TRANS) settle(rd);
-    if (kon && sl == 0) wait_parent(a, d, 0);
+    if (sl == 0) wait_parent(a, d, 0);
     __syncwarp();
     T* x = a.xt + (row * a.K + k) * a.RV + t.r0;
     if (n && sl >= ns) ld_row<T, NR>(x, n, vec, v);
-    if (SEG == 32) {
-      // positions beyond the first 32 (one front a warp): ancestors' solutions, 32 at a time
-      for (int j0 = 32; j0 < F; j0 += 32) {
-        const int j = j0 + sl, m = min(32, F - j0);
-        const bool in = kon && j < F;
-        const int64_t rj = ld_early(a.rows + d.ro + j - ns, in);
-        T y[NR];
-        ld_row<T, NR>(a.xt + (rj * a.K + k) * a.RV + t.r0, in ? nr : 0, vec, y);
-        for (int jj = 0; jj < m; ++jj) {
-          const T u = coef<T, TRANS>(f, F, sl, j0 + jj, kon && sl < ns);
-#pragma unroll
-          for (int r = 0; r < NR; ++r)
-            if (r < nrw) v[r] -= u * __shfl_sync(kFull, y[r], jj);
-        }
-      }
-    }
     for (int jb = top; jb >= 0; jb -= 8) {
       if (jb != top) load8(jb);
 #pragma unroll
       for (int q = 7; q >= 0; --q) {
         const int j = jb + q;
-        if (j >= Fw) continue;
+        if (j >= F) continue;
 #pragma unroll
         for (int r = 0; r < NR; ++r)
-          if (r < nrw) {
+          if (r < nr) {
             if (!TRANS && sl == j) v[r] *= rd;  // rd = 1 beyond the pivots
-            v[r] -= C[q] * __shfl_sync(kFull, v[r], j, SEG);
+            v[r] -= C[q] * __shfl_sync(kFull, v[r], j);
           }
       }
     }
@@ -578,7 +560,7 @@ __device__ __forceinline__ void seg_backward_rhs(const SolveArgs<T>& a, const Se
       if (a.xd) st_xd_row<T, NR>(a.xd + (row * a.K + k) * a.RX + t.r0, n, a.vecd, a.xd_mode, v);
     }
     __syncwarp();
-    if (kon && sl == 0) publish_self(a, d, 0);
+    if (sl == 0) publish_self(a, d, 0);
   }
 }
 
@@ -753,7 +735,7 @@ __device__ __forceinline__ void thin_backward1(const SolveArgs<T>& a, const Fron
 
 // ---------------------------------------------------------------------------
 // Backward solves of several right-hand sides, fronts with at most 32 pivots (but for
-// those with many pivots to few right-hand sides, kUnitSeg16/32): a
+// those with many pivots to few right-hand sides, kUnitSeg32): a
 // warp takes one front for 32 of its K x RV columns (k, r), one a lane.
 // Structure is read once for the 32 columns, V and xt a whole row segment at a
 // time, and no lane idles on a front's shape; the columns of the front are
@@ -1012,10 +994,18 @@ __device__ __forceinline__ void col_backward(const SolveArgs<T>& a, const FrontD
 // (One CTA walking all the rows of a front, values in shared memory and blocks
 // solved one right-hand side a warp, took 6.7 us a block on a 1600-row root,
 // 3.2 us on a 320-row one.)
+// Many such tasks share the SMs' pipes, and a block that one warp solves leaves its
+// SM's idle: there the owning warp hands its block to as many warps as there are
+// right-hand sides and takes the solution back, two barriers a block (kSpread).
 // ---------------------------------------------------------------------------
 constexpr int kWideRows = kSolveThreads;
+constexpr int kTri = 32 * kBS + 32;  // a staged triangle and its reciprocal pivots
+// right-hand sides of a task compiled for the spread form (at most), and for the other
+template <typename T> constexpr int kWideSpread = 8;
+template <typename T> constexpr int kWideAlone = sizeof(T) == 8 ? 1 : 4;
+template <typename T, int RC> constexpr bool kSpread = RC == kWideSpread<T>;
 
-template <typename T> struct WideTile { static constexpr int C = 16, LD = C + 1; };
+template <typename T> struct WideTile { static constexpr int C = sizeof(T) == 8 ? 8 : 16, LD = C + 1; };
 
 // L[c] = coefficient (i, col0 + c), c < nb, of this thread's row i (rows past
 // lim repeat the last one).  The columns of a row are F apart in memory unless
@@ -1057,18 +1047,41 @@ __device__ __forceinline__ void load_panel(T (&L)[32], const T* f, int F, int i,
 // w -= sum_c L[c] y(c, :), y 32 rows of RC values in shared memory (zero where
 // the coefficients are)
 template <typename T, int RC>
-__device__ __forceinline__ void apply_panel(const T (&L)[32], T (&w)[RC], const T* y) {
+__device__ __forceinline__ void apply_panel(const T (&L)[32], T (&w)[RC], const T* y, int nr) {
+  if constexpr (sizeof(T) == 8 && RC > 1) {  // the FP64 pipe's time is the columns': only those there are
 #pragma unroll
-  for (int c = 0; c < 32; ++c) {
-    if (c % (16 / RC) == 0) keep_order();
+    for (int r = 0; r < RC; ++r)
+      if (r < nr) {
 #pragma unroll
-    for (int r = 0; r < RC; ++r) w[r] -= L[c] * y[c * RC + r];
+        for (int c = 0; c < 32; ++c) {
+          if (c % 8 == 0) keep_order();
+          w[r] -= L[c] * y[c * RC + r];
+        }
+      }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      if (c % (16 / RC) == 0) keep_order();
+#pragma unroll
+      for (int r = 0; r < RC; ++r) w[r] -= L[c] * y[c * RC + r];
+    }
   }
 }
 
+// The CTA: block `own` (its warp's number) of nb <= 32 pivots, handed over in y [32][RC] by
+// the warp that owns it, solved one right-hand side a warp.  All threads call.
+template <typename T, bool LOWER, bool UNIT, int RC>
+__device__ __forceinline__ void spread_solve(const T* B, int own, T* y, int nr, int nb, int wid, int lane) {
+  __syncthreads();
+  if (wid < nr) {
+    const T* Bo = B + own * kTri;
+    y[lane * RC + wid] = block_solve<T, LOWER, UNIT>(Bo, Bo + 32 * kBS, y[lane * RC + wid], nb, lane);
+  }
+  __syncthreads();
+}
+
 // This warp's diagonal block (nb pivots from p0) into B, zero outside the
-// triangle, and unless UNIT the reciprocal pivots behind it.
-constexpr int kTri = 32 * kBS + 32;
+// triangle, and unless UNIT the reciprocal pivots behind it (1 past the pivots).
 template <typename T, bool LOWER, bool UNIT, bool TRANS>
 __device__ __forceinline__ void stage_triangle(T* B, const T* f, int F, int p0, int nb, int lane) {
   T rd = T(1);
@@ -1093,15 +1106,15 @@ __device__ __forceinline__ void stage_triangle(T* B, const T* f, int F, int p0, 
 // (in the order their own lanes would), which quarters the chain of shuffles.
 // FP64 goes one at a time: its multiply-adds, at 2 a clock and SM, cost more
 // than the shuffles.  Rows already solved meet zero coefficients and keep
-// their values.
+// their values (FP64 leaves out the steps past the nb pivots of a short block).
 template <typename T, bool LOWER, bool UNIT, int RC>
-__device__ __forceinline__ void triangle_solve(const T* B, T (&v)[RC], int lane) {
+__device__ __forceinline__ void triangle_solve(const T* B, T (&v)[RC], int nb, int lane) {
   const T* bl = B + lane * kBS;
   const T* rd = B + 32 * kBS;
   if constexpr (sizeof(T) == 8) {
 #pragma unroll 4
-    for (int q = 0; q < 32; ++q) {
-      const int c = LOWER ? q : 31 - q;
+    for (int q = 0; q < nb; ++q) {
+      const int c = LOWER ? q : nb - 1 - q;
       const T b = bl[c], rc = UNIT ? T(1) : rd[c];
 #pragma unroll
       for (int r = 0; r < RC; ++r) {
@@ -1146,12 +1159,19 @@ __device__ __forceinline__ void triangle_solve(const T* B, T (&v)[RC], int lane)
   }
 }
 
+// whether right-hand sides r0 .. r0 + nr fill pairs of a row but for its padding: a
+// chunk of four or eight does, one of one or two (FP64) may not
+template <typename T>
+__device__ __forceinline__ bool whole_pairs(const SolveArgs<T>& a, int r0, int nr) {
+  return sizeof(T) == 4 || (r0 % 2 == 0 && (nr % 2 == 0 || r0 + nr == a.R));
+}
+
 template <typename T, bool TRANS, int RC>
-__device__ __forceinline__ void wide_forward(const SolveArgs<T>& a, const FrontDesc& d, int k, int q, int ch, int r0,
-                                             int nr, T* sm) {
+__device__ __forceinline__ void wide_forward(const SolveArgs<T>& a, const FrontDesc& d, int k, int q, int ch, int rc,
+                                             int r0, int nr, T* sm) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int ns = d.ns, F = d.F;
-  const bool vec = a.vec && (r0 % Vec16<T>::N == 0);
+  const bool vec = a.vec && whole_pairs<T>(a, r0, nr);
   T* ys = sm;                                    // kWideRows x RC: solved blocks
   T* B = ys + kWideRows * RC + wid * kTri;       // this warp's triangle
   T* tile = ys + kWideRows * RC + kSolveWarps * kTri + wid * 32 * WideTile<T>::LD;  // TRANS
@@ -1165,7 +1185,7 @@ __device__ __forceinline__ void wide_forward(const SolveArgs<T>& a, const FrontD
   const int last = min(mine, nblk - 1);                   // last block this warp takes part in
   const bool rows = i - lane < F;                         // this warp has rows
   const bool shared = F > kWideRows;                      // other CTAs take this front's other rows
-  int* flag = a.wide + (int64_t)(d.flag + (k * ((a.R + RC - 1) / RC) + ch)) * kCtrStride;
+  int* flag = a.wide + (int64_t)(d.flag + (k * ((a.R + rc - 1) / rc) + ch)) * kCtrStride;
   if (mine < nblk) stage_triangle<T, true, !TRANS, TRANS>(B, f, F, mine * 32, min(32, ns - mine * 32), lane);
   Gather g = gather_begin<T>(a, d, i, i < F);
   if (tid == 0) wait_children(a, d, k);
@@ -1205,7 +1225,7 @@ __device__ __forceinline__ void wide_forward(const SolveArgs<T>& a, const FrontD
     __syncthreads();
     for (int e = 0; e < m; ++e, ++p) {
       if (!rows) continue;
-      apply_panel<T, RC>(L, w, ys + e * 32 * RC);
+      apply_panel<T, RC>(L, w, ys + e * 32 * RC, nr);
       if (p + 1 <= last && p + 1 != mine)
         load_panel<T, TRANS>(L, f, F, i, F, (p + 1) * 32, min(32, ns - (p + 1) * 32), tile, lane);
     }
@@ -1214,26 +1234,39 @@ __device__ __forceinline__ void wide_forward(const SolveArgs<T>& a, const FrontD
   // this CTA's own blocks
   for (int p = b0; p < min(b0 + kSolveWarps, nblk); ++p) {
     T* y = ys + (p & 1) * 32 * RC;
+    const int nb = min(32, ns - p * 32);
+    if constexpr (kSpread<T, RC>) {
+      if (mine == p) {
+#pragma unroll
+        for (int r = 0; r < RC; ++r) y[lane * RC + r] = lane < nb ? w[r] : T(0);
+      }
+      spread_solve<T, true, !TRANS, RC>(ys + kWideRows * RC, p - b0, y, nr, nb, wid, lane);
+    }
     if (mine == p) {
-      const int nb = min(32, ns - p * 32);
       // rows past the pivots in this warp (a short last block) have zeros in
       // the triangle: their coefficients follow below
-      triangle_solve<T, true, !TRANS, RC>(B, w, lane);
+      if constexpr (kSpread<T, RC>) {
 #pragma unroll
-      for (int r = 0; r < RC; ++r) y[lane * RC + r] = lane < nb ? w[r] : T(0);
+        for (int r = 0; r < RC; ++r) w[r] = lane < nb ? y[lane * RC + r] : w[r];
+      } else {
+        triangle_solve<T, true, !TRANS, RC>(B, w, nb, lane);
+#pragma unroll
+        for (int r = 0; r < RC; ++r) y[lane * RC + r] = lane < nb ? w[r] : T(0);
+      }
       if (i < ns) st_row<T, RC>(Vs + i * st, nr, vec, w);
       if (nb < 32) load_panel<T, TRANS>(L, f, F, i, F, p * 32, nb, tile, lane);
     }
-    __syncthreads();
+    if constexpr (kSpread<T, RC>) __syncwarp();
+    else __syncthreads();
     if (shared && mine == p && lane == 0) publish(flag);  // behind the barrier: off the chain of blocks
     if (rows && (mine > p || (mine == p && p * 32 + 32 > ns))) {
       if (mine > p) {
-        apply_panel<T, RC>(L, w, y);
+        apply_panel<T, RC>(L, w, y, nr);
       } else {
         T u[RC];
 #pragma unroll
         for (int r = 0; r < RC; ++r) u[r] = w[r];
-        apply_panel<T, RC>(L, u, y);
+        apply_panel<T, RC>(L, u, y, nr);
 #pragma unroll
         for (int r = 0; r < RC; ++r) w[r] = i >= ns ? u[r] : w[r];
       }
@@ -1249,11 +1282,11 @@ __device__ __forceinline__ void wide_forward(const SolveArgs<T>& a, const FrontD
 // The rows are the pivots, solved from the last block up; the update rows'
 // values, known, come first as further blocks of columns.
 template <typename T, bool TRANS, int RC>
-__device__ __forceinline__ void wide_backward(const SolveArgs<T>& a, const FrontDesc& d, int k, int q, int ch, int r0,
-                                              int nr, T* sm) {
+__device__ __forceinline__ void wide_backward(const SolveArgs<T>& a, const FrontDesc& d, int k, int q, int ch, int rc,
+                                              int r0, int nr, T* sm) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int ns = d.ns, F = d.F, ms = F - ns;
-  const bool vec = a.vec && (r0 % Vec16<T>::N == 0);
+  const bool vec = a.vec && whole_pairs<T>(a, r0, nr);
   T* ys = sm;
   T* B = ys + kWideRows * RC + wid * kTri;
   T* tile = ys + kWideRows * RC + kSolveWarps * kTri + wid * 32 * WideTile<T>::LD;
@@ -1267,7 +1300,7 @@ __device__ __forceinline__ void wide_backward(const SolveArgs<T>& a, const Front
   const int mine = b0 + wid;
   const bool rows = i - lane < ns;
   const bool shared = ns > kWideRows;
-  int* flag = a.wide + (int64_t)(d.flag + (k * ((a.R + RC - 1) / RC) + ch)) * kCtrStride;
+  int* flag = a.wide + (int64_t)(d.flag + (k * ((a.R + rc - 1) / rc) + ch)) * kCtrStride;
   if (rows) stage_triangle<T, false, TRANS, TRANS>(B, f, F, mine * 32, min(32, ns - mine * 32), lane);
   T w[RC];
 #pragma unroll
@@ -1289,7 +1322,7 @@ __device__ __forceinline__ void wide_backward(const SolveArgs<T>& a, const Front
       __syncthreads();
       for (int e = 0; e < m; e += 32) {
         if (!rows) continue;
-        apply_panel<T, RC>(L, w, ys + e * RC);
+        apply_panel<T, RC>(L, w, ys + e * RC, nr);
         const int jn = j0 + e + 32;
         if (jn < ms) load_panel<T, TRANS>(L, f, F, i, ns, ns + jn, min(32, ms - jn), tile, lane);
       }
@@ -1317,28 +1350,42 @@ __device__ __forceinline__ void wide_backward(const SolveArgs<T>& a, const Front
     __syncthreads();
     for (; p >= lo; --p) {
       if (!rows) continue;
-      apply_panel<T, RC>(L, w, ys + (p - lo) * 32 * RC);
+      apply_panel<T, RC>(L, w, ys + (p - lo) * 32 * RC, nr);
       if (p - 1 > mine) load_panel<T, TRANS>(L, f, F, i, ns, (p - 1) * 32, 32, tile, lane);
     }
   }
   if (top > hi) __syncthreads();
   for (int p = hi; p >= b0; --p) {
     T* y = ys + (p & 1) * 32 * RC;
-    if (mine == p) {
-      triangle_solve<T, false, TRANS, RC>(B, w, lane);
+    if constexpr (kSpread<T, RC>) {
+      if (mine == p) {
 #pragma unroll
-      for (int r = 0; r < RC; ++r) y[lane * RC + r] = i < ns ? w[r] : T(0);
+        for (int r = 0; r < RC; ++r) y[lane * RC + r] = w[r];
+      }
+      spread_solve<T, false, TRANS, RC>(ys + kWideRows * RC, p - b0, y, nr, min(32, ns - p * 32), wid, lane);
+    }
+    if (mine == p) {
+      if constexpr (kSpread<T, RC>) {
+#pragma unroll
+        for (int r = 0; r < RC; ++r) w[r] = y[lane * RC + r];
+      } else {
+        triangle_solve<T, false, TRANS, RC>(B, w, min(32, ns - p * 32), lane);
+#pragma unroll
+        for (int r = 0; r < RC; ++r) y[lane * RC + r] = i < ns ? w[r] : T(0);
+      }
       if (i < ns) st_row<T, RC>(xk + (d.c0 + i) * st, nr, vec, w);
     }
-    __syncthreads();
+    if constexpr (kSpread<T, RC>) __syncwarp();
+    else __syncthreads();
     if (shared && mine == p && lane == 0) publish(flag);
     if (mine < p) {
-      apply_panel<T, RC>(L, w, y);
+      apply_panel<T, RC>(L, w, y, nr);
       if (p - 1 > mine) load_panel<T, TRANS>(L, f, F, i, ns, (p - 1) * 32, 32, tile, lane);
     }
   }
   if (i < ns && a.xd)
-    st_xd_row<T, RC>(a.xd + ((int64_t)(d.c0 + i) * a.K + k) * a.RX + r0, nr, a.vecd && (r0 & 1) == 0, a.xd_mode, w);
+    st_xd_row<T, RC>(a.xd + ((int64_t)(d.c0 + i) * a.K + k) * a.RX + r0, nr, a.vecd && whole_pairs<T>(a, r0, nr),
+                     a.xd_mode, w);
   __syncthreads();
   if (tid == 0) publish_self(a, d, k);
 }
@@ -1356,17 +1403,15 @@ __device__ __forceinline__ void wide_backward(const SolveArgs<T>& a, const Front
 // Without completion counters (one launch per stage) nothing waits but the
 // tasks of one front with more than 32 pivots for each other.
 // ---------------------------------------------------------------------------
-// right-hand sides of a task of a front with more than 32 pivots
-template <typename T> constexpr int wide_chunk() { return sizeof(T) == 4 ? 4 : 2; }
-
 template <typename T, bool FWD, bool TRANS, int RC>
 __device__ __forceinline__ void wide_task(const SolveArgs<T>& a, int slot, int b, int ch, T* sm) {
   const FrontDesc d = ld_desc(a.desc + slot);
   if (a.act && !a.act[d.inst]) return;
-  const int r0 = ch * RC, nr = min(RC, a.R - r0);
-  const int k = b & 255, q = b >> 8;  // shift; rows [256 q, 256 q + 256)
-  if (FWD) wide_forward<T, TRANS, RC>(a, d, k, q, ch, r0, nr, sm);
-  else wide_backward<T, TRANS, RC>(a, d, k, q, ch, r0, nr, sm);
+  const int rc = sizeof(T) == 8 && RC > 1 ? b >> 4 & 15 : RC;
+  const int r0 = ch * rc, nr = min(rc, a.R - r0);
+  const int k = b & 15, q = b >> 8;  // shift; rows [256 q, 256 q + 256)
+  if (FWD) wide_forward<T, TRANS, RC>(a, d, k, q, ch, rc, r0, nr, sm);
+  else wide_backward<T, TRANS, RC>(a, d, k, q, ch, rc, r0, nr, sm);
 }
 // The same with registers of its own: with several right-hand sides the other
 // tasks of the kernel spill less beside it.
@@ -1375,7 +1420,9 @@ __device__ __noinline__ void wide_call(const SolveArgs<T>& a, int slot, int b, i
   wide_task<T, FWD, TRANS, RC>(a, slot, b, ch, sm);
 }
 
-template <typename T, bool FWD, bool TRANS, int MINB, bool ONE>
+// WIDE: right-hand sides that the tasks of fronts with more than 32 pivots are compiled
+// for; one call of one form, since a second would have each keep registers for the other
+template <typename T, bool FWD, bool TRANS, int MINB, bool ONE, int WIDE>
 __global__ void __launch_bounds__(kSolveThreads, MINB) k_solve(const __grid_constant__ SolveArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int s_unit[2];
@@ -1393,7 +1440,7 @@ __global__ void __launch_bounds__(kSolveThreads, MINB) k_solve(const __grid_cons
     const int kind = U.x & 15;
     if (kind == kUnitWide) {
       if constexpr (ONE) wide_task<T, FWD, TRANS, 1>(a, U.a, U.b, U.c, sm);
-      else wide_call<T, FWD, TRANS, wide_chunk<T>()>(a, U.a, U.b, U.c, sm);
+      else wide_call<T, FWD, TRANS, WIDE>(a, U.a, U.b, U.c, sm);
     } else if constexpr (FWD || ONE) {
       constexpr int NR = ONE ? 1 : 8;
       FrontDesc d;
@@ -1418,15 +1465,10 @@ __global__ void __launch_bounds__(kSolveThreads, MINB) k_solve(const __grid_cons
         if constexpr (FWD) seg_forward<T, 32, TRANS, NR>(a, t, d, tid % 32, sm + wid * 32 * NR);
         else seg_backward<T, 32, TRANS>(a, t, d, tid % 32);
       }
-    } else if (kind == kUnitSeg16 || kind == kUnitSeg32) {
+    } else if (MINB == 2 && kind == kUnitSeg32) {  // compiled for more CTAs, it would spill the columns' registers
       FrontDesc d;
-      if (kind == kUnitSeg16) {
-        const SegTask t = seg_task<T>(a, U, (unsigned)U.b + tid / 16, 8, d);
-        seg_backward_rhs<T, 16, TRANS, 8>(a, t, d, tid % 16);
-      } else {
-        const SegTask t = seg_task<T>(a, U, (unsigned)U.b + tid / 32, 8, d);
-        seg_backward_rhs<T, 32, TRANS, 8>(a, t, d, tid % 32);
-      }
+      const SegTask t = seg_task<T>(a, U, (unsigned)U.b + wid, 8, d);
+      seg_backward_rhs<T, TRANS, 8>(a, t, d, tid & 31);
     } else {
       // a CTA task, its 8 warps sharing the front, or per warp task q of the
       // group: front q / NG, columns [32 g, 32 g + 32), g = q % NG
@@ -1450,21 +1492,21 @@ __global__ void __launch_bounds__(kSolveThreads, MINB) k_solve(const __grid_cons
   }
 }
 
-template <typename T, bool FWD, bool TRANS, int MINB, bool ONE>
+template <typename T, bool FWD, bool TRANS, int MINB, bool ONE, int WIDE>
 int launch_one(const SolveArgs<T>& a, int nunits, size_t smem, cudaStream_t st) {
   static std::atomic<int> nsm_dev[kMaxDevices];
   const int dev = current_device();
   int nsm = nsm_dev[dev].load(std::memory_order_acquire);
   if (!nsm) {
-    cudaFuncSetAttribute(k_solve<T, FWD, TRANS, MINB, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSolveSmemMax);
+    cudaFuncSetAttribute(k_solve<T, FWD, TRANS, MINB, ONE, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSolveSmemMax);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     nsm = std::max(nsm, 1);
     nsm_dev[dev].store(nsm, std::memory_order_release);
   }
   int occ = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_solve<T, FWD, TRANS, MINB, ONE>, kSolveThreads, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_solve<T, FWD, TRANS, MINB, ONE, WIDE>, kSolveThreads, smem);
   const int grid = std::max(1, std::min(nunits, std::max(1, occ) * nsm));
-  k_solve<T, FWD, TRANS, MINB, ONE><<<grid, kSolveThreads, smem, st>>>(a);
+  k_solve<T, FWD, TRANS, MINB, ONE, WIDE><<<grid, kSolveThreads, smem, st>>>(a);
   return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
@@ -1493,18 +1535,23 @@ int launch_solve_dir(bool trans, const SolveArgs<T>& a0, int32_t nunits, int32_t
     a.stage = col_stage<T>(nk);
     e = col_smem<T>(nk);
   }
-  if (wide > 0) e = std::max(e, wide_smem<T>(wide, trans));
+  const bool spread = wide > kWideAlone<T>;
+  if (wide > 0) e = std::max(e, wide_smem<T>(a.R == 1 ? 1 : spread ? kWideSpread<T> : kWideAlone<T>, trans));
   const size_t smem = e * sizeof(T);
-  static_assert(col_smem<T>(PISP_K_MAX) * sizeof(T) <= kSolveSmemMax && wide_smem<T>(wide_chunk<T>(), true) * sizeof(T) <= kSolveSmemMax &&
+  static_assert(col_smem<T>(PISP_K_MAX) * sizeof(T) <= kSolveSmemMax && wide_smem<T>(kWideSpread<T>, true) * sizeof(T) <= kSolveSmemMax &&
                     std::max(thin_smem(FWD, 8), kSolveWarps * 32 * 8) * sizeof(T) <= kSolveSmemMax,
                 "every launch of a solve fits");
   if (a.R == 1)
-    return trans ? launch_one<T, FWD, true, 2, true>(a, nunits, smem, st)
-                 : launch_one<T, FWD, false, 2, true>(a, nunits, smem, st);
-  if (trans) return launch_one<T, FWD, true, 2, false>(a, nunits, smem, st);
-  if (ctas >= 4) return launch_one<T, FWD, false, 4, false>(a, nunits, smem, st);
-  if (ctas == 3) return launch_one<T, FWD, false, 3, false>(a, nunits, smem, st);
-  return launch_one<T, FWD, false, 2, false>(a, nunits, smem, st);
+    return trans ? launch_one<T, FWD, true, 2, true, 1>(a, nunits, smem, st)
+                 : launch_one<T, FWD, false, 2, true, 1>(a, nunits, smem, st);
+  constexpr int A = kWideAlone<T>, W = kWideSpread<T>;
+  if (spread)  // the registers of two CTAs an SM
+    return trans ? launch_one<T, FWD, true, 2, false, W>(a, nunits, smem, st)
+                 : launch_one<T, FWD, false, 2, false, W>(a, nunits, smem, st);
+  if (trans) return launch_one<T, FWD, true, 2, false, A>(a, nunits, smem, st);
+  if (ctas >= 4) return launch_one<T, FWD, false, 4, false, A>(a, nunits, smem, st);
+  if (ctas == 3) return launch_one<T, FWD, false, 3, false, A>(a, nunits, smem, st);
+  return launch_one<T, FWD, false, 2, false, A>(a, nunits, smem, st);
 }
 
 }  // namespace pisp
