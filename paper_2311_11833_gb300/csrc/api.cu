@@ -68,6 +68,7 @@ struct pisp_handle {
   int32_t units_K = 0, units_R = 0;
   int32_t n_units_f = 0, n_units_b = 0;
   int32_t units_wide[2] = {};                 // right-hand sides of a task of a front with more than 32 pivots, per direction
+  bool units_segs = false;                    // the backward list has segments of several right-hand sides
   size_t ctr_tickets = 0, ctr_half = 0;       // tickets, and all counters, of one direction
   std::vector<int32_t> lvl_units_f, lvl_units_b;  // first unit of each stage (one launch per stage)
   // front records in unit-list order; counters, forward then backward: the
@@ -757,6 +758,8 @@ int build_units(pisp_handle* h, int32_t K, int32_t R) {
   h->lvl_units_b = b.start;
   h->units_wide[0] = wide[0];
   h->units_wide[1] = wide[1];
+  h->units_segs = false;
+  for (const pisp::Supernode& n : S.sn) h->units_segs = h->units_segs || (R > 1 && few_columns(h, n, R));
   h->ctr_tickets = (f.start.size() + b.start.size()) / 8 * 8 + 8;  // more than one per stage
   h->ctr_half = h->ctr_tickets + (nS * (size_t)NG + (size_t)nflags) * pisp::kCtrStride;
   h->units_K = K;
@@ -884,8 +887,9 @@ int solve_pass_t(pisp_handle* h, bool trans, const SolveIO& io, int32_t R, const
     const int pb = prof_begin(h);
     int n = 0;
     auto go = [&](int count) {
-      return dir == 0 ? pisp::launch_solve_dir<T, true>(trans, a, count, h->units_wide[dir], h->solve_ctas, h->stream)
-                      : pisp::launch_solve_dir<T, false>(trans, a, count, h->units_wide[dir], h->solve_ctas, h->stream);
+      return dir == 0 ? pisp::launch_solve_dir<T, true>(trans, a, count, h->units_wide[dir], false, h->solve_ctas, h->stream)
+                      : pisp::launch_solve_dir<T, false>(trans, a, count, h->units_wide[dir], h->units_segs, h->solve_ctas,
+                                                         h->stream);
     };
     const int total = dir == 0 ? h->n_units_f : h->n_units_b;
     a.NG = counter_groups(h, h->K, R, dir == 0);

@@ -284,9 +284,11 @@ inline int32_t rhs_stride64(int32_t R) { return R == 1 ? 1 : (R + 1) / 2 * 2; }
 // One launch of the forward (L, or U^T with trans) or backward (U, L^T) solve;
 // ctas = resident CTAs per SM it is compiled for with several right-hand sides
 // (2, 3, 4; <= 0, or transposed: 2); wide = the most right-hand sides of a task of a
-// front with more than 32 pivots, 0 if there is none.  Returns the kernels launched or -1.
+// front with more than 32 pivots, 0 if there is none; segs: the list has backward
+// segments of several right-hand sides.  Returns the kernels launched or -1.
 template <typename T, bool FWD>
-int launch_solve_dir(bool trans, const SolveArgs<T>& a, int32_t nunits, int32_t wide, int32_t ctas, cudaStream_t st);
+int launch_solve_dir(bool trans, const SolveArgs<T>& a, int32_t nunits, int32_t wide, bool segs, int32_t ctas,
+                     cudaStream_t st);
 constexpr int kWideUnitRows = 256;  // rows of a task of a front with more than 32 pivots
 int launch_combine(const SymDev& sd, const double* X, const Shifts& sh, int32_t R, double* x,
                    cudaStream_t st);

@@ -1421,8 +1421,10 @@ __device__ __noinline__ void wide_call(const SolveArgs<T>& a, int slot, int b, i
 }
 
 // WIDE: right-hand sides that the tasks of fronts with more than 32 pivots are compiled
-// for; one call of one form, since a second would have each keep registers for the other
-template <typename T, bool FWD, bool TRANS, int MINB, bool ONE, int WIDE>
+// for; one call of one form, since a second would have each keep registers for the other.
+// SEGS: backward segments of several right-hand sides, a kernel of their own for the same
+// reason (2000 buses, six solves of 16 right-hand sides: 310 us, 317 with them compiled in)
+template <typename T, bool FWD, bool TRANS, int MINB, bool ONE, int WIDE, bool SEGS>
 __global__ void __launch_bounds__(kSolveThreads, MINB) k_solve(const __grid_constant__ SolveArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int s_unit[2];
@@ -1465,7 +1467,7 @@ __global__ void __launch_bounds__(kSolveThreads, MINB) k_solve(const __grid_cons
         if constexpr (FWD) seg_forward<T, 32, TRANS, NR>(a, t, d, tid % 32, sm + wid * 32 * NR);
         else seg_backward<T, 32, TRANS>(a, t, d, tid % 32);
       }
-    } else if (MINB == 2 && kind == kUnitSeg32) {  // compiled for more CTAs, it would spill the columns' registers
+    } else if (SEGS && kind == kUnitSeg32) {
       FrontDesc d;
       const SegTask t = seg_task<T>(a, U, (unsigned)U.b + wid, 8, d);
       seg_backward_rhs<T, TRANS, 8>(a, t, d, tid & 31);
@@ -1492,21 +1494,21 @@ __global__ void __launch_bounds__(kSolveThreads, MINB) k_solve(const __grid_cons
   }
 }
 
-template <typename T, bool FWD, bool TRANS, int MINB, bool ONE, int WIDE>
+template <typename T, bool FWD, bool TRANS, int MINB, bool ONE, int WIDE, bool SEGS = false>
 int launch_one(const SolveArgs<T>& a, int nunits, size_t smem, cudaStream_t st) {
   static std::atomic<int> nsm_dev[kMaxDevices];
   const int dev = current_device();
   int nsm = nsm_dev[dev].load(std::memory_order_acquire);
   if (!nsm) {
-    cudaFuncSetAttribute(k_solve<T, FWD, TRANS, MINB, ONE, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSolveSmemMax);
+    cudaFuncSetAttribute(k_solve<T, FWD, TRANS, MINB, ONE, WIDE, SEGS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSolveSmemMax);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     nsm = std::max(nsm, 1);
     nsm_dev[dev].store(nsm, std::memory_order_release);
   }
   int occ = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_solve<T, FWD, TRANS, MINB, ONE, WIDE>, kSolveThreads, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_solve<T, FWD, TRANS, MINB, ONE, WIDE, SEGS>, kSolveThreads, smem);
   const int grid = std::max(1, std::min(nunits, std::max(1, occ) * nsm));
-  k_solve<T, FWD, TRANS, MINB, ONE, WIDE><<<grid, kSolveThreads, smem, st>>>(a);
+  k_solve<T, FWD, TRANS, MINB, ONE, WIDE, SEGS><<<grid, kSolveThreads, smem, st>>>(a);
   return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
@@ -1522,7 +1524,8 @@ constexpr size_t wide_smem(int wide, bool trans) {
 }
 
 template <typename T, bool FWD>
-int launch_solve_dir(bool trans, const SolveArgs<T>& a0, int32_t nunits, int32_t wide, int32_t ctas, cudaStream_t st) {
+int launch_solve_dir(bool trans, const SolveArgs<T>& a0, int32_t nunits, int32_t wide, bool segs, int32_t ctas,
+                     cudaStream_t st) {
   if (nunits <= 0) return 0;
   SolveArgs<T> a = a0;
   size_t e;
@@ -1545,6 +1548,14 @@ int launch_solve_dir(bool trans, const SolveArgs<T>& a0, int32_t nunits, int32_t
     return trans ? launch_one<T, FWD, true, 2, true, 1>(a, nunits, smem, st)
                  : launch_one<T, FWD, false, 2, true, 1>(a, nunits, smem, st);
   constexpr int A = kWideAlone<T>, W = kWideSpread<T>;
+  if constexpr (!FWD) {
+    if (segs && spread)
+      return trans ? launch_one<T, FWD, true, 2, false, W, true>(a, nunits, smem, st)
+                   : launch_one<T, FWD, false, 2, false, W, true>(a, nunits, smem, st);
+    if (segs)
+      return trans ? launch_one<T, FWD, true, 2, false, A, true>(a, nunits, smem, st)
+                   : launch_one<T, FWD, false, 2, false, A, true>(a, nunits, smem, st);
+  }
   if (spread)  // the registers of two CTAs an SM
     return trans ? launch_one<T, FWD, true, 2, false, W>(a, nunits, smem, st)
                  : launch_one<T, FWD, false, 2, false, W>(a, nunits, smem, st);
