@@ -333,9 +333,9 @@ int tile_ctas(const pisp_handle* h, int precision) {
 // 2043; with 100 of 1000, 171 k: 1941 / 2510; the one-launch figures past the lines
 // are with fronts of up to 160 rows by CTAs).
 // In FP64 tiles are small.  One grid's fronts are bound by the FP64 pipe whichever
-// way they are launched (300 buses 164 / 164, 1354 buses 573 / 567; 118 buses 110 /
-// 129, of which 22 are the segments that the one-launch form takes for fronts of at
-// most 32 rows); many grids' fronts fill the SMs (48 grids 3939 / 2470).
+// way they are launched (300 buses 154 / 156, 1354 buses 565 / 570; 118 buses 99 /
+// 122: the one-launch form takes segments for fronts of at most 32 rows); many grids'
+// fronts fill the SMs (48 grids 3939 / 2470, with the bodies of that time).
 // Fronts that wait for no others (dense systems) need no more than a launch a size
 // class, and no counters, while a CTA holds each: FP32, K 4, 16 systems of 40 rows
 // 36 / 39, of 97 81 / 90, of 160 139 / 156, of 200 (owner tiles) 191 / 144, of 9 to 137
@@ -546,7 +546,8 @@ int counter_groups(const pisp_handle* h, int32_t K, int32_t R, bool fwd) {
 // 32) CTA tasks per (shift, RHS chunk of 8); the rest segment tasks of 8, 16 or
 // 32 lanes by their size, one per group of h->kfuse consecutive shifts and RHS
 // chunk of 8.  Backward solves of several right-hand sides take column groups
-// instead: one CTA task, or one warp's task (8 a unit), per front and group.
+// instead: one CTA task, or one warp's task (8 a unit), per front and group; fronts
+// with many pivots to few right-hand sides (few_columns) segments of 32 lanes.
 // The forward list goes by the fronts' height above the leaves, the backward
 // list by their depth below the root: each as soon as what it waits for can be
 // done, so that the CTAs in flight hold ready units (by falling height, a

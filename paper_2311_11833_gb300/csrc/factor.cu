@@ -2236,9 +2236,9 @@ int factor_small_group(const SymDev& sd, const LevelPlan& lp, int g, const int32
     if (G.cluster == 0) {
       const int32_t* lst = d_small + G.off;
       bool seg_class = false;
-      // FP64 takes a CTA for the narrowest fronts too: its threads are dealt the
-      // elements, where rows as lanes leave some idle (118 buses 114 us against
-      // 136 with segments, 300 buses 168 against 185)
+      // FP64 takes a CTA for the narrowest fronts too: its warps share the columns,
+      // where rows as lanes leave some idle (118 buses 99 us, 136 with segments; 300
+      // buses 154, 185)
       if constexpr (sizeof(T) == 4) {
         const int n = G.count * K;
         auto seg = [&](auto S) {

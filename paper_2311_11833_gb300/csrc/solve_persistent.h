@@ -996,7 +996,8 @@ __device__ __forceinline__ void col_backward(const SolveArgs<T>& a, const FrontD
 // 3.2 us on a 320-row one.)
 // Many such tasks share the SMs' pipes, and a block that one warp solves leaves its
 // SM's idle: there the owning warp hands its block to as many warps as there are
-// right-hand sides and takes the solution back, two barriers a block (kSpread).
+// right-hand sides and takes the solution back, two barriers a block (kSpread;
+// 100 dense systems of 97 rows, K 10, R 8, FP32: 50 us forward, 70 without).
 // ---------------------------------------------------------------------------
 constexpr int kWideRows = kSolveThreads;
 constexpr int kTri = 32 * kBS + 32;  // a staged triangle and its reciprocal pivots
