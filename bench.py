@@ -46,7 +46,13 @@ L2_BYTES = 129 * 1024 * 1024
 # to the full workload where the capture ran a reduced batch); an entry is
 # removed when its kernel changes.
 # Keys: (workload, family, instances, library options as sorted (name, value) pairs).
-TRAFFIC_PER_LAUNCH = {}
+BATCH_TUNED = (("factor_policy", 0), ("relax_small", 8), ("relax_zeros", 0.05), ("solve_ctas_per_sm", 4),
+               ("solve_kfuse", 2), ("solve_schedule", 0), ("solve_warp_maxF", 64))
+TRAFFIC_PER_LAUNCH = {
+    ("batching", "factor_persistent", 256, BATCH_TUNED): 1419.53e6,  # 663.36 MB read + 756.17 MB written
+    ("batching", "forward", 256, BATCH_TUNED): 507.10e6,             # 331.34 MB read + 175.75 MB written
+    ("batching", "backward", 256, BATCH_TUNED): 679.44e6,            # 496.38 MB read + 183.06 MB written
+}
 
 # factor precision and FP64 residual sweeps per workload; refine_tol > 0:
 # adaptive sweeps (pisp_set_refinement), `sweeps` is then the maximum
