@@ -73,8 +73,10 @@ typedef struct pisp_options {
                              1 = one launch per height, or depth */
   int32_t factor_policy;  /* 0 (default) = by the work: one launch as under 4, with
                              its options chosen, where that was measured ahead
-                             (FP32 while no front is wider than 1024; FP64 from
-                             8192 (front, shift) pairs on), else level by level:
+                             (FP32 while no front is wider than 1024 and the
+                             widest leaves room on an SM for the work of the
+                             others; FP64 from 8192 (front, shift) pairs on; not
+                             for dense systems of up to 160), else level by level:
                              fronts of at most 32 by segments (FP64: one CTA
                              each), wider ones one CTA each while
                              the front fits in shared memory; larger fronts, of
@@ -98,7 +100,8 @@ typedef struct pisp_options {
                              a task waits (boundedly) only for its children's
                              completion counters */
   int32_t solve_kfuse;    /* solves by segments (forward, and backward with one
-                             right-hand side): shifts per segment task of a front
+                             right-hand side or with many pivots to few of them):
+                             shifts per segment task of a front
                              with at most 32 pivots (0 = 1): larger values pay a
                              front's dependency wait and structure loads once
                              for several shifts, smaller ones run more tasks
